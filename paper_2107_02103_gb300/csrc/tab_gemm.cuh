@@ -21,12 +21,55 @@
 // outputs are NaN and one timeout is counted (dp_tc_wait_timeouts).
 #pragma once
 
+#include "fixed.cuh"
 #include "tc_gemm.cuh"
 
 namespace dpc {
 namespace {
 namespace tg {
 using namespace tc;
+
+// ---- the backward's results as fixed points, for the rows kernel's integer arithmetic
+// dW[k][q] of (atom, interval) is exact in the GEMM's epilogue (a 128-bit integer).  The rows kernel takes
+// the constant d_0 = dW[k][0] and the derivative's coefficients D_q = q dW[k][q] 2^(-e q) (u = t 2^e, the
+// derivative sum_q D_q u^(q-1) by u), rounded to units of 2^(X + G - 61).  G bounds the atom's column,
+// sum_m |dT_km| < 2^G; X comes from the table's rows of the interval (exponents E_q, max_m |c_q| < 2^E_q),
+// apart for the constant and the rest so that neither loses places to the other:
+//   q >= 1: 2^slope > sum_q q 2^(E_q - e q), which bounds the derivative and its terms' sum;
+//   q = 0:  value = max(E_0, slope) + 1, which bounds the polynomial and all its parts.
+// (With one exponent for all six the derivative would lose seven places at Delta = 0.01.)
+constexpr int kGradPlaces = 61;
+constexpr int kGradLimb = 30;
+
+__device__ __forceinline__ int2 key_exps(const int *__restrict__ E6, int e) {  // (value, slope); kNonFinite
+  int E[6], top = -(1 << 21);
+  bool nf1 = false;
+#pragma unroll
+  for (int q = 0; q < 6; ++q) {
+    E[q] = __ldg(E6 + q);
+    if (q > 0) {
+      nf1 |= E[q] >= kNonFinite;
+      top = max(top, E[q] - e * q);
+    }
+  }
+  unsigned sum = 0;  // above sum_q q 2^(E_q - e q - top + 20), below 2^24
+#pragma unroll
+  for (int q = 1; q < 6; ++q) sum += (((unsigned)q << 20) >> min(top - (E[q] - e * q), 31)) + 1u;
+  const int slope = nf1 ? kNonFinite : top - 20 + 32 - __clz((int)sum);
+  return make_int2(nf1 || E[0] >= kNonFinite ? kNonFinite : max(E[0], slope) + 1, slope);
+}
+
+// The 128-bit integer (hi, lo) times max(q, 1), |.| < 2^80, over 2^sh to the nearest integer (halves up).
+__device__ __forceinline__ fx::Fix grad_fix(long long hi, unsigned long long lo, int q, int sh) {
+  const unsigned f = (unsigned)max(q, 1);
+  hi = hi * (long long)f + (long long)__umul64hi(lo, (unsigned long long)f);
+  lo *= f;
+  const int a = min(sh, 63), b = min(max(sh - 64, 0), 62);
+  const unsigned long long low = (lo >> a) | ((unsigned long long)hi << 1 << (63 - a));
+  const unsigned long long half = sh > 0 ? (lo >> max(a - 1, 0)) & 1ull : 0ull;
+  const unsigned long long half_h = b > 0 ? (unsigned long long)(hi >> (b - 1)) & 1ull : lo >> 63;
+  return fx::limbs<kGradLimb>(sh < 64 ? (long long)(low + half) : (hi >> b) + (long long)half_h);
+}
 
 constexpr int kEpiWarps = 8;    // two per TMEM lane quadrant
 constexpr long long kPartNaN = 1ll << 62;  // high word of a piece's output whose accumulators were not read
@@ -60,7 +103,11 @@ struct Params {
   // backward: output tile (tile, mt) wanted when one of K slices 8 mt .. 8 mt + 7 is flagged
   const unsigned char *sflags;  // [ntiles][nsf]
   int nsf;
-  double *scat;  // [natoms][cap][24]: the wanted outputs, per run slot, finished to f64
+  fx::Fix *scat;     // [natoms][cap][24]: the wanted outputs, per run slot, as fixed points (key_exps)
+  const int2 *kexp;  // [nkeys] of the launch's centre type
+  const int *gexp;   // [Np]
+  int n0, nint, e0, e1;  // fine intervals, intervals; binary places of u in the two segments
+  int *bad;              // set when a CTA gave up a wait: the rows kernel's results are then NaN
   const short *keys;
   const int *nslots;
   int cap, nkeys, kq;
@@ -402,6 +449,8 @@ __global__ void __launch_bounds__(kThreadsP, 1) tgemm_kernel(const Params P) {
       const int key = kFwd ? 0 : (int)((m0 + rl) / P.kq), qq = kFwd ? 0 : (int)(m0 + rl - (int64_t)key * P.kq);
       const int key_l = kFwd ? 0 : key - (int)(m0 / P.kq);
       const bool row_wanted = !kFwd && qq < 6 && key < P.nkeys;
+      const int qe = kFwd ? 0 : qq * (key % P.nint < P.n0 ? P.e0 : P.e1);  // d_q = dW[k][q] 2^-qe
+      const int2 ke = row_wanted ? P.kexp[key] : make_int2(0, 0);
       longlong2 *outp = kFwd && !direct ? P.part + (size_t)U.slot * kTN * P.Mp + m0 + rl : nullptr;
       // the warp's 24 columns of accumulators, four (one atom) at a time: each output's nine diagonals
       // recombined exactly as an integer and rounded once to f64 (diag_to_f64: integer operations, no
@@ -441,6 +490,19 @@ __global__ void __launch_bounds__(kThreadsP, 1) tgemm_kernel(const Params P) {
           if (slot >= 0) at = ((int64_t)((n0 >> 2) + al) * P.cap + slot) * 24 + qq, ldk = 6;
         }
         if (!__any_sync(0xffffffffu, at >= 0)) continue;
+        if constexpr (!kFwd) {
+          if (at >= 0)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              long long hi;
+              unsigned long long lo;
+              diag_s128(v, k, hi, lo);  // |.| < 2^74, in units three places above the finest asked for
+              const int c = c_lo + c0 + k;
+              const int sh = (qq ? ke.y : ke.x) + P.gexp[n0 + c] - kGradPlaces - (Erow - qe + fexp_s[c] + kOutExp) + 3;
+              P.scat[at + k * ldk] = grad_fix(hi << 3 | (long long)(lo >> 61), lo << 3, qq, clampi(sh, 0, 126));
+            }
+          continue;
+        }
         double val[4];
         int F[4];
         bool rare = false;
@@ -452,9 +514,9 @@ __global__ void __launch_bounds__(kThreadsP, 1) tgemm_kernel(const Params P) {
 #pragma unroll
           for (int k = 0; k < 4; ++k)
             val[k] = output_value_rare(v[0][k], v[1][k], v[2][k], v[3][k], v[4][k], v[5][k], v[6][k], v[7][k], v[8][k],
-                                       Erow, F[k], false);
+                                       Erow, F[k]);
         if (at >= 0) {
-          double *dst = (direct ? P.tout : P.scat) + at;
+          double *dst = P.tout + at;
 #pragma unroll
           for (int k = 0; k < 4; ++k) dst[k * ldk] = ok ? val[k] : __longlong_as_double(0x7ff8000000000000ll);
         }
@@ -469,7 +531,10 @@ __global__ void __launch_bounds__(kThreadsP, 1) tgemm_kernel(const Params P) {
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
-  if (tid == 0 && *abortf) atomicAdd(&g_wait_timeouts, 1u);
+  if (tid == 0 && *abortf) {
+    atomicAdd(&g_wait_timeouts, 1u);
+    if (!kFwd) *P.bad = 1;
+  }
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols));
 }
 

@@ -15,7 +15,7 @@
 // ahead of the epilogue ("tbl_full", released by "tbl_empty"), and eight epilogue warps (two per TMEM
 // lane quadrant, 16 columns each) finish the outputs.  (Measured: with the epilogue warps building the
 // tables themselves, the tensor core waited for the epilogue about 40 % of the time.)  Every wait is bounded; a wait that gives up stops the CTA's copies and MMAs,
-// its remaining outputs are NaN and one timeout is counted (dp_tc_wait_timeouts).
+// the rows kernel's results are then NaN (bad) and one timeout is counted (dp_tc_wait_timeouts).
 #pragma once
 
 #include "tab_gemm.cuh"
@@ -52,7 +52,11 @@ struct Params {
   const unsigned char *bplanes;  // B = dT^T of the chunk: blocks [ntiles][ka] of kSB x kPlaneBB bytes
   const int *Fexp;               // [32 ntiles] column exponents
   int64_t Mp;
-  double *scat;       // [natoms][cap][24]: the wanted outputs, per run slot, finished to f64
+  fx::Fix *scat;      // [natoms][cap][24]: the wanted outputs, per run slot, as fixed points (tg::key_exps)
+  const int2 *kexp;   // [nkeys] of the launch's centre type
+  const int *gexp;    // [32 ntiles]
+  int n0, nint, e0, e1;  // fine intervals, intervals; binary places of u in the two segments
+  int *bad;              // set when a CTA gave up a wait: the rows kernel's results are then NaN
   const short *keys;  // [atom0 + natoms][cap]: each atom's slot keys
   const int *nslots;  // [atom0 + natoms]
   int cap, nkeys, kq;
@@ -83,7 +87,7 @@ __global__ void __launch_bounds__(kThreadsB, 1) bgemm_kernel(const Params P) {
   uint64_t *tbl_empty = tbl_full + 2;
   uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(smem + kMiscOffB);
   volatile int *abortf = reinterpret_cast<volatile int *>(smem + kMiscOffB + 4);
-  // table buffer b: (key of the unit, atom) -> slot or -1, then the unit's 32 column exponents
+  // table buffer b: (key of the unit, atom) -> slot or -1, then G - F of the unit's 32 columns
   int *tables = reinterpret_cast<int *>(smem + kStabOffB);
   int *uflag = tables + 2 * kTableInts;  // [0]: the unit's accumulators and table are ready
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -194,7 +198,7 @@ __global__ void __launch_bounds__(kThreadsB, 1) bgemm_kernel(const Params P) {
       const int64_t a_first = (int64_t)tile * kAtomsB;
       const int key0 = (int)((int64_t)mt * kTM / P.kq);
       for (int x = lane; x < kScatKeysB * kAtomsB; x += 32) stab[x] = -1;
-      fexp_s[lane] = P.Fexp[(int64_t)tile * kTNB + lane];
+      fexp_s[lane] = P.gexp[(int64_t)tile * kTNB + lane] - P.Fexp[(int64_t)tile * kTNB + lane];
       __syncwarp();
       // the slot counts of the unit's atoms (0: past the chunk or not of type alpha), lane al < 8
       int nsl = 0;
@@ -245,9 +249,13 @@ __global__ void __launch_bounds__(kThreadsB, 1) bgemm_kernel(const Params P) {
       const int key_l = key - key0;
       const bool row_wanted = qq < 6 && key < P.nkeys;
       const uint32_t trow = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)b * kBufColsB;
+      // the row's part of the shift from the exact integer's units to the fixed point's
+      const int2 ke = row_wanted ? P.kexp[key] : make_int2(0, 0);
+      const int qe = qq * (key % P.nint < P.n0 ? P.e0 : P.e1);  // d_q = dW[k][q] 2^-qe
+      const int shr = (qq ? ke.y : ke.x) - tg::kGradPlaces - (Erow - qe + kOutExp7x8);
       // the warp's 16 columns, four (one atom) at a time: each output's seven diagonals recombined
-      // exactly as an integer and rounded once to f64 (diag7_to_f64), only where a row of the warp wants
-      // the atom's slot of that interval
+      // exactly as an integer and rounded once to the fixed point's units, only where a row of the warp
+      // wants the atom's slot of that interval
 #pragma unroll 1
       for (int c0 = 0; c0 < kEpiColsB; c0 += 4) {
         float v[kSB][4];
@@ -268,21 +276,17 @@ __global__ void __launch_bounds__(kThreadsB, 1) bgemm_kernel(const Params P) {
           if (slot >= 0) at = ((a_first + al) * P.cap + slot) * 24 + qq;
         }
         if (!__any_sync(0xffffffffu, at >= 0)) continue;
-        double val[4];
-        int F[4];
-        bool rare = false;
+        fx::Fix val[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) F[k] = fexp_s[c_lo + c0 + k];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) val[k] = diag7_to_f64(v, k, Erow, F[k], rare);
-        if (__any_sync(0xffffffffu, rare))  // warp-uniform, and never taken with these operands
-#pragma unroll
-          for (int k = 0; k < 4; ++k)
-            val[k] = output_value_rare(v[0][k], v[1][k], v[2][k], v[3][k], v[4][k], v[5][k], v[6][k], 0.f, 0.f, Erow,
-                                       F[k], true);
+        for (int k = 0; k < 4; ++k) {
+          long long hi;
+          unsigned long long lo;
+          diag7_s128(v, k, hi, lo);
+          val[k] = tg::grad_fix(hi, lo, qq, clampi(shr + fexp_s[c_lo + c0 + k], 0, 126));
+        }
         if (at >= 0)
 #pragma unroll
-          for (int k = 0; k < 4; ++k) P.scat[at + 6 * k] = ok ? val[k] : __longlong_as_double(0x7ff8000000000000ll);
+          for (int k = 0; k < 4; ++k) P.scat[at + 6 * k] = val[k];
       }
       asm volatile("tcgen05.fence::before_thread_sync;");
       __syncwarp();
@@ -297,7 +301,10 @@ __global__ void __launch_bounds__(kThreadsB, 1) bgemm_kernel(const Params P) {
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
-  if (tid == 0 && *abortf) atomicAdd(&g_wait_timeouts, 1u);
+  if (tid == 0 && *abortf) {
+    atomicAdd(&g_wait_timeouts, 1u);
+    *P.bad = 1;
+  }
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols));
 }
 

@@ -16,8 +16,8 @@
 //   dW_i[k][(l, q)] = (1/N_c) sum_m dT_i[k][m] c_q^{l,m},
 //   dE/dR~_j[k] = sum_q dW_i[k][(l, q)] t_j^q,
 //   dE/ds_j     = sum_k R~_j[k] sum_{q >= 1} q dW_i[k][(l, q)] t_j^(q-1)   (0 where s_j was clamped).
-// The FP64 pipe keeps the per-row work (24 FMAs per row for W, 40 for the
-// derivatives); the per-interval work (24 M1 FMAs per interval and atom in
+// The FP64 pipe keeps 24 FMAs per row for W; the rows' derivatives (40 multiply-adds) run in fixed point on
+// the integer pipes (fixed.cuh); the per-interval work (24 M1 FMAs per interval and atom in
 // each direction), which is most of it, runs as exact digit-split GEMMs on
 // the tensor cores (tc_gemm.cuh), at f64 accuracy.
 //
@@ -53,6 +53,7 @@
 
 #include "dp_common.cuh"
 #include "env_row.cuh"
+#include "fixed.cuh"
 #include "tab_gemm.cuh"
 #include "tab_gemm_b8.cuh"
 #include "tc_gemm.cuh"
@@ -70,8 +71,12 @@ constexpr int kShareSlices = kMaxShareSlices;  // used K slices per forward shar
 constexpr size_t kPartBudget = (size_t)1 << 30;  // bytes of the forward's partial results per chunk at most
 constexpr int kMaxCtasF = 160;  // CTAs of the forward GEMM at most (its part slots are sized for them)
 constexpr int kEpiCost = 6;     // a forward unit's epilogue, in slices' time, for the forward schedule
+constexpr int kBadFlag = DP_MAX_TYPES;  // after the backward's unit counts: set when a GEMM wait gave up
 constexpr int kMaxKeys = 4096;  // ntypes x nint: each warp's key map (int16) lives in shared memory
 static_assert(kChunkAtoms % kTileAtoms == 0 && kChunkAtoms % 8 == 0, "whole tiles per chunk");
+
+// Shorts of one atom's key -> slot map: whole 16-byte words.
+__host__ __device__ constexpr int map_stride(int nkeys) { return (nkeys + 7) / 8 * 8; }
 
 // Sizes shared by the kernels, the plan and the work-buffer layout.
 struct Shape {
@@ -176,7 +181,7 @@ Layout make_layout(const Shape &s) {
   L.slist = take(off, (size_t)s.ntypes * s.ntiles * s.nsl * sizeof(short));
   L.scount = take(off, (size_t)s.ntypes * s.ntiles * sizeof(int));
   L.units = take(off, (size_t)s.ntypes * std::max(s.maxunits, s.maxunits8) * sizeof(int));
-  L.nunits = take(off, (size_t)s.ntypes * sizeof(int));
+  L.nunits = take(off, (size_t)(kBadFlag + 1) * sizeof(int));
   L.pieces = take(off, (size_t)s.maxpieces * sizeof(int4));
   L.pcta = take(off, (size_t)s.maxpieces * sizeof(int));
   L.cta_start = take(off, (size_t)(kMaxCtasF + 1) * sizeof(int));
@@ -375,17 +380,16 @@ __device__ __forceinline__ int valid_rows(const int32_t *nvalid, const int *sel,
 
 // Row index of valid row v (type segments in order, the valid rows of each first) and its segment.
 __device__ __forceinline__ int valid_row(int v, const int *nvb, const int *sel, int ntypes, int &b) {
-  int cum = 0, lim = nvb[0], off = 0;
+  int row = v;
   b = 0;
-#pragma unroll
-  for (int q = 1; q < DP_MAX_TYPES; ++q)
-    if (q < ntypes && v >= lim) {
+  int lim = nvb[0];
+  for (int q = 1; q < ntypes; ++q)  // uniform; none for one type
+    if (v >= lim) {
       b = q;
-      cum = lim;
+      row += sel[q - 1] - nvb[q - 1];
       lim += nvb[q];
-      off += sel[q - 1];
     }
-  return off + (v - cum);
+  return row;
 }
 
 // One warp per atom: the runs of rows sharing an interval (consecutive rows with one key; rows
@@ -534,6 +538,16 @@ __global__ void __launch_bounds__(128) slice_list_kernel(const unsigned char *__
   if (lane == 0) count[(size_t)t * ntiles + tile] = rank;
 }
 
+// The exponents of the backward's fixed points: from the row exponents Eexp [ntypes][Mp] of its A operand,
+// kexp [ntypes][nkeys] and, of the chunk's dT columns, gexp.
+struct GradExps {
+  const int *Eexp;
+  int64_t Mp;
+  int nkeys, n0, nint, e0, e1;
+  int2 *kexp;
+  int *gexp;
+};
+
 // Exclusive prefix sum over a block of 1024 threads of one value per thread; the block's total in *total.
 __device__ long long block_scan_1024(long long v, long long *red, long long *total) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -635,12 +649,27 @@ __global__ void __launch_bounds__(1024) fwd_schedule_kernel(const int *__restric
   }
 }
 
+// The exponents of the backward's fixed points for every centre type and key (tg::key_exps), from the row
+// exponents of its A operand; a share of them per block of the units kernels below.
+__device__ __forceinline__ void fill_key_exps(const GradExps &X, int ntypes) {
+  const int total = ntypes * X.nkeys;
+  for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < total; x += gridDim.x * blockDim.x) {
+    const int t = x / X.nkeys, key = x - t * X.nkeys;
+    X.kexp[x] = tg::key_exps(X.Eexp + (size_t)t * X.Mp + kQ * key, key % X.nint < X.n0 ? X.e0 : X.e1);
+  }
+}
+
 // The backward GEMM's units: the (tile, 128-row output tile) pairs whose K slices some atom of the tile
 // uses, per centre type (one thread per (type, tile)).
 __global__ void __launch_bounds__(128) bwd_units_kernel(const unsigned char *__restrict__ occ, int64_t tiles_all,
                                                         int64_t tile0, int64_t ntiles, int ntypes, int nsl, int nmt,
                                                         int64_t maxunits, int *__restrict__ units,
-                                                        int *__restrict__ nunits) {
+                                                        int *__restrict__ nunits, const GradExps X,
+                                                        const int *__restrict__ fexp, int log_M1) {
+  fill_key_exps(X, ntypes);
+  // sum_m |dT_km| < M1 2^F of every column
+  for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < ntiles * kTN; c += (int64_t)gridDim.x * blockDim.x)
+    X.gexp[c] = fexp[c] >= kNonFinite ? kNonFinite : fexp[c] + log_M1;
   const int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (x >= (int64_t)ntypes * ntiles) return;
   const int t = (int)(x / ntiles);
@@ -665,7 +694,9 @@ __global__ void __launch_bounds__(32 * tb::kAtomsB) bwd_units8_kernel(const shor
                                                                     const int32_t *__restrict__ atype, int ntypes,
                                                                     int cap, int64_t atom0, int64_t natoms,
                                                                     int64_t ntiles8, int64_t maxunits8,
-                                                                    int *__restrict__ units, int *__restrict__ nunits) {
+                                                                    int *__restrict__ units, int *__restrict__ nunits,
+                                                                    const GradExps X) {
+  fill_key_exps(X, ntypes);
   __shared__ unsigned bits[kMaxRowTiles / 32];
   const int lane = threadIdx.x & 31, al = threadIdx.x >> 5;
   const int t = (int)(blockIdx.x / ntiles8);
@@ -773,32 +804,121 @@ struct RowsParams {
   int sel[DP_MAX_TYPES];
   const short *keys;   // [nloc][cap]: key of each slot
   const int *nslots;   // [nloc]
-  const double *dW;    // [natoms][cap][24]: the backward GEMM's result per slot, dW[k][q] at 6 k + q
+  const fx::Fix *dW;   // [natoms][cap][24]: the backward GEMM's result per slot, dW[k][q] at 6 k + q
+  const int2 *kexp;    // [ntypes][nkeys] exponents of those fixed points (key_exps), and
+  const int *gexp;     // [4 natoms]: 2^gexp > sum_m |dT_km| of atom a at 4 a + k
+  int e0, e1;          // binary places of u = t 2^e in the fine and the coarse segment
+  const int *bad;      // nonzero: a GEMM wait gave up, the results are NaN
   double *ds, *dRt;
   int64_t natoms;
   EnvRow env;             // rows_force_kernel: rows from coordinates,
   double *F, *virial;     // and the forces [nall][3] and virial [9] they add to
 };
 
+// The atom's exponents gexp, every one nonfinite where a GEMM wait gave up; `plain`: results made with them
+// and with plain key exponents (|.| <= 400) stay normal doubles, however small or large.
+__device__ __forceinline__ int4 atom_exps(const RowsParams &P, int64_t a, bool &plain) {
+  int4 g = __ldg(reinterpret_cast<const int4 *>(P.gexp) + a);
+  if (__ldg(P.bad)) g = make_int4(kNonFinite, kNonFinite, kNonFinite, kNonFinite);
+  plain = max(max(abs(g.x), abs(g.y)), max(abs(g.z), abs(g.w))) <= 400;
+  return g;
+}
+
+__device__ __noinline__ double odd_double(long long v, int e, bool nan) {
+  return nan ? __longlong_as_double(0x7ff8000000000000ll) : scalbn((double)v, e);
+}
+
+// One row's dE/dR~[k] = P_k(t) = sum_q dW[k][q] t^q and dE/ds = sum_k R~[k] P_k'(t), from its slot's 24
+// fixed points (tg::key_exps), in integer arithmetic (fixed.cuh): with u = t 2^e,
+//   P_k = d_0 + sum_q D_q u^q / q,   P_k' = 2^e sum_q D_q u^(q-1),
+// two sums of products per k, each rounded once to f64.  Why: 42 FP64 instructions a row bound the kernel
+// (91 % of that pipe); the limb products take the integer pipes 250 clocks of a sub-partition against 2,900,
+// and the FP64 pipe keeps the conversions and the last dot product (14 instructions).  Measured with 1.7 M
+// rows (copper, 4,096 atoms): 0.137 -> 0.073 ms; 1.1 M (water): 0.089 -> 0.061 ms.
+struct RowPoly {
+  fx::Fix u1, u2, u3, u4, w2, w3, w4, w5;  // u^q and u^q / q
+  int2 ke;
+  int e, drop;
+  bool plain, nan;
+};
+__device__ __forceinline__ RowPoly row_poly(const int2 ke, bool plain, double t, int e) {
+  constexpr int L = tg::kGradLimb;
+  using fx::Fix;
+  RowPoly R;
+  R.u1 = fx::limbs<L>(fx::from_double(t, 2 * L + e));
+  const long long s2 = fx::mul<L>(R.u1, R.u1);
+  R.u2 = fx::limbs<L>(s2);
+  R.u3 = fx::limbs<L>(fx::mul<L>(R.u2, R.u1));
+  const long long s4 = fx::mul<L>(R.u2, R.u2);
+  R.u4 = fx::limbs<L>(s4);
+  constexpr Fix third{0x15555555, 0x15555555}, fifth{0x33333333, 0x0ccccccc};  // 2^60 / 3, 2^60 / 5
+  R.w2 = fx::limbs<L>(s2 >> 1);
+  R.w3 = fx::limbs<L>(fx::mul<L>(R.u3, third));
+  R.w4 = fx::limbs<L>(s4 >> 2);
+  R.w5 = fx::limbs<L>(fx::mul<L>(fx::limbs<L>(fx::mul<L>(R.u4, R.u1)), fifth));
+  R.ke = ke;
+  R.e = e;
+  R.drop = ke.x - ke.y;  // the constant's units over the slope's, as a shift: >= 1
+  R.plain = plain && max(abs(ke.x), abs(ke.y)) <= 400 && R.drop < 32;
+  R.nan = (__double2hiint(t) & 0x7ff00000) == 0x7ff00000;  // a NaN s
+  return R;
+}
+// P_k and P_k' of component k, whose column's exponent is g.
+__device__ __forceinline__ void row_component(const RowPoly &R, const fx::Fix *__restrict__ slot, int k, int g,
+                                              double &P, double &dP) {
+  constexpr int L = tg::kGradLimb;
+  using fx::Fix;
+  const int4 *c = reinterpret_cast<const int4 *>(slot) + 3 * k;
+  const int4 c01 = __ldg(c), c23 = __ldg(c + 1), c45 = __ldg(c + 2);
+  const Fix c0{c01.x, c01.y}, c1{c01.z, c01.w}, c2{c23.x, c23.y}, c3{c23.z, c23.w}, c4{c45.x, c45.y},
+      c5{c45.z, c45.w};
+  fx::Acc p, q;
+  p.mad(c1, R.u1);
+  p.mad(c2, R.w2);
+  p.mad(c3, R.w3);
+  p.mad(c4, R.w4);
+  p.mad(c5, R.w5);
+  q.mad(c2, R.u1);
+  q.mad(c3, R.u2);
+  q.mad(c4, R.u3);
+  q.mad(c5, R.u4);
+  const long long pv = fx::over_unit<L>(p, 5), qv = fx::whole<L>(c1) + fx::over_unit<L>(q, 4);
+  const int ep = R.ke.x + g - tg::kGradPlaces, eq = R.ke.y + g - tg::kGradPlaces + R.e;
+  if (R.plain) {
+    const int ph = (int)(pv >> 32);
+    const long long ps = (long long)(ph >> R.drop) << 32 | __funnelshift_r((unsigned)pv, (unsigned)ph, R.drop);
+    P = fx::to_double(fx::whole<L>(c0) + ps, ep);
+    dP = fx::to_double(qv, eq);
+  } else {  // an inf or NaN in dT or the table, an abandoned GEMM wait, or an extreme scale
+    P = odd_double(fx::whole<L>(c0) + (pv >> min(max(R.drop, 1), 63)), ep, R.ke.x >= kNonFinite || g >= kNonFinite);
+    dP = odd_double(qv, eq, R.ke.y >= kNonFinite || g >= kNonFinite);
+  }
+  if (R.nan) P = dP = __longlong_as_double(0x7ff8000000000000ll);
+}
+
 // One warp per atom, a lane per valid row: the row's interval from s, its run slot from the atom's key map
 // (shared memory), the slot's gradient coefficients dW[k][q] read through L1 (the rows of a run share
-// them), and dE/dR~ and dE/ds by Horner's rule in u with its derivative; padded rows get zeros.
-__global__ void __launch_bounds__(32 * kRowsWarps) rows_kernel(const RowsParams P) {
+// them), and dE/dR~ and dE/ds from them (row_grad); padded rows get zeros.
+__global__ void __launch_bounds__(32 * kRowsWarps, 7) rows_kernel(const RowsParams P) {
   __shared__ int nvbw[kRowsWarps][DP_MAX_TYPES];
-  extern __shared__ short smapw[];  // [kRowsWarps][nkeys]
+  extern __shared__ __align__(16) short smapw[];  // [kRowsWarps][map_stride(nkeys)]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t a = (int64_t)blockIdx.x * kRowsWarps + warp;
   if (a >= P.natoms) return;  // warp-uniform
   int *nvb = nvbw[warp];
-  short *smap = smapw + (size_t)warp * P.nkeys;
+  short *smap = smapw + (size_t)warp * map_stride(P.nkeys);
   const int64_t i = P.atom0 + a;
   const short *keys = P.keys + i * P.cap;
   const int nslot = P.nslots[i];
-  for (int k = lane; k < P.nkeys; k += 32) smap[k] = -1;
+  for (int k = lane; k < map_stride(P.nkeys) / 8; k += 32)
+    reinterpret_cast<int4 *>(smap)[k] = make_int4(-1, -1, -1, -1);
   __syncwarp();
   for (int x = lane; x < nslot; x += 32) smap[keys[x]] = (short)x;  // the map of the atom's keys
   const int nv = valid_rows(P.nvalid, P.sel, P.ntypes, i, lane, nvb);  // (its __syncwarp orders the map)
-  const double *dWa = P.dW + (size_t)a * P.cap * 24;
+  const fx::Fix *dWa = P.dW + (size_t)a * P.cap * 24;
+  const int2 *kexp = P.kexp + (size_t)(P.atype ? clampi(__ldg(P.atype + i), 0, P.ntypes - 1) : 0) * P.nkeys;
+  bool plain;
+  const int4 ge = atom_exps(P, a, plain);
   const double *srow = P.s + i * P.nnei;
   const double *Rrow = P.Rt + i * P.nnei * 4;
   double *dsrow = P.ds + i * P.nnei;
@@ -806,29 +926,26 @@ __global__ void __launch_bounds__(32 * kRowsWarps) rows_kernel(const RowsParams 
   for (int v = lane; v < nv; v += 32) {
     int b;
     const int row = valid_row(v, nvb, P.sel, P.ntypes, b);
+    const double sv = __ldg(srow + row);
     double t;
     bool clamped;
-    const int l = locate_fast(P.g, P.gf, P.nodes, __ldg(srow + row), t, clamped);
-    const Vec4<double> rr = ld4(Rrow + (size_t)row * 4);
-    const double2 *dw = reinterpret_cast<const double2 *>(dWa + (size_t)smap[b * P.g.nint + l] * 24);
-    const double r4[4] = {rr.x, rr.y, rr.z, rr.w};
-    double d4[4], ds = 0.0;
+    const int l = locate_fast(P.g, P.gf, P.nodes, sv, t, clamped);
+    const int key = b * P.g.nint + l;
+    const fx::Fix *slot = dWa + (size_t)smap[key] * 24;
+    const RowPoly R = row_poly(__ldg(kexp + key), plain, t, l < P.g.n0 ? P.e0 : P.e1);
+    const double2 *rr = reinterpret_cast<const double2 *>(Rrow + (size_t)row * 4);
+    double2 *dr = reinterpret_cast<double2 *>(drow + (size_t)row * 4);
+    double ds = 0.0;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {  // P_k(t) = sum_q dW[k][q] t^q and P_k'(t): 5 + 4 FMA
-      const double2 c01 = __ldg(dw + 3 * k), c23 = __ldg(dw + 3 * k + 1), c45 = __ldg(dw + 3 * k + 2);
-      double p = fma(c45.y, t, c45.x), dp = c45.y;
-      dp = fma(dp, t, p);
-      p = fma(p, t, c23.y);
-      dp = fma(dp, t, p);
-      p = fma(p, t, c23.x);
-      dp = fma(dp, t, p);
-      p = fma(p, t, c01.y);
-      dp = fma(dp, t, p);
-      d4[k] = fma(p, t, c01.x);
-      ds = fma(r4[k], dp, ds);
+    for (int h = 0; h < 2; ++h) {
+      const double2 r = __ldg(rr + h);
+      double p0, p1, dp0, dp1;
+      row_component(R, slot, 2 * h, h ? ge.z : ge.x, p0, dp0);
+      row_component(R, slot, 2 * h + 1, h ? ge.w : ge.y, p1, dp1);
+      dr[h] = make_double2(p0, p1);
+      ds = fma(r.y, dp1, fma(r.x, dp0, ds));
     }
     dsrow[row] = clamped ? 0.0 : ds;
-    st4(drow + (size_t)row * 4, d4[0], d4[1], d4[2], d4[3]);
   }
   // padded rows of each segment
   int off = 0;
@@ -848,20 +965,24 @@ __global__ void __launch_bounds__(32 * kRowsWarps) rows_kernel(const RowsParams 
 // reach memory.  The per-atom sums are reduced over the warp and added once.
 __global__ void __launch_bounds__(32 * kRowsWarps) rows_force_kernel(const RowsParams P) {
   __shared__ int nvbw[kRowsWarps][DP_MAX_TYPES];
-  extern __shared__ short smapw[];  // [kRowsWarps][nkeys]
+  extern __shared__ __align__(16) short smapw[];  // [kRowsWarps][map_stride(nkeys)]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t a = (int64_t)blockIdx.x * kRowsWarps + warp;
   if (a >= P.natoms) return;  // warp-uniform
   int *nvb = nvbw[warp];
-  short *smap = smapw + (size_t)warp * P.nkeys;
+  short *smap = smapw + (size_t)warp * map_stride(P.nkeys);
   const int64_t i = P.atom0 + a;
   const short *keys = P.keys + i * P.cap;
   const int nslot = P.nslots[i];
-  for (int k = lane; k < P.nkeys; k += 32) smap[k] = -1;
+  for (int k = lane; k < map_stride(P.nkeys) / 8; k += 32)
+    reinterpret_cast<int4 *>(smap)[k] = make_int4(-1, -1, -1, -1);
   __syncwarp();
   for (int x = lane; x < nslot; x += 32) smap[keys[x]] = (short)x;  // the map of the atom's keys
   const int nv = env_valid_rows(P.env, P.nnei, P.sel, P.ntypes, i, lane, nvb, nullptr);  // (orders the map)
-  const double *dWa = P.dW + (size_t)a * P.cap * 24;
+  const fx::Fix *dWa = P.dW + (size_t)a * P.cap * 24;
+  const int2 *kexp = P.kexp + (size_t)(P.atype ? clampi(__ldg(P.atype + i), 0, P.ntypes - 1) : 0) * P.nkeys;
+  bool plain;
+  const int4 ge = atom_exps(P, a, plain);
   double f[3] = {0.0, 0.0, 0.0}, w[9];
 #pragma unroll
   for (int x = 0; x < 9; ++x) w[x] = 0.0;
@@ -873,20 +994,14 @@ __global__ void __launch_bounds__(32 * kRowsWarps) rows_force_kernel(const RowsP
     double t;
     bool clamped;
     const int l = locate_fast(P.g, P.gf, P.nodes, ev.r4[0], t, clamped);
-    const double2 *dw = reinterpret_cast<const double2 *>(dWa + (size_t)smap[b * P.g.nint + l] * 24);
+    const int key = b * P.g.nint + l;
+    const fx::Fix *slot = dWa + (size_t)smap[key] * 24;
+    const RowPoly R = row_poly(__ldg(kexp + key), plain, t, l < P.g.n0 ? P.e0 : P.e1);
     double d4[4], ds = 0.0;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {  // as rows_kernel
-      const double2 c01 = __ldg(dw + 3 * k), c23 = __ldg(dw + 3 * k + 1), c45 = __ldg(dw + 3 * k + 2);
-      double p = fma(c45.y, t, c45.x), dp = c45.y;
-      dp = fma(dp, t, p);
-      p = fma(p, t, c23.y);
-      dp = fma(dp, t, p);
-      p = fma(p, t, c23.x);
-      dp = fma(dp, t, p);
-      p = fma(p, t, c01.y);
-      dp = fma(dp, t, p);
-      d4[k] = fma(p, t, c01.x);
+    for (int k = 0; k < 4; ++k) {
+      double dp;
+      row_component(R, slot, k, k == 0 ? ge.x : k == 1 ? ge.y : k == 2 ? ge.z : ge.w, d4[k], dp);
       ds = fma(ev.r4[k], dp, ds);
     }
     ds = clamped ? 0.0 : ds;
@@ -1011,6 +1126,13 @@ int make_plan(const double *table, const dp_table_info *info, int nnei, int ntyp
   out->ntypes = ntypes;
   out->M1 = M1;
   return DP_OK;
+}
+
+// Binary places e with |t| 2^e < 1 over an interval of this step, with 5 % to spare (t may lie a hair outside).
+int unit_places(double stride) {
+  int e = 0;
+  std::frexp(1.05 * stride, &e);
+  return -e;
 }
 
 RunsParams runs_params(const double *s, const double *Rt, const int32_t *nvalid, const int32_t *atype,
@@ -1186,7 +1308,17 @@ int grad(const dp_tc_plan *plan, const dp_table_info *info, const double *s, con
   RunsParams R = runs_params(s, Rt, nvalid, atype, g, seg, S, L, wk, nnei,
                              reinterpret_cast<const double *>(pk + PL.nodes));
   const int mtiles = S.Mpb / kTM;
-  double *dW = reinterpret_cast<double *>(wk + L.w);
+  fx::Fix *dW = reinterpret_cast<fx::Fix *>(wk + L.w);
+  GradExps X{};  // in the region of the forward's partial results, which the backward does not use
+  X.Eexp = reinterpret_cast<const int *>(pk + PL.ebwd);
+  X.Mp = S.Mpb;
+  X.nkeys = S.nkeys;
+  X.n0 = g.n0;
+  X.nint = g.nint;
+  X.e0 = unit_places(g.stride0);
+  X.e1 = unit_places(g.stride1);
+  X.gexp = reinterpret_cast<int *>(wk + L.part);
+  X.kexp = reinterpret_cast<int2 *>(wk + L.part + (size_t)std::max(S.Np, S.Np8) * sizeof(int));
   RowsParams Q{};
   Q.s = s;
   Q.Rt = Rt;
@@ -1203,6 +1335,11 @@ int grad(const dp_tc_plan *plan, const dp_table_info *info, const double *s, con
   Q.keys = R.keys;
   Q.nslots = R.nslots;
   Q.dW = dW;
+  Q.kexp = X.kexp;
+  Q.gexp = X.gexp;
+  Q.e0 = X.e0;
+  Q.e1 = X.e1;
+  Q.bad = reinterpret_cast<const int *>(wk + L.nunits) + kBadFlag;
   Q.ds = ds;
   Q.dRt = dRt;
   if (env) {
@@ -1228,15 +1365,15 @@ int grad(const dp_tc_plan *plan, const dp_table_info *info, const double *s, con
     if (S.b8) {
       // B = dT^T on 8-atom tiles in the 7 x 8-bit digits: the columns 4 a + k are the rows of this chunk's dT
       if ((rc = split_rows_1k<Digits7x8>(dT + c0 * kCols * M1, M1, 1, kCols * n, M1, round_up(kCols * n, tb::kTNB),
-                                         S.Kpm, tb::kTNB, wk + L.bplanes, wk + L.fexp, st, who)))
+                                         S.Kpm, tb::kTNB, wk + L.bplanes, wk + L.fexp, X.gexp, st, who)))
         return rc;
       prof_mark("tc_split_dT", st);
-      if (cudaMemsetAsync(wk + L.nunits, 0, (size_t)ntypes * sizeof(int), st) != cudaSuccess)
+      if (cudaMemsetAsync(wk + L.nunits, 0, (kBadFlag + 1) * sizeof(int), st) != cudaSuccess)
         return set_error(DP_ERR_CUDA, "%s: cudaMemsetAsync: %s", who, cudaGetErrorString(cudaGetLastError()));
       const int64_t ntiles8 = (n + tb::kAtomsB - 1) / tb::kAtomsB, nlist = (int64_t)ntypes * ntiles8;
       bwd_units8_kernel<<<(unsigned)nlist, 32 * tb::kAtomsB, 0, st>>>(
           R.keys, R.nslots, atype, ntypes, S.cap, c0, n, ntiles8, S.maxunits8, reinterpret_cast<int *>(wk + L.units),
-          reinterpret_cast<int *>(wk + L.nunits));
+          reinterpret_cast<int *>(wk + L.nunits), X);
       if ((rc = launch_status(who))) return rc;
       prof_mark("tc_units", st);
       for (int t = 0; t < ntypes; ++t) {
@@ -1248,6 +1385,13 @@ int grad(const dp_tc_plan *plan, const dp_table_info *info, const double *s, con
         G.Fexp = R.fexp;
         G.Mp = S.Mpb;
         G.scat = dW;
+        G.kexp = X.kexp + (size_t)t * S.nkeys;
+        G.gexp = X.gexp;
+        G.n0 = g.n0;
+        G.nint = g.nint;
+        G.e0 = X.e0;
+        G.e1 = X.e1;
+        G.bad = reinterpret_cast<int *>(wk + L.nunits) + kBadFlag;
         G.keys = R.keys;
         G.nslots = R.nslots;
         G.cap = S.cap;
@@ -1269,13 +1413,16 @@ int grad(const dp_tc_plan *plan, const dp_table_info *info, const double *s, con
                            who)))
         return rc;
       prof_mark("tc_split_dT", st);
-      if (cudaMemsetAsync(wk + L.nunits, 0, (size_t)ntypes * sizeof(int), st) != cudaSuccess)
+      if (cudaMemsetAsync(wk + L.nunits, 0, (kBadFlag + 1) * sizeof(int), st) != cudaSuccess)
         return set_error(DP_ERR_CUDA, "%s: cudaMemsetAsync: %s", who, cudaGetErrorString(cudaGetLastError()));
       const int64_t nlist = (int64_t)ntypes * ntiles;
+      int log_M1 = 0;
+      while ((1 << log_M1) < M1) ++log_M1;
       bwd_units_kernel<<<(unsigned)((nlist + 127) / 128), 128, 0, st>>>(wk + L.occ, S.tiles_all, tile0, ntiles, ntypes,
                                                                         S.nsl, mtiles, S.maxunits,
                                                                         reinterpret_cast<int *>(wk + L.units),
-                                                                        reinterpret_cast<int *>(wk + L.nunits));
+                                                                        reinterpret_cast<int *>(wk + L.nunits), X,
+                                                                        R.fexp, log_M1);
       if ((rc = launch_status(who))) return rc;
       prof_mark("tc_units", st);
       for (int t = 0; t < ntypes; ++t) {
@@ -1293,6 +1440,13 @@ int grad(const dp_tc_plan *plan, const dp_table_info *info, const double *s, con
         G.sflags = wk + L.occ + ((size_t)t * S.tiles_all + tile0) * S.nsl;
         G.nsf = S.nsl;
         G.scat = dW;
+        G.kexp = X.kexp + (size_t)t * S.nkeys;
+        G.gexp = X.gexp;
+        G.n0 = g.n0;
+        G.nint = g.nint;
+        G.e0 = X.e0;
+        G.e1 = X.e1;
+        G.bad = reinterpret_cast<int *>(wk + L.nunits) + kBadFlag;
         G.keys = R.keys;
         G.nslots = R.nslots;
         G.cap = S.cap;
@@ -1313,9 +1467,9 @@ int grad(const dp_tc_plan *plan, const dp_table_info *info, const double *s, con
     Q.natoms = n;
     const dim3 qgrid((unsigned)((n + kRowsWarps - 1) / kRowsWarps));
     if (env)
-      rows_force_kernel<<<qgrid, 32 * kRowsWarps, kRowsWarps * S.nkeys * sizeof(short), st>>>(Q);
+      rows_force_kernel<<<qgrid, 32 * kRowsWarps, kRowsWarps * map_stride(S.nkeys) * sizeof(short), st>>>(Q);
     else
-      rows_kernel<<<qgrid, 32 * kRowsWarps, kRowsWarps * S.nkeys * sizeof(short), st>>>(Q);
+      rows_kernel<<<qgrid, 32 * kRowsWarps, kRowsWarps * map_stride(S.nkeys) * sizeof(short), st>>>(Q);
     if ((rc = launch_status(who))) return rc;
     prof_mark("tc_rows", st);
   }

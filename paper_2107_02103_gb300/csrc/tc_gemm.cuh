@@ -32,7 +32,7 @@ namespace {
 // converts it to f64 once -- or, in the tabulation's GEMMs, recombines the
 // diagonals exactly as one 128-bit integer and rounds that once (diag_s128,
 // s128_to_f64).  The tabulation's backward, whose K is M1 <= 144, splits into
-// seven 8-bit digits instead (Digits7x8; 28 products, diag7_to_f64).
+// seven 8-bit digits instead (Digits7x8; 28 products, diag7_s128).
 // What rounds is that conversion, the 53-bit truncation of the operands and
 // the dropped terms: |error| <~ K 2^-49 max_k|a_ik| max_k|b_kj|, against
 // K 2^-53 sum_k |a_ik b_kj| for an f64 dot product.  A row or column with an
@@ -476,39 +476,21 @@ __device__ __forceinline__ double diag_to_f64(const float (&v)[kS][W], int c, in
 // integer S = sum_d v[d][c] 2^(8 (6 - d)), |S| < 2^72.01; an output is S 2^(E + F + kOutExp7x8).
 constexpr int kOutExp7x8 = 2 * Digits7x8::kPad - 2 * 8 - 8 * 6;
 template <int W>
-__device__ __forceinline__ __int128 diag7_int(const float (&v)[7][W], int c) {
-  long long A = 0;  // diagonals 3 .. 6: below 2^24 2^24 256/255 < 2^49
-#pragma unroll
-  for (int d = 3; d < 7; ++d) A += (long long)exact_int(v[d][c]) << (8 * (6 - d));
-  const long long T = (long long)exact_int(v[0][c]) * 65536 + (long long)exact_int(v[1][c]) * 256 + exact_int(v[2][c]);
-  return ((__int128)T << 32) + A;
-}
-template <int W>
-__device__ __forceinline__ double diag7_to_f64(const float (&v)[7][W], int c, int E, int F, bool &rare) {
+__device__ __forceinline__ void diag7_s128(const float (&v)[7][W], int c, long long &hi, unsigned long long &lo) {
   int x[7];
 #pragma unroll
   for (int d = 0; d < 7; ++d) x[d] = exact_int(v[d][c]);
   const long long T = (long long)x[0] * 65536 + (long long)x[1] * 256 + x[2];  // |T| < 2^40.01
   const long long A = (long long)x[3] * 16777216 + (long long)x[4] * 65536 + (long long)x[5] * 256 + x[6];  // < 2^48.01
   const unsigned long long tl = (unsigned long long)T << 32;
-  const unsigned long long lo = tl + (unsigned long long)A;
-  const long long hi = (T >> 32) + (A >> 63) + (lo < tl ? 1 : 0);
-  return s128_to_f64<kOutExp7x8>(hi, lo, E, F, rare);
-}
-__device__ __forceinline__ double output_value7(__int128 S, int E, int F) {
-  if (E >= kNonFinite || F >= kNonFinite) return __longlong_as_double(0x7ff8000000000000ll);
-  return i128_to_double(S, E + F + kOutExp7x8);
+  lo = tl + (unsigned long long)A;
+  hi = (T >> 32) + (A >> 63) + (lo < tl ? 1 : 0);
 }
 
-// The rare case of diag_to_f64 / diag7_to_f64 (a result outside the normal range), out of line so that
-// the epilogue loops stay small: one output from its diagonal sums (the seventh to ninth unused by the
-// 7 x 8 scheme).
+// The rare case of diag_to_f64 (a result outside the normal range), out of line so that the epilogue
+// loops stay small: one output from its diagonal sums.
 __device__ __noinline__ double output_value_rare(float v0, float v1, float v2, float v3, float v4, float v5, float v6,
-                                                 float v7, float v8, int E, int F, bool seven) {
-  if (seven) {
-    const float v[7][1] = {{v0}, {v1}, {v2}, {v3}, {v4}, {v5}, {v6}};
-    return output_value7(diag7_int(v, 0), E, F);
-  }
+                                                 float v7, float v8, int E, int F) {
   const float v[kS][1] = {{v0}, {v1}, {v2}, {v3}, {v4}, {v5}, {v6}, {v7}, {v8}};
   return output_value(diag_int(v, 0), E, F);
 }
@@ -737,11 +719,13 @@ int set_smem(const char *who) {
 // split_rows_kernel with the row exponents found in the same kernel: one warp per group of 8 rows and
 // all of K (lane = (row ri8 = lane / 4, pair of k kp = lane % 4)), a first pass over the rows for their
 // largest exponents (reduced over the row's four lanes), a second for the digits.  For short rows
-// (the tabulation's dT^T, K = M1), where a launch per pass costs more than the passes.
+// (the tabulation's dT^T, K = M1 <= 256), where a launch per pass costs more than the passes.  Also G with
+// sum_k |x_rk| < 2^G per row, G >= E (gexps; kNonFinite for a row with an inf or NaN).
 template <class D>
 __global__ void __launch_bounds__(128) split_rows_1k_kernel(const double *__restrict__ X, int64_t ld_r, int64_t ld_k,
                                                             int64_t nrows, int K, int64_t rows_p, int Kp, int RT,
-                                                            unsigned char *__restrict__ planes, int *__restrict__ exps) {
+                                                            unsigned char *__restrict__ planes, int *__restrict__ exps,
+                                                            int *__restrict__ gexps) {
   constexpr int NS = D::kNS;
   const int lane = threadIdx.x & 31, ri8 = lane >> 2, kp = lane & 3;
   const int64_t g = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);  // 8-row group
@@ -754,7 +738,20 @@ __global__ void __launch_bounds__(128) split_rows_1k_kernel(const double *__rest
   eb = max(eb, __shfl_xor_sync(0xffffffffu, eb, 1));
   eb = max(eb, __shfl_xor_sync(0xffffffffu, eb, 2));
   const int E = exp_of_max(eb);
-  if (kp == 0) exps[r] = E;
+  // the row's sum of magnitudes in units of 2^(E - 20), each rounded up: below 2^28 + 2^8
+  unsigned mag = 0;
+  for (int k0 = 0; k0 < Kp; k0 += 8)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const unsigned hw = (unsigned)__double2hiint(x(k0 + 2 * kp + h)) & 0x7fffffffu;  // |x| < (1 + m) 2^-20 2^(e - 1023)
+      mag += hw ? (((hw & 0xfffffu) + 0x100001u) >> min(max(E + 1023 - (int)(hw >> 20), 0), 31)) + 1u : 0u;
+    }
+  mag += __shfl_xor_sync(0xffffffffu, mag, 1);
+  mag += __shfl_xor_sync(0xffffffffu, mag, 2);
+  if (kp == 0) {
+    exps[r] = E;
+    gexps[r] = E >= kNonFinite ? kNonFinite : max(E, E - 20 + 32 - __clz((int)mag));
+  }
   const size_t plane = (size_t)RT * kTK * 2, block = NS * plane;
   const int ri = (int)(r % RT);
   unsigned char *rowbase = planes + (size_t)(r / RT) * (Kp / kTK) * block + (ri >> 3) * kSBO + (ri & 7) * 16 + kp * 4;
@@ -770,9 +767,9 @@ __global__ void __launch_bounds__(128) split_rows_1k_kernel(const double *__rest
 
 template <class D>
 int split_rows_1k(const double *X, int64_t ld_r, int64_t ld_k, int64_t nrows, int K, int64_t rows_p, int Kp, int RT,
-                  unsigned char *planes, unsigned char *exps, cudaStream_t st, const char *who) {
-  split_rows_1k_kernel<D><<<(unsigned)((rows_p / 8 + 3) / 4), 128, 0, st>>>(X, ld_r, ld_k, nrows, K, rows_p, Kp, RT,
-                                                                            planes, reinterpret_cast<int *>(exps));
+                  unsigned char *planes, unsigned char *exps, int *gexps, cudaStream_t st, const char *who) {
+  split_rows_1k_kernel<D><<<(unsigned)((rows_p / 8 + 3) / 4), 128, 0, st>>>(
+      X, ld_r, ld_k, nrows, K, rows_p, Kp, RT, planes, reinterpret_cast<int *>(exps), gexps);
   return launch_status(who);
 }
 
