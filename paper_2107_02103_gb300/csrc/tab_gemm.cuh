@@ -87,10 +87,11 @@ struct Params {
   int ka;   // K slices per row of blocks (forward: every K slice of the table; backward: M1 / 16)
   int nmt;  // 128-row tiles of A
   // B: blocks [ntiles][ka] of kS x kPlaneB bytes, or (W != NULL) made by the split warps from the
-  // moments W[natoms][cap][24] and the run map [natoms][nkeys]; F: [Np] column exponents
+  // moments W[natoms][cap][24] and the run map [natoms][mstride]; F: [Np] column exponents
   const unsigned char *bplanes;
   const double *W;
-  const int *map;
+  const short *map;
+  int mstride;
   const int *Fexp;
   int64_t ntiles, Np, Mp;
   // forward: the tile's used slices, in order ([ntiles][ka] and [ntiles]), in shares of 28
@@ -354,7 +355,7 @@ __global__ void __launch_bounds__(kThreadsP, 1) tgemm_kernel(const Params P) {
           const int key = (sl * kTK + 2 * kp) / 6;
 #pragma unroll
           for (int i = 0; i < kPairs; ++i)
-            slot[i] = (av[i] && key < P.nkeys) ? P.map[(a_base + i) * P.nkeys + key] : -1;
+            slot[i] = (av[i] && key < P.nkeys) ? P.map[(a_base + i) * P.mstride + key] : -1;
         };
         int j = ((w - g0) % kStages + kStages) % kStages;  // the warp's first slice of the unit
         // the warp's slices of the unit (at most 112 / 4 = 28): lane l holds entry j + 4 l of the list

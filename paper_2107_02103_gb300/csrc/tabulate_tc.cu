@@ -16,8 +16,8 @@
 //   dW_i[k][(l, q)] = (1/N_c) sum_m dT_i[k][m] c_q^{l,m},
 //   dE/dR~_j[k] = sum_q dW_i[k][(l, q)] t_j^q,
 //   dE/ds_j     = sum_k R~_j[k] sum_{q >= 1} q dW_i[k][(l, q)] t_j^(q-1)   (0 where s_j was clamped).
-// The FP64 pipe keeps 24 FMAs per row for W; the rows' derivatives (40 multiply-adds) run in fixed point on
-// the integer pipes (fixed.cuh); the per-interval work (24 M1 FMAs per interval and atom in
+// The per-row work (24 multiply-adds per row for W, 40 for the derivatives) runs in fixed point on the
+// integer pipes (fixed.cuh), the FP64 pipe converting; the per-interval work (24 M1 FMAs per interval and atom in
 // each direction), which is most of it, runs as exact digit-split GEMMs on
 // the tensor cores (tc_gemm.cuh), at f64 accuracy.
 //
@@ -177,7 +177,7 @@ Layout make_layout(const Shape &s) {
   L.keys = take(off, (size_t)std::max<int64_t>(s.nloc, 1) * s.cap * sizeof(short));
   L.nslots = take(off, (size_t)std::max<int64_t>(s.nloc, 1) * sizeof(int));
   L.occ = take(off, (size_t)s.ntypes * std::max<int64_t>(s.tiles_all, 1) * s.nsl);
-  L.map = take(off, (size_t)s.chunk * s.nkeys * sizeof(int));
+  L.map = take(off, std::max((size_t)s.chunk * s.nkeys * sizeof(int), (size_t)s.chunk * map_stride(s.nkeys) * sizeof(short)));
   L.slist = take(off, (size_t)s.ntypes * s.ntiles * s.nsl * sizeof(short));
   L.scount = take(off, (size_t)s.ntypes * s.ntiles * sizeof(int));
   L.units = take(off, (size_t)s.ntypes * std::max(s.maxunits, s.maxunits8) * sizeof(int));
@@ -349,17 +349,29 @@ struct RunsParams {
   short *keys;         // [nloc][cap]: key of each slot (every atom of the call)
   int *nslots;         // [nloc]: slots in use
   unsigned char *occ;  // [ntypes][tiles_all][nsl]: the K slices some atom of the tile uses
-  int *map;            // forward: [natoms][nkeys] run slot of the key, or -1 (this chunk)
+  short *map;          // forward: [natoms][map_stride(nkeys)] run slot of the key, or -1 (this chunk)
   double *W;           // forward: [natoms][cap][24] moments W[k][q] at 6 k + q
   int *fexp;           // forward: [Np] exponents of the columns 4 a + k
 };
 
+// A batch of 32 rows: R~ and the powers of u as fixed points (fx::Fix), or as doubles in a wild batch.
+// A row is a column of the stage (33 entries a row of it: neither the lanes' stores nor the reads of one row
+// by the 24 (k, q) lanes meet in a bank).
 struct alignas(16) RunsStage {
-  double r[32][4];
-  double tp[32][6];
-  int key[32];
+  long long r[4][33];
+  long long tp[6][33];
   int nvb[DP_MAX_TYPES];
 };
+static_assert(sizeof(fx::Fix) == sizeof(double), "a stage entry holds either");
+
+// The binary places of a batch's R~[k]: |R~[k]| 2^sh < 2^57 over its rows, from the largest high word
+// (sign off) of its values.  `wild`: an inf, a NaN or values so large or small that the sums' exponents
+// could leave the normal range; such a batch is summed on the FP64 pipe.
+__device__ __forceinline__ int batch_places(int hiword, bool &wild) {
+  const int eb = hiword >> 20;
+  wild |= hiword != 0 && (eb < 200 || eb > 1800);
+  return hiword ? 57 + 1022 - eb : 0;
+}
 
 // Valid rows per type segment of atom i (clamped into [0, sel]) into nvb; returns their total.
 __device__ __forceinline__ int valid_rows(const int32_t *nvalid, const int *sel, int ntypes, int64_t i, int lane,
@@ -392,123 +404,163 @@ __device__ __forceinline__ int valid_row(int v, const int *nvb, const int *sel, 
   return row;
 }
 
+// Warps (one atom each) per block of the runs and rows kernels: a few per block, so that launching
+// thousands of tiny blocks does not set the pace of a short kernel.
+constexpr int kRunsWarps = 4, kRowsWarps = 4;
 // One warp per atom: the runs of rows sharing an interval (consecutive rows with one key; rows
 // sorted by distance give one run per interval, and a key met again adds to its slot), each
 // interval's slot (a shared-memory map of the keys; each slot's key and the slot count are written
 // out) and the flags of its K slices for the atom's tile; forward also the map, its moments W and
 // the atom's four column exponents (over every value written, which bounds the final ones).
-// Warps (one atom each) per block of the runs and rows kernels: a few per block, so that launching
-// thousands of tiny blocks does not set the pace of a short kernel.
-constexpr int kRunsWarps = 4, kRowsWarps = 4;
-
+// Rows go in batches of 32, a lane per row.  The batch's new keys get their slots together (a lane per
+// run; the lowest lane of a key met twice leads), then the runs are summed one by one, lane 6 k + q
+// taking R~[k] u^q: limb products on the integer pipes (fixed.cuh) against the batch's largest R~[k] and
+// unit u, one conversion to f64 per run and lane.  Why: with FP64 moments the kernel took 80 sub-partition
+// clocks a row (24 of 32 lanes of a 68-clock FMA, the powers of u); 24 FMAs as limb products take 10.  And
+// with one pass of bookkeeping per run short runs spent longer on that than on their sums.  Measured:
+// copper 0.133 -> 0.078 ms, water (2.7 rows a run) 0.099 -> 0.084 ms.
 template <bool kMom, bool kEnv = false>
-__global__ void __launch_bounds__(32 * kRunsWarps) runs_kernel(const RunsParams P) {
+__global__ void __launch_bounds__(32 * kRunsWarps, 7) runs_kernel(const RunsParams P) {
+  constexpr int L = 28;  // limbs of the moments: 32 rows' products of 57 and 56 places stay below 2^63
+  using fx::Fix;
   __shared__ RunsStage stw[kRunsWarps];
-  extern __shared__ short smapw[];  // [kRunsWarps][nkeys]
+  extern __shared__ __align__(16) short smapw[];  // [kRunsWarps][map_stride(nkeys)]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t a = (int64_t)blockIdx.x * kRunsWarps + warp;
   if (a >= P.natoms) return;  // warp-uniform
   RunsStage &st = stw[warp];
-  short *smap = smapw + (size_t)warp * P.nkeys;
+  short *smap = smapw + (size_t)warp * map_stride(P.nkeys);
   const int64_t i = P.atom0 + a;
-  for (int k = lane; k < P.nkeys; k += 32) smap[k] = -1;
+  for (int k = lane; k < map_stride(P.nkeys) / 8; k += 32)
+    reinterpret_cast<int4 *>(smap)[k] = make_int4(-1, -1, -1, -1);
   const int nv = kEnv ? env_valid_rows(P.env, P.nnei, P.sel, P.ntypes, i, lane, st.nvb, P.nvalid_out)
                       : valid_rows(P.nvalid, P.sel, P.ntypes, i, lane, st.nvb);  // (their __syncwarp orders the reset)
   const int alpha = P.atype ? clampi(__ldg(P.atype + i), 0, P.ntypes - 1) : 0;
   unsigned char *occ = P.occ + ((size_t)alpha * P.tiles_all + (size_t)(i / kTileAtoms)) * P.nsl;
   short *keys = P.keys + i * P.cap;
-  double *Wa = kMom ? P.W + (size_t)a * P.cap * 24 : nullptr;
+  double *Wl = kMom ? P.W + (size_t)a * P.cap * 24 + min(lane, 23) : nullptr;
   int nslot = 0;
-  int cur = -1;       // key of the open run (uniform)
-  double wv = 0.0;    // its moment W[k][q] on lane 6 k + q < 24
-  int eb = 0;         // largest exponent field written by this lane
-  auto flush = [&]() {  // uniform
-    int slot = smap[cur];
-    const bool fresh = slot < 0;
-    __syncwarp();
-    if (fresh) {
-      slot = nslot++;
-      if (lane == 0) {
-        smap[cur] = (short)slot;
-        keys[slot] = (short)cur;
-        occ[kQ * cur / kTK] = 1;  // the key's entries 6 key .. 6 key + 5, in one or two slices
-        occ[(kQ * cur + kQ - 1) / kTK] = 1;
-      }
-    }
-    if (kMom && lane < 24) {
-      double *w = Wa + (size_t)slot * 24 + lane;
-      const double x = fresh ? wv : *w + wv;
-      *w = x;
-      eb = max(eb, exp_bits(x));
-    }
-    __syncwarp();
-  };
+  int eb = 0;  // largest exponent field written by this lane
+  const int lk = min(lane / 6, 3), lq = lane - 6 * (lane / 6);
   const double *srow = P.s + i * P.nnei;
   const double *Rrow = P.Rt + i * P.nnei * 4;
   for (int base = 0; base < nv; base += 32) {
     const int v = base + lane;
+    double r[4] = {0.0, 0.0, 0.0, 0.0}, u = 0.0;
+    int key = -1;
     if (v < nv) {
       int b;
-      const int row = valid_row(v, st.nvb, P.sel, P.ntypes, b);
-      double t, sv, r4[4];
+      double sv;
+      double t;
       if constexpr (kEnv) {
+        const int row = valid_row(v, st.nvb, P.sel, P.ntypes, b);
         const EnvVals ev = env_vals(P.env, i, __ldg(P.env.nlist + i * P.nnei + row));
         sv = ev.r4[0];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) r4[k] = ev.r4[k];
+        for (int k = 0; k < 4; ++k) r[k] = ev.r4[k];
       } else {
+        const int row = valid_row(v, st.nvb, P.sel, P.ntypes, b);
         sv = __ldg(srow + row);
+        if constexpr (kMom) {
+          const Vec4<double> rr = ld4(Rrow + (size_t)row * 4);
+          r[0] = rr.x, r[1] = rr.y, r[2] = rr.z, r[3] = rr.w;
+        }
       }
       bool clamped;
       const int l = locate_fast(P.g, P.gf, P.nodes, sv, t, clamped);
-      st.key[lane] = b * P.g.nint + l;
-      if constexpr (kMom) {
-        Vec4<double> rr;
-        if constexpr (kEnv)
-          rr = Vec4<double>{r4[0], r4[1], r4[2], r4[3]};
-        else
-          rr = ld4(Rrow + (size_t)row * 4);
-        st.r[lane][0] = rr.x;
-        st.r[lane][1] = rr.y;
-        st.r[lane][2] = rr.z;
-        st.r[lane][3] = rr.w;
-        const double u = t * (l < P.g.n0 ? P.g.inv0 : P.g.inv1);
-        const double u2 = u * u, u3 = u2 * u;
-        st.tp[lane][0] = 1.0;
-        st.tp[lane][1] = u;
-        st.tp[lane][2] = u2;
-        st.tp[lane][3] = u3;
-        st.tp[lane][4] = u2 * u2;
-        st.tp[lane][5] = u3 * u2;
-      }
+      key = b * P.g.nint + l;
+      u = t * (l < P.g.n0 ? P.g.inv0 : P.g.inv1);
     }
-    __syncwarp();
-    const int cnt = min(32, nv - base);
-    const int mykey = lane < cnt ? st.key[lane] : -1;
-    const int prev = __shfl_up_sync(0xffffffffu, mykey, 1);
-    unsigned starts = __ballot_sync(0xffffffffu, lane < cnt && (lane == 0 || mykey != prev));
-    while (starts) {  // uniform, run by run
-      const int u0 = __ffs(starts) - 1;
-      starts &= starts - 1;
-      const int e = starts ? __ffs(starts) - 1 : cnt;
-      const int key = __shfl_sync(0xffffffffu, mykey, u0);
-      if (key != cur) {
-        if (cur >= 0) flush();
-        cur = key;
-        wv = 0.0;
+    // the batch's runs and their slots
+    const int prev = __shfl_up_sync(0xffffffffu, key, 1);
+    const bool start = v < nv && (lane == 0 || key != prev);
+    int slot = start ? (int)smap[key] : 0;
+    const bool need = slot < 0;
+    unsigned starts = __ballot_sync(0xffffffffu, start);
+    bool fresh = false;
+    if (__any_sync(0xffffffffu, need)) {
+      const unsigned peers = __match_any_sync(0xffffffffu, need ? key : ~lane);
+      fresh = need && lane == __ffs(peers) - 1;
+      const unsigned lead = __ballot_sync(0xffffffffu, fresh);
+      if (fresh) {
+        slot = nslot + __popc(lead & ((1u << lane) - 1u));
+        smap[key] = (short)slot;
+        keys[slot] = (short)key;
+        occ[kQ * key / kTK] = 1;  // the key's entries 6 key .. 6 key + 5, in one or two slices
+        occ[(kQ * key + kQ - 1) / kTK] = 1;
       }
-      if (kMom && lane < 24) {
-        const int k = lane / 6, q = lane - 6 * (lane / 6);
-        for (int j = u0; j < e; ++j) wv = fma(st.r[j][k], st.tp[j][q], wv);
+      const int led = __shfl_sync(0xffffffffu, slot, __ffs(peers) - 1);
+      if (need) slot = led;
+      nslot += __popc(lead);
+    }
+    if constexpr (kMom) {
+      bool wild = false;  // uniform
+      int sh[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        sh[k] = batch_places(__reduce_max_sync(0xffffffffu, __double2hiint(r[k]) & 0x7fffffff), wild);
+      // |u| < 1.125 unless s is NaN (t lies in its interval but for a hair)
+      wild = wild || __any_sync(0xffffffffu, (__double2hiint(u) & 0x7fffffff) >= 0x3ff20000);
+      if (!wild) {
+        Fix *fr = reinterpret_cast<Fix *>(&st.r[0][lane]), *ft = reinterpret_cast<Fix *>(&st.tp[0][lane]);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) fr[33 * k] = fx::limbs<L>(fx::from_double(r[k], sh[k]));
+        const Fix u1 = fx::limbs<L>(fx::from_double(u, 2 * L)), u2 = fx::limbs<L>(fx::mul<L>(u1, u1)),
+                  u3 = fx::limbs<L>(fx::mul<L>(u2, u1));
+        ft[33 * 0] = Fix{0, 1 << L};
+        ft[33 * 1] = u1;
+        ft[33 * 2] = u2;
+        ft[33 * 3] = u3;
+        ft[33 * 4] = fx::limbs<L>(fx::mul<L>(u2, u2));
+        ft[33 * 5] = fx::limbs<L>(fx::mul<L>(u3, u2));
+      } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) st.r[k][lane] = __double_as_longlong(r[k]);
+        double up = 1.0;
+#pragma unroll
+        for (int q = 0; q < 6; ++q, up *= u) st.tp[q][lane] = __double_as_longlong(up);
+      }
+      __syncwarp();
+      const int scale = -(lk < 2 ? (lk ? sh[1] : sh[0]) : (lk == 2 ? sh[2] : sh[3]));
+      const int tag = slot | (fresh ? 1 << 16 : 0);
+      const int cnt = min(32, nv - base);
+      while (starts) {  // uniform, run by run
+        const int j0 = __ffs(starts) - 1;
+        starts &= starts - 1;
+        const int j1 = starts ? __ffs(starts) - 1 : cnt;
+        const int run = __shfl_sync(0xffffffffu, tag, j0);
+        if (lane < 24) {
+          double *w = Wl + (run & 0xffff) * 24;
+          const bool add = !(run >> 16);
+          const double old = add ? *w : 0.0;
+          double x = 0.0;
+          if (!wild) {
+            const Fix *pr = reinterpret_cast<const Fix *>(st.r[lk]), *pt = reinterpret_cast<const Fix *>(st.tp[lq]);
+            fx::Acc acc;
+            int j = j0;
+            for (; j + 4 <= j1; j += 4)
+#pragma unroll
+              for (int h = 0; h < 4; ++h) acc.mad(pr[j + h], pt[j + h]);
+#pragma unroll 1
+            for (; j < j1; ++j) acc.mad(pr[j], pt[j]);
+            x = fx::to_double(fx::over_unit<L>(acc, j1 - j0), scale);
+          } else {
+            for (int j = j0; j < j1; ++j)
+              x = fma(__longlong_as_double(st.r[lk][j]), __longlong_as_double(st.tp[lq][j]), x);
+          }
+          if (add) x += old;
+          *w = x;
+          eb = max(eb, exp_bits(x));
+        }
       }
     }
     __syncwarp();
   }
-  if (cur >= 0) flush();
   if (lane == 0) P.nslots[i] = nslot;
   if constexpr (kMom) {
-    int *map = P.map + a * P.nkeys;
-    for (int k = lane; k < P.nkeys; k += 32) map[k] = smap[k];
+    short *map = P.map + a * map_stride(P.nkeys);
+    for (int k = lane; k < map_stride(P.nkeys) / 8; k += 32)
+      reinterpret_cast<int4 *>(map)[k] = reinterpret_cast<const int4 *>(smap)[k];
     int m = eb;  // per k: the largest over its six lanes
 #pragma unroll
     for (int q = 1; q < 6; ++q) m = max(m, __shfl_sync(0xffffffffu, eb, min(lane + q, 31)));
@@ -898,7 +950,8 @@ __device__ __forceinline__ void row_component(const RowPoly &R, const fx::Fix *_
 
 // One warp per atom, a lane per valid row: the row's interval from s, its run slot from the atom's key map
 // (shared memory), the slot's gradient coefficients dW[k][q] read through L1 (the rows of a run share
-// them), and dE/dR~ and dE/ds from them (row_grad); padded rows get zeros.
+// them), and dE/dR~ and dE/ds from them (row_component); padded rows get zeros.  Seven blocks an SM keep 4,096
+// atoms in one wave (copper: six 0.094 ms, eight, with spills, 0.079).
 __global__ void __launch_bounds__(32 * kRowsWarps, 7) rows_kernel(const RowsParams P) {
   __shared__ int nvbw[kRowsWarps][DP_MAX_TYPES];
   extern __shared__ __align__(16) short smapw[];  // [kRowsWarps][map_stride(nkeys)]
@@ -1155,7 +1208,7 @@ RunsParams runs_params(const double *s, const double *Rt, const int32_t *nvalid,
   R.keys = reinterpret_cast<short *>(wk + L.keys);
   R.nslots = reinterpret_cast<int *>(wk + L.nslots);
   R.occ = wk + L.occ;
-  R.map = reinterpret_cast<int *>(wk + L.map);
+  R.map = reinterpret_cast<short *>(wk + L.map);
   R.fexp = reinterpret_cast<int *>(wk + L.fexp);
   R.nodes = nodes;
   return R;
@@ -1216,9 +1269,9 @@ int fwd(const dp_tc_plan *plan, const dp_table_info *info, const double *s, cons
     R.natoms = n;
     const dim3 rgrid((unsigned)((n + kRunsWarps - 1) / kRunsWarps));
     if (env)
-      runs_kernel<true, true><<<rgrid, 32 * kRunsWarps, kRunsWarps * S.nkeys * sizeof(short), st>>>(R);
+      runs_kernel<true, true><<<rgrid, 32 * kRunsWarps, kRunsWarps * map_stride(S.nkeys) * sizeof(short), st>>>(R);
     else
-      runs_kernel<true><<<rgrid, 32 * kRunsWarps, kRunsWarps * S.nkeys * sizeof(short), st>>>(R);
+      runs_kernel<true><<<rgrid, 32 * kRunsWarps, kRunsWarps * map_stride(S.nkeys) * sizeof(short), st>>>(R);
     if ((rc = launch_status(who))) return rc;
     prof_mark("tc_runs_moments", st);
     const int64_t nlist = (int64_t)ntypes * ntiles;
@@ -1245,6 +1298,7 @@ int fwd(const dp_tc_plan *plan, const dp_table_info *info, const double *s, cons
     G.W = R.W;  // B made from the moments inside the GEMM
     G.map = R.map;
     G.nkeys = S.nkeys;
+    G.mstride = map_stride(S.nkeys);
     G.cap = S.cap;
     G.Fexp = R.fexp;
     G.ntiles = ntiles;
@@ -1356,9 +1410,9 @@ int grad(const dp_tc_plan *plan, const dp_table_info *info, const double *s, con
     if (!reuse) {
       const dim3 rgrid((unsigned)((n + kRunsWarps - 1) / kRunsWarps));
       if (env)
-        runs_kernel<false, true><<<rgrid, 32 * kRunsWarps, kRunsWarps * S.nkeys * sizeof(short), st>>>(R);
+        runs_kernel<false, true><<<rgrid, 32 * kRunsWarps, kRunsWarps * map_stride(S.nkeys) * sizeof(short), st>>>(R);
       else
-        runs_kernel<false><<<rgrid, 32 * kRunsWarps, kRunsWarps * S.nkeys * sizeof(short), st>>>(R);
+        runs_kernel<false><<<rgrid, 32 * kRunsWarps, kRunsWarps * map_stride(S.nkeys) * sizeof(short), st>>>(R);
       if ((rc = launch_status(who))) return rc;
       prof_mark("tc_runs", st);
     }
