@@ -5,7 +5,7 @@
 // 32 x 32 + 64-bit integer multiply-add per 2.4 sub-partition clocks.  A sum of products
 //   sum_i a_i b_i,  a = ah 2^L + al,  b = bh 2^L + bl  (al, bl in [0, 2^L); ah, bh signed),
 // needs no carries when its two leading limb products are summed apart,
-//   hi += ah bh,  mid += ah bl + al bh,  sum = hi 2^2L + mid 2^L + (al bl, dropped: its mean is added once),
+//   hi += ah bh,  mid += ah bl + al bh,  sum = hi 2^2L + mid 2^L + (al bl, dropped: below 2^2L a term),
 // three multiply-adds a term, a ninth of the one FP64 instruction it replaces.  The values are fixed
 // points against a power of two that bounds them (the largest of a batch of rows; a row of the table times
 // a column of dE/dT), with 56 to 61 places below it: each term's error lies below that of an f64 product
@@ -49,11 +49,11 @@ struct Acc {
     mid = mad_wide(a.lo, b.hi, mid);
   }
 };
-// The sum over 2^2L, of n terms, to the nearest integer but for the spread of the dropped limb products
-// (each between 0 and 1, 1/4 on average).
+// The sum over 2^2L to the nearest integer but for the dropped limb products (each between 0 and 1); a sum
+// of zeros is zero.
 template <int L>
-__device__ __forceinline__ long long over_unit(const Acc &p, int n) {
-  return p.hi + ((p.mid + ((2ll + n) << (L - 2))) >> L);
+__device__ __forceinline__ long long over_unit(const Acc &p) {
+  return p.hi + ((p.mid + (1ll << (L - 1))) >> L);
 }
 
 // a b / 2^2L as limbs: the product of a fixed point in units of 2^-2L with any other.
@@ -61,7 +61,7 @@ template <int L>
 __device__ __forceinline__ long long mul(const Fix a, const Fix b) {
   Acc p;
   p.mad(a, b);
-  return over_unit<L>(p, 1);
+  return over_unit<L>(p);
 }
 
 // x 2^sh truncated toward zero, |x 2^sh| < 2^62: the exponent moved by an integer add, one conversion on

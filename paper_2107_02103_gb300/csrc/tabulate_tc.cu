@@ -543,7 +543,7 @@ __global__ void __launch_bounds__(32 * kRunsWarps, 7) runs_kernel(const RunsPara
               for (int h = 0; h < 4; ++h) acc.mad(pr[j + h], pt[j + h]);
 #pragma unroll 1
             for (; j < j1; ++j) acc.mad(pr[j], pt[j]);
-            x = fx::to_double(fx::over_unit<L>(acc, j1 - j0), scale);
+            x = fx::to_double(fx::over_unit<L>(acc), scale);
           } else {
             for (int j = j0; j < j1; ++j)
               x = fma(__longlong_as_double(st.r[lk][j]), __longlong_as_double(st.tp[lq][j]), x);
@@ -934,7 +934,7 @@ __device__ __forceinline__ void row_component(const RowPoly &R, const fx::Fix *_
   q.mad(c3, R.u2);
   q.mad(c4, R.u3);
   q.mad(c5, R.u4);
-  const long long pv = fx::over_unit<L>(p, 5), qv = fx::whole<L>(c1) + fx::over_unit<L>(q, 4);
+  const long long pv = fx::over_unit<L>(p), qv = fx::whole<L>(c1) + fx::over_unit<L>(q);
   const int ep = R.ke.x + g - tg::kGradPlaces, eq = R.ke.y + g - tg::kGradPlaces + R.e;
   if (R.plain) {
     const int ph = (int)(pv >> 32);

@@ -25,15 +25,15 @@ def acc(terms, b):
     return hi, mid
 
 
-def over_unit(p, n, b):
+def over_unit(p, b):
     hi, mid = p
-    mid += (2 + n) << (b - 2)
+    mid += 1 << (b - 1)
     assert abs(mid) < 1 << 63
     return hi + (mid >> b)
 
 
 def mul(x, y, b):
-    return over_unit(acc([(x, y)], b), 1, b)
+    return over_unit(acc([(x, y)], b), b)
 
 
 def key_exps(E, e):
@@ -71,8 +71,8 @@ def test_row_polynomial(case):
         D = [round(q * d[q] / Fr(2) ** (slope + G - PLACES)) for q in range(6)]
         d0 = round(d[0] / Fr(2) ** (value + G - PLACES))
         assert sum(abs(x) for x in D) < 1 << PLACES
-        p = over_unit(acc([(D[q], w[q]) for q in range(1, 6)], L), 5, L)
-        g = D[1] + over_unit(acc([(D[q], uq[q - 1]) for q in range(2, 6)], L), 4, L)
+        p = over_unit(acc([(D[q], w[q]) for q in range(1, 6)], L), L)
+        g = D[1] + over_unit(acc([(D[q], uq[q - 1]) for q in range(2, 6)], L), L)
         P = d0 + (p >> (value - slope))
         assert abs(P) < 1 << 62 and abs(g) < 1 << 62
         ex = sum(d[q] * u**q for q in range(6)) / Fr(2) ** (value + G - PLACES)
@@ -94,7 +94,7 @@ def test_moment_sums():
         u3 = mul(u2, u1, b)
         powers = [1 << 56, u1, u2, u3, mul(u2, u2, b), mul(u3, u2, b)]
         for q in range(6):
-            got = over_unit(acc([(int(x), powers[q]) for x in r], b), 32, b)
+            got = over_unit(acc([(int(x), powers[q]) for x in r], b), b)
             # the power's own error (at most q + 1 units of 2^-56) times R~ < 2^57, and the dropped limbs
             assert abs(got - sum(r) * u**q) <= 32 * (2 * (q + 1) + 1)
             assert abs(got) < 1 << 63

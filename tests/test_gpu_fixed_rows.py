@@ -87,6 +87,15 @@ def test_infs_nans_and_zero_columns(setup, M1):
     assert _same(g, ds)
 
 
+def test_zero_components_stay_zero(setup):
+    """A plane of atoms: R~'s z components are zero in every batch, and so are T's z row and its part of ds."""
+    w, m, x = setup[20]
+    Rt = x["Rt"].clone()
+    Rt[..., 3] = 0.0
+    T, T0 = _fwd(m, x, w, Rt=Rt), _fwd(m, x, w)
+    assert not T[:, 3].any() and _same(T[:, :3], T0[:, :3])
+
+
 def test_every_nvalid_and_order(setup):
     """Rows in random order (keys met again within a batch of 32 and in later ones) against the sorted rows:
     T within the rounding of its sums, each row's gradients to the bit."""
