@@ -6,6 +6,9 @@
 // in storage order: every FP64 instruction has 32 busy lanes (M1*M2 is a
 // multiple of 32 for the paper's shapes) and every store is coalesced.
 // Both kernels also run in df64 arithmetic on double arrays (io_t).
+#include <type_traits>
+
+#include "desc_fixed.cuh"
 #include "dp_common.cuh"
 
 namespace dpc {
@@ -43,6 +46,17 @@ __global__ void __launch_bounds__(kDescWarps * 32)
       ++m;
     }
   }
+}
+
+// The same in f64: a block per atom, in fixed point (desc_fixed.cuh).
+__global__ void __launch_bounds__(kDescWarps * 32)
+    descriptor_f64_kernel(const double *__restrict__ T, int M1, int M2, double *__restrict__ D) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  double *Ts = reinterpret_cast<double *>(smem_raw);
+  const int64_t i = blockIdx.x;
+  for (int e = threadIdx.x; e < 4 * M1; e += blockDim.x) Ts[e] = __ldg(T + i * 4 * M1 + e);
+  __syncthreads();
+  dfx::desc_tile(Ts, M1, M2, D + i * (int64_t)M1 * M2);
 }
 
 // dD_i is staged in shared memory (read once, coalesced, converted once) in df64, where each
@@ -173,16 +187,21 @@ int descriptor(const io_t<real> *T, int64_t nloc, int M1, int M2, io_t<real> *D,
   if (M1 > 4096) return set_error(DP_ERR_UNSUPPORTED, "M1 = %d > 4096", M1);
   if (nloc == 0) return DP_OK;
   if (!T || !D) return set_error(DP_ERR_NULL, "T or D is NULL");
-  const int64_t blocks = (nloc + kDescWarps - 1) / kDescWarps;
+  constexpr bool f64 = std::is_same<real, double>::value;
+  const int64_t blocks = f64 ? nloc : (nloc + kDescWarps - 1) / kDescWarps;
   if (blocks > 2147483647LL) return set_error(DP_ERR_SHAPE, "nloc too large");
-  const size_t smem = (size_t)kDescWarps * 4 * M1 * sizeof(real);
-  if (smem > 227 * 1024) return set_error(DP_ERR_UNSUPPORTED, "M1 = %d needs too much shared memory", M1);
+  if ((size_t)kDescWarps * 4 * M1 * sizeof(real) > 227 * 1024)
+    return set_error(DP_ERR_UNSUPPORTED, "M1 = %d needs too much shared memory", M1);
+  const size_t smem = (size_t)(f64 ? 2 : kDescWarps) * 4 * M1 * sizeof(real);
+  const void *kernel = f64 ? (const void *)descriptor_f64_kernel : (const void *)descriptor_kernel<real>;
   if (smem > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(descriptor_kernel<real>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)smem);
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return set_error(DP_ERR_CUDA, "dp_descriptor_contract: %s", cudaGetErrorString(e));
   }
-  descriptor_kernel<real><<<(unsigned)blocks, kDescWarps * 32, smem, (cudaStream_t)stream>>>(T, nloc, M1, M2, D);
+  if constexpr (f64)
+    descriptor_f64_kernel<<<(unsigned)blocks, kDescWarps * 32, smem, (cudaStream_t)stream>>>(T, M1, M2, D);
+  else
+    descriptor_kernel<real><<<(unsigned)blocks, kDescWarps * 32, smem, (cudaStream_t)stream>>>(T, nloc, M1, M2, D);
   return launch_status("dp_descriptor_contract");
 }
 

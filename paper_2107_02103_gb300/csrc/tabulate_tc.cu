@@ -51,6 +51,7 @@
 #include <algorithm>
 #include <cstdint>
 
+#include "desc_fixed.cuh"
 #include "dp_common.cuh"
 #include "env_row.cuh"
 #include "fixed.cuh"
@@ -786,8 +787,8 @@ __global__ void __launch_bounds__(32 * tb::kAtomsB) bwd_units8_kernel(const shor
 // tile, a 128-row tile of A) was cut into several pieces -- the pieces' exact integers added as 128-bit
 // integers and rounded once to f64 (s128_to_f64: no FP64 instruction) -- or has no used slices (T = 0);
 // the other atoms' T the GEMM wrote.  Then, when D is wanted, the atom's descriptor D[m][n] =
-// sum_k T[k][m] T[k][n] (n < M2) from its T staged in shared memory, in descriptor_kernel's order of
-// operations, so that the two give the same bits.
+// sum_k T[k][m] T[k][n] (n < M2) from its T staged in shared memory, by the descriptor call's own function,
+// so that the two give the same bits.
 __global__ void __launch_bounds__(128) fwd_finish_kernel(const longlong2 *__restrict__ part, int Mp,
                                                          const int *__restrict__ eexp, const int *__restrict__ fexp,
                                                          const int *__restrict__ npieces,
@@ -795,7 +796,7 @@ __global__ void __launch_bounds__(128) fwd_finish_kernel(const longlong2 *__rest
                                                          int64_t atom0, const int32_t *__restrict__ atype,
                                                          int ntypes, int M1, double *__restrict__ T, int M2,
                                                          double *__restrict__ D) {
-  extern __shared__ double Ts[];  // [4][M1], when D is wanted
+  extern __shared__ double Ts[];  // [4][M1] twice, when D is wanted: T and its fixed points
   const int64_t a = blockIdx.x;
   const int64_t tile = a / kTileAtoms;
   const int al = (int)(a - tile * kTileAtoms);
@@ -834,15 +835,7 @@ __global__ void __launch_bounds__(128) fwd_finish_kernel(const longlong2 *__rest
   }
   if (!D) return;  // uniform
   __syncthreads();
-  double *Da = D + (atom0 + a) * (int64_t)M1 * M2;
-  for (int e = threadIdx.x; e < M1 * M2; e += blockDim.x) {
-    const int m = e / M2, n = e - m * M2;
-    double v = Ts[m] * Ts[n];
-    v = fma(Ts[M1 + m], Ts[M1 + n], v);
-    v = fma(Ts[2 * M1 + m], Ts[2 * M1 + n], v);
-    v = fma(Ts[3 * M1 + m], Ts[3 * M1 + n], v);
-    Da[e] = v;
-  }
+  dfx::desc_tile(Ts, M1, M2, D + (atom0 + a) * (int64_t)M1 * M2);
 }
 
 struct RowsParams {
@@ -1318,7 +1311,7 @@ int fwd(const dp_tc_plan *plan, const dp_table_info *info, const double *s, cons
     G.ntypes = ntypes;
     if ((rc = tg::launch(G, st, who, ncta))) return rc;
     prof_mark("tc_gemm_fwd", st);
-    fwd_finish_kernel<<<(unsigned)n, 128, D ? (size_t)kCols * M1 * sizeof(double) : 0, st>>>(
+    fwd_finish_kernel<<<(unsigned)n, 128, D ? (size_t)2 * kCols * M1 * sizeof(double) : 0, st>>>(
         part, S.Mpf, G.Eexp, R.fexp, reinterpret_cast<const int *>(wk + L.npieces),
         reinterpret_cast<const int *>(wk + L.pfirst), ntiles, nmt, c0, atype, ntypes, M1, T, M2, D);
     if ((rc = launch_status(who))) return rc;
