@@ -154,6 +154,132 @@ __global__ void __launch_bounds__(kDescWarps * 32)
   for (int e = lane; e < 4 * M1; e += 32) dTi[e] = to_io(Gs[e]);
 }
 
+// The same in f64, a block per atom, in fixed point (fixed.cuh): T_i [4][M1] and dD_i [M1][M2] staged in
+// shared memory as two-limb integers (T against the largest of each k, dD against its own), every sum taken in
+// pieces of 16 terms whose limb products stay exact in 64 bits (57 places, limbs of 28 bits: hi below 2^62),
+// one conversion to f64 per piece.  First the 4 M1 sums over n (M2 terms), then the 4 M2 sums over m' (M1
+// terms), spread over the block by piece and added in their order.  Rows of dD are padded to M2 + 1 entries.
+// Why: 8 M1 M2 FP64 multiply-adds an atom bound the kernel above (79 % of that pipe, copper); as limb
+// products they cost a ninth, and the FP64 pipe converts M1 M2 inputs and a sum per 16 terms.
+// Measured: copper (4,096 x 100 x 16) 0.104 -> 0.058 ms; 1,536 atoms 0.047 -> 0.031 ms.
+constexpr int kGradPiece = 16, kGradL = 28, kDescGradPlaces = 57;
+constexpr int kDescGradThreads = 128;
+__host__ __device__ constexpr int pieces_of(int n) { return (n + kGradPiece - 1) / kGradPiece; }
+// 8-byte entries of shared memory: T, dD, the first term, the second term's pieces
+__host__ __device__ constexpr size_t desc_grad_f64_entries(int M1, int M2) {
+  return (size_t)8 * M1 + (size_t)M1 * (M2 + 1) + (size_t)4 * M2 * pieces_of(M1);
+}
+__global__ void __launch_bounds__(kDescGradThreads)
+    descriptor_grad_f64_kernel(const double *__restrict__ T, const double *__restrict__ dD, int M1, int M2,
+                               double *__restrict__ dT) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int red[5];  // the largest high words: of T's rows, of dD
+  using fx::Fix;
+  Fix *Tf = reinterpret_cast<Fix *>(smem_raw);              // [4][M1]
+  double *G = reinterpret_cast<double *>(Tf + 4 * M1);       // [4][M1]
+  Fix *Df = reinterpret_cast<Fix *>(G + 4 * M1);             // [M1][M2 + 1]
+  double *H = reinterpret_cast<double *>(Df + M1 * (M2 + 1));  // [pieces][4 M2]
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int64_t i = blockIdx.x;
+  const double *Ti = T + i * 4 * M1, *Di = dD + i * (int64_t)M1 * M2;
+  double *Td = reinterpret_cast<double *>(Tf), *Dd = reinterpret_cast<double *>(Df);
+  if (tid < 5) red[tid] = 0;
+  __syncthreads();
+  int hd = 0;
+  {
+    const int step_m = kDescGradThreads / M2, step_n = kDescGradThreads - step_m * M2;
+    int m = tid / M2, n = tid - m * M2;
+#pragma unroll 4
+    for (int e = tid; e < M1 * M2; e += kDescGradThreads) {
+      const double x = __ldg(Di + e);
+      Dd[m * (M2 + 1) + n] = x;
+      hd = max(hd, __double2hiint(x) & 0x7fffffff);
+      m += step_m;
+      n += step_n;
+      if (n >= M2) n -= M2, ++m;
+    }
+  }
+  hd = __reduce_max_sync(0xffffffffu, hd);
+  if (lane == 0) atomicMax(red + 4, hd);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    int ht = 0;
+    for (int m = tid; m < M1; m += kDescGradThreads) {
+      const double x = __ldg(Ti + k * M1 + m);
+      Td[k * M1 + m] = x;
+      ht = max(ht, __double2hiint(x) & 0x7fffffff);
+    }
+    ht = __reduce_max_sync(0xffffffffu, ht);
+    if (lane == 0) atomicMax(red + k, ht);
+  }
+  __syncthreads();
+  bool wild = false;
+  const int sd = dfx::places_of(red[4], kDescGradPlaces, wild);
+  int st[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) st[k] = dfx::places_of(red[k], kDescGradPlaces, wild);
+  auto places_t = [&](int k) { return k < 2 ? (k ? st[1] : st[0]) : (k == 2 ? st[2] : st[3]); };
+  const int np = pieces_of(M1);
+  if (!wild) {  // uniform over the block
+    // (the padding entries hold whatever the memory held and are not read again)
+    for (int e = tid; e < M1 * (M2 + 1); e += kDescGradThreads) Df[e] = fx::limbs<kGradL>(fx::from_double(Dd[e], sd));
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      for (int m = tid; m < M1; m += kDescGradThreads)
+        Tf[k * M1 + m] = fx::limbs<kGradL>(fx::from_double(Td[k * M1 + m], st[k]));
+    __syncthreads();
+    // sum over cnt <= 16 terms of a (stride sa) times b (consecutive), over 2^(2 L)
+    auto piece = [&](const Fix *a, int sa, const Fix *b, int cnt) {
+      fx::Acc p;
+      if (cnt == kGradPiece) {
+#pragma unroll
+        for (int q = 0; q < kGradPiece; ++q, a += sa) p.mad(*a, b[q]);
+      } else {
+        for (int q = 0; q < cnt; ++q, a += sa) p.mad(*a, b[q]);
+      }
+      return fx::over_unit<kGradL>(p);
+    };
+    for (int p = tid; p < 4 * M1; p += kDescGradThreads) {  // pairs 4 m + k
+      const int m = p >> 2, k = p & 3, ex = 2 * kGradL - sd - places_t(k);
+      double v = 0.0;
+      for (int n = 0; n < M2; n += kGradPiece)
+        v += fx::to_double(piece(Df + m * (M2 + 1) + n, 1, Tf + k * M1 + n, min(kGradPiece, M2 - n)), ex);
+      G[k * M1 + m] = v;
+    }
+    for (int p = tid; p < 4 * M2 * np; p += kDescGradThreads) {  // (piece, k, m), m fastest
+      const int c = p / (4 * M2), r = p - c * 4 * M2, k = r / M2, m = r - k * M2, m0 = c * kGradPiece;
+      H[p] = fx::to_double(piece(Df + m0 * (M2 + 1) + m, M2 + 1, Tf + k * M1 + m0, min(kGradPiece, M1 - m0)),
+                           2 * kGradL - sd - places_t(k));
+    }
+  } else {
+    for (int p = tid; p < 4 * M1; p += kDescGradThreads) {
+      const int m = p >> 2, k = p & 3;
+      double v = 0.0;
+      for (int n = 0; n < M2; ++n) v = fma(Dd[m * (M2 + 1) + n], Td[k * M1 + n], v);
+      G[k * M1 + m] = v;
+    }
+    for (int p = tid; p < 4 * M2 * np; p += kDescGradThreads) {
+      const int c = p / (4 * M2), r = p - c * 4 * M2, k = r / M2, m = r - k * M2;
+      double v = 0.0;
+      for (int mp = c * kGradPiece; mp < min(M1, c * kGradPiece + kGradPiece); ++mp)
+        v = fma(Dd[mp * (M2 + 1) + m], Td[k * M1 + mp], v);
+      H[p] = v;
+    }
+  }
+  __syncthreads();
+  double *dTi = dT + i * 4 * M1;
+  for (int e = tid; e < 4 * M1; e += kDescGradThreads) {
+    const int k = e / M1, m = e - k * M1;
+    double v = G[e];
+    if (m < M2) {
+      double s = H[k * M2 + m];
+      for (int c = 1; c < np; ++c) s += H[c * 4 * M2 + k * M2 + m];
+      v += s;
+    }
+    dTi[e] = v;
+  }
+}
+
 template <typename real>
 int descriptor_grad(const io_t<real> *T, const io_t<real> *dD, int64_t nloc, int M1, int M2, io_t<real> *dT,
                     void *stream) {
@@ -166,6 +292,20 @@ int descriptor_grad(const io_t<real> *T, const io_t<real> *dD, int64_t nloc, int
   if (!T || !dD || !dT) return set_error(DP_ERR_NULL, "T, dD or dT is NULL");
   const int64_t blocks = (nloc + kDescWarps - 1) / kDescWarps;
   if (blocks > 2147483647LL) return set_error(DP_ERR_SHAPE, "nloc too large");
+  if constexpr (std::is_same<real, double>::value) {
+    // in fixed point wherever the staged dD_i leaves at least four blocks to an SM; the kernel below, which
+    // does not stage it, for wider ones
+    const size_t need = desc_grad_f64_entries(M1, M2) * sizeof(double);
+    if (need <= 56 * 1024 && nloc <= 2147483647LL && M1 <= 1024) {
+      if (need > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(descriptor_grad_f64_kernel,
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
+        if (e != cudaSuccess) return set_error(DP_ERR_CUDA, "dp_descriptor_contract_grad: %s", cudaGetErrorString(e));
+      }
+      descriptor_grad_f64_kernel<<<(unsigned)nloc, kDescGradThreads, need, (cudaStream_t)stream>>>(T, dD, M1, M2, dT);
+      return launch_status("dp_descriptor_contract_grad");
+    }
+  }
   const size_t smem = (size_t)kDescWarps * desc_grad_smem_per_warp<real>(M1, M2) * sizeof(real);
   if (smem > 227 * 1024) return set_error(DP_ERR_UNSUPPORTED, "M1 = %d, M2 = %d need too much shared memory", M1, M2);
   if (smem > 48 * 1024) {
