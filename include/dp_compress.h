@@ -607,12 +607,12 @@ int dp_fitting_grad_df64(const double *params, const int32_t *widths, int nlayer
  * The f64 fitting net with its hidden-layer GEMMs on the tensor cores
  * (tcgen05).  Same inputs, outputs and results as dp_fitting_fwd_f64 /
  * dp_fitting_grad_f64 (Sec. II: E_i from D_i, and dE_i/dD_i), to f64
- * accuracy: every GEMM operand element is split exactly into nine balanced
- * 6-bit digits scaled by its row's (A) or column's (B) power of two, the 45 digit
+ * accuracy: every GEMM operand element is split exactly into eight balanced
+ * 7-bit digits scaled by its row's (A) or column's (B) power of two, the 36 digit
  * products that matter run as fp16 MMAs whose fp32 sums are exact integers
- * (at most 1792 of K per partial sum), and those sums are recombined exactly
+ * (at most 512 of K per partial sum), and those sums are recombined exactly
  * before one rounding to f64.  Per output the error is below about
- * K 2^-49 max_k |a_ik| max_k |b_kj| (an f64 dot product: K 2^-53 sum_k
+ * K 2^-50 max_k |a_ik| max_k |b_kj| (an f64 dot product: K 2^-53 sum_k
  * |a_ik b_kj|).  A row or column holding inf or NaN gives NaN outputs.  The
  * paper computes the net in double; this is that computation on hardware
  * whose FP64 rate is ~1000 times below its fp16 tensor rate.

@@ -24,7 +24,7 @@
 #include <cstdint>
 
 #include "dp_common.cuh"
-#include "tc_gemm.cuh"
+#include "fit_gemm.cuh"
 
 namespace dpc {
 namespace {
@@ -401,61 +401,8 @@ int fitting_grad(const io_t<real> *params, const int32_t *widths, int nlayer, in
 }
 
 // ------------------------------------------------- f64 GEMMs on the tensor cores
-// (tc_gemm.cuh: the digit splitting, the split kernels and gemm_kernel)
-namespace tc {
-
-// The layer's epilogue over the chunk's n x N outputs, from the shares' partial results summed in
-// a fixed order (so a call's results do not depend on timing):
-//   forward:  t = tanh(acc + bias); act[row][col] = t; V[row][col] = t (+ A[row][col] when the layer
-//             keeps its width: the identity skip, v_l = t_l + v_{l-1})
-//   backward: s = acc (+ S[row][col] or g_row wo_col when the layer kept its width); then either
-//             out[row][col] = s (dE/dD, the last GEMM) or S_next[row][col] = s and
-//             Z[row][col] = s (1 - t_prev^2) with t_prev = T[row][col] (the next GEMM's A)
-
-template <bool kFwd>
-__global__ void __launch_bounds__(256) epilogue_kernel(const TcGemm P, int ksplit) {
-  // rows over the grid, columns over the block (no 64-bit division per element)
-  for (int64_t rc = blockIdx.x; rc < P.n; rc += gridDim.x)
-  for (int nn = threadIdx.x; nn < P.N; nn += blockDim.x) {
-    const int64_t row = P.r0 + rc;
-    Sum3 acc;
-    for (int z = 0; z < ksplit; ++z) acc.add(P.part[((size_t)z * P.Mp + rc) * P.Np + nn]);
-    double v = acc.value(P.Eexp[rc], P.Fexp[nn]);
-    if constexpr (kFwd) {
-      if (P.lin) {
-        P.V[row * P.ldv + nn] = v + P.bias[nn];
-      } else {
-        const double t = dfl::tanh_d(v + P.bias[nn]);
-        P.act[row * P.ldact + nn] = t;
-        P.V[row * P.ldv + nn] = P.skip ? t + P.A[row * P.lda + nn] : t;
-      }
-    } else {
-      if (P.skip) v += P.S ? P.S[row * P.ldS + nn] : (P.g ? P.g[row] : 1.0) * P.wo[nn];
-      if (P.T) {
-        const double t = P.T[row * P.ldT + nn];
-        P.Snext[row * P.ldz + nn] = v;
-        P.Z[row * P.ldz + nn] = v * fma(-t, t, 1.0);
-      } else {
-        P.out[row * P.ldo + nn] = v;
-      }
-    }
-  }
-}
-
-// dz of the last hidden layer: Z[row][k] = s (1 - t_k^2), t its tanh outputs and s = dE/dv of that layer:
-// g_row wo_k (one output) or S[row][k] (several: g W_out^T, made first)
-__global__ void __launch_bounds__(256) last_dz_kernel(int64_t r0, int64_t n, int K, const double *__restrict__ g,
-                                                      const double *__restrict__ wo, const double *__restrict__ S,
-                                                      int64_t ldS, const double *__restrict__ T, int64_t ldT,
-                                                      double *__restrict__ Z, int64_t ldz) {
-  for (int64_t rr = blockIdx.x; rr < n; rr += gridDim.x)
-  for (int k = threadIdx.x; k < K; k += blockDim.x) {
-    const int64_t row = r0 + rr;
-    const double t = T[row * ldT + k];
-    const double sv = S ? S[row * ldS + k] : (g ? g[row] : 1.0) * wo[k];
-    Z[row * ldz + k] = sv * fma(-t, t, 1.0);
-  }
-}
+// (tc_gemm.cuh: the digit splitting; fit_gemm.cuh: the GEMM with its epilogues and the split kernels)
+namespace tf {
 
 // The GEMMs on the tensor cores: the hidden layers, and with several outputs the output layer too
 // (forward: v W_out + b_out; backward: g W_out^T, first).  GEMM q of a direction works on layer
@@ -465,10 +412,7 @@ int gemm_layer(const FitShape &s, bool fwd, int q) {
   return fwd ? q + 1 : s.nlayer - q - (s.nout > 1 ? 0 : 1);
 }
 
-// Where the B planes and column exponents of each GEMM of one type sit in the work buffer.  After
-// them come the A planes and row exponents of one chunk of at most kChunkRows atoms, and the
-// [nloc][max hidden width] buffers between layers (forward: 2, backward: 4).
-constexpr int64_t kChunkRows = 16384;
+// Where the B planes and column exponents of each GEMM sit in one type's share of the work buffer.
 struct Layer {
   int K, N, Np, Kp;
   size_t planes, fexp;  // byte offsets
@@ -480,112 +424,233 @@ size_t layout(const FitShape &s, bool fwd, Layer *out) {
     Layer &L = out[q];
     L.K = fwd ? s.w[l - 1] : s.w[l];
     L.N = fwd ? s.w[l] : s.w[l - 1];
-    L.Np = (int)round_up(L.N, kTN);
+    L.Np = (int)round_up(L.N, kTNF);
     L.Kp = (int)round_up(L.K, kTK);
     L.planes = off;
-    off += (size_t)round_up((int64_t)kS * L.Np * L.Kp * 2, 256);
+    off += (size_t)round_up((int64_t)kSF * L.Np * L.Kp * 2, 256);
     L.fexp = off;
     off += (size_t)round_up((int64_t)L.Np * 4, 256);
   }
   return off;
 }
 
-struct WorkMap {
-  size_t bplanes;          // bytes of the B planes (the larger of the two directions)
-  size_t aplanes, aexp;    // byte offsets of the A planes and row exponents of one chunk
-  int64_t Mp;              // rows of A planes per chunk
-  int Kpmax;
-  size_t part;             // byte offset of the shares' partial results
-  size_t buffers;          // byte offset of the buffers between layers
-};
-
-// K shares of one GEMM: at most kMaxShareK each (the exactness bound), and more when the tiles
-// alone would not give every SM a few CTAs (one CTA per SM), but at least kMinShareSlices slices
-// each (a CTA's pipeline fill and combine are paid once per share).
-constexpr int64_t kTargetCtas = 4 * 152;
+// Shares of K of one GEMM: at most kMaxSharesK slices each (the exactness bound), and more where that still
+// gives each SM at most one unit, but at least kMinShareSlices slices each (copper's hidden layers, 128 tiles:
+// one share, the layer finished in the GEMM, 26 us; two shares and the reduction 53 us).
+constexpr int kTargetUnits = 152;
 constexpr int kMinShareSlices = 6;
-int ksplit_for(int64_t Mp, int Np, int Kp) {
-  const int64_t tiles = (Mp / kTM) * (Np / kTN);
-  const int slices = Kp / kTK;
-  int want = (int)std::min<int64_t>((kTargetCtas + tiles - 1) / tiles, std::max(1, slices / kMinShareSlices));
-  want = std::max(want, (slices + kMaxShareSlices - 1) / kMaxShareSlices);
+int shares_for(int64_t tiles, int slices) {
+  int want = (int)std::min<int64_t>(std::max<int64_t>(1, kTargetUnits / tiles), std::max(1, slices / kMinShareSlices));
+  want = std::max(want, (slices + kMaxSharesK - 1) / kMaxSharesK);
   const int per = (slices + want - 1) / want;
-  return (slices + per - 1) / per;  // no empty share; per <= kMaxShareSlices
+  return (slices + per - 1) / per;  // no empty share
 }
 
-WorkMap work_map(const FitShape &s, int64_t nloc) {
-  Layer L[DP_MAX_LAYERS + 1];
+// The work buffer: the B planes of a batch of types, the A planes and row exponents of a chunk of row tiles,
+// the shares' partial results, and the [nloc][max hidden width] buffers between layers (four).  Types go
+// through in batches, and a batch's row tiles in chunks, of as many as the caller's buffer holds; the results
+// do not depend on either (every output is summed exactly and rounded once).
+constexpr int64_t kChunkRows = 16384;
+struct WorkMap {
+  int types, tiles;         // per batch, per chunk
+  size_t bstride;           // bytes of one type's B planes (the larger of the two directions)
+  size_t tanh_table, aplanes, aexp, part, buffers, total;
+};
+WorkMap work_map(const FitShape &s, int64_t nloc, int types, int tiles) {
+  Layer L[kMaxGemms];
   WorkMap m{};
-  m.bplanes = std::max(layout(s, true, L), layout(s, false, L));
+  m.types = types;
+  m.tiles = tiles;
+  m.bstride = std::max(layout(s, true, L), layout(s, false, L));
   int kmax = 1;
   for (int l = 0; l <= s.nlayer; ++l) kmax = std::max(kmax, s.w[l]);  // every GEMM's K is a layer width
-  m.Kpmax = (int)round_up(kmax, kTK);
-  int64_t maxn = 0;  // rows of the largest type
-  for (int t = 0; t < s.ntypes; ++t) maxn = std::max<int64_t>(maxn, s.start[t + 1] - s.start[t]);
-  m.Mp = round_up(std::min<int64_t>(std::max<int64_t>(maxn, 1), kChunkRows), kTM);
-  m.aplanes = m.bplanes;
-  m.aexp = m.aplanes + (size_t)round_up((int64_t)kS * m.Mp * m.Kpmax * 2, 256);
-  m.part = m.aexp + (size_t)round_up(m.Mp * 4, 256);
-  // shares x Mp x Np over the GEMMs: below kTargetCtas tiles plus the largest chunk's Mp x Np, or
-  // the exactness bound's shares at the largest chunk (a smaller chunk stays under both)
-  int Npmax = kTN;
-  for (int l = 0; l <= s.nlayer; ++l) Npmax = std::max(Npmax, (int)round_up(s.w[l], kTN));
-  int64_t part = kTargetCtas * kTM * kTN + m.Mp * Npmax;
-  for (int q = 0; q < gemm_count(s); ++q)
-    for (int dir = 0; dir < 2; ++dir) {
-      layout(s, dir == 0, L);
-      part = std::max<int64_t>(part, (int64_t)ksplit_for(m.Mp, L[q].Np, L[q].Kp) * m.Mp * L[q].Np);
+  m.tanh_table = m.bstride * types;
+  m.aplanes = m.tanh_table + (size_t)round_up((int64_t)kTanhEntries * (int64_t)sizeof(TanhEntry), 256);
+  m.aexp = m.aplanes + (size_t)round_up((int64_t)tiles * kSF * kPlaneAF * (round_up(kmax, kTK) / kTK), 256);
+  m.part = m.aexp + (size_t)round_up((int64_t)tiles * kTM * 4, 256);
+  int64_t units = 0;  // of any chunk of at most `tiles` row tiles, where K takes several shares
+  for (int dir = 0; dir < 2; ++dir) {
+    layout(s, dir == 0, L);
+    for (int q = 0; q < gemm_count(s); ++q) {
+      const int64_t nt = L[q].Np / kTNF, slices = L[q].Kp / kTK, least = (slices + kMaxSharesK - 1) / kMaxSharesK;
+      if (least > 1) units = std::max<int64_t>(units, least * tiles * nt);
+      units = std::max<int64_t>(units, kTargetUnits + std::min<int64_t>(tiles * nt, kTargetUnits));
     }
-  m.buffers = m.part + (size_t)round_up(part * 16, 256);
+  }
+  m.buffers = m.part + (size_t)(units * kTM * kTNF) * sizeof(longlong2);
+  m.total = m.buffers + (s.nlayer > 1 ? (size_t)4 * (size_t)nloc * (size_t)s.maxh * sizeof(double) : 0);
   return m;
 }
-
+int query_tiles(int64_t nloc) { return (int)(round_up(std::min<int64_t>(std::max<int64_t>(nloc, 1), kChunkRows), kTM) / kTM); }
 size_t work_bytes(const FitShape &s, int64_t nloc) {
-  const WorkMap m = work_map(s, nloc);
-  return m.buffers + (s.nlayer > 1 ? (size_t)4 * (size_t)nloc * (size_t)s.maxh * sizeof(double) : 0);
+  const int types = (int)std::min<int64_t>(DP_MAX_TYPES, std::max<int64_t>(nloc, 1));
+  return work_map(s, nloc, types, query_tiles(nloc) + types - 1).total;
 }
-
-
-// The weights of one layer as B planes: forward B[k][n] = W[k][n] (W is [K][N]), backward B[k][n] = W[n][k]
-int split_b(const double *W, const Layer &L, bool fwd, unsigned char *work, cudaStream_t st, const char *who) {
-  return fwd ? split_rows(W, 1, L.N, L.N, L.K, L.Np, L.Kp, kTN, work + L.planes, work + L.fexp, st, who)
-             : split_rows(W, L.K, 1, L.N, L.K, L.Np, L.Kp, kTN, work + L.planes, work + L.fexp, st, who);
-}
-
-// G over its rows in chunks of at most kChunkRows: each chunk's A rows split into planes, then the GEMM
-template <bool kFwd>
-int gemm(TcGemm G, const Layer &L, unsigned char *work, const WorkMap &m, cudaStream_t st, const char *who) {
-  G.planes = work + L.planes;
-  G.Fexp = reinterpret_cast<const int *>(work + L.fexp);
-  G.Np = L.Np;
-  G.Kp = L.Kp;
-  G.aplanes = work + m.aplanes;
-  G.Eexp = reinterpret_cast<const int *>(work + m.aexp);
-  G.part = reinterpret_cast<float4 *>(work + m.part);
-  const int64_t r_end = G.r0 + G.n;
-  for (int64_t r0 = G.r0; r0 < r_end; r0 += kChunkRows) {
-    TcGemm C = G;
-    C.r0 = r0;
-    C.n = std::min<int64_t>(kChunkRows, r_end - r0);
-    C.Mp = round_up(C.n, kTM);
-    int rc = split_rows(G.A + r0 * G.lda, G.lda, 1, C.n, G.K, C.Mp, L.Kp, kTM, work + m.aplanes, work + m.aexp, st, who);
-    if (rc) return rc;
-    const int ksplit = ksplit_for(C.Mp, L.Np, L.Kp);
-    C.slices_per_split = (L.Kp / kTK + ksplit - 1) / ksplit;
-    const dim3 grid((unsigned)(L.Np / kTN), (unsigned)(C.Mp / kTM), (unsigned)ksplit);
-    gemm_kernel<<<grid, kThreads, kSmemTotal, st>>>(C);
-    if ((rc = launch_status(who))) return rc;
-    epilogue_kernel<kFwd><<<(unsigned)std::min<int64_t>(C.n, 152 * 32), 256, 0, st>>>(C, ksplit);
-    if ((rc = launch_status(who))) return rc;
+// The smallest buffer taken: what the query gives, or, where that is less, what it gave when types went one by
+// one with nine 6-bit digits and four floats an output through memory -- callers may hold buffers of that size.
+size_t least_bytes(const FitShape &s, int64_t nloc) {
+  Layer L[kMaxGemms];
+  const int64_t Mp = (int64_t)query_tiles(nloc) * kTM;
+  int64_t kmax = 1, nmax = 48, planes = 0, part = 0;
+  for (int l = 0; l <= s.nlayer; ++l) {
+    kmax = std::max<int64_t>(kmax, s.w[l]);
+    nmax = std::max(nmax, round_up(s.w[l], 48));
   }
+  for (int dir = 0; dir < 2; ++dir) {
+    layout(s, dir == 0, L);
+    int64_t sum = 0;
+    for (int q = 0; q < gemm_count(s); ++q) {
+      const int64_t Np = round_up(L[q].N, 48), slices = L[q].Kp / kTK, tiles = Mp / kTM * (Np / 48);
+      sum += round_up(9 * Np * L[q].Kp * 2, 256) + round_up(Np * 4, 256);
+      const int64_t want = std::max(std::min((608 + tiles - 1) / tiles, std::max<int64_t>(1, slices / 6)), (slices + 111) / 112);
+      const int64_t per = (slices + want - 1) / want;
+      part = std::max(part, (slices + per - 1) / per * Mp * Np);
+    }
+    planes = std::max(planes, sum);
+  }
+  part = std::max(part, 608 * 128 * 48 + Mp * nmax);
+  const int64_t old = planes + round_up(9 * Mp * round_up(kmax, kTK) * 2, 256) + round_up(Mp * 4, 256) +
+                      round_up(part * 16, 256) + (s.nlayer > 1 ? 4 * nloc * s.maxh * (int64_t)sizeof(double) : 0);
+  return std::min(work_bytes(s, nloc), (size_t)old);
+}
+// The largest map that the buffer holds: fewer types a batch first, then fewer row tiles a chunk.
+bool fit_map(const FitShape &s, int64_t nloc, size_t nbytes, WorkMap *out) {
+  for (int types = s.ntypes; types >= 1; --types) {
+    *out = work_map(s, nloc, types, query_tiles(nloc) + types - 1);
+    if (out->total <= nbytes) return true;
+  }
+  for (int tiles = query_tiles(nloc); tiles >= 1; tiles /= 2) {
+    *out = work_map(s, nloc, 1, tiles);
+    if (out->total <= nbytes) return true;
+  }
+  return false;
+}
+int check_work(const FitShape &s, int64_t nloc, const void *work, size_t nbytes, const char *who, WorkMap *m) {
+  if (gemm_count(s) == 0) return DP_OK;
+  if (!work) return set_error(DP_ERR_NULL, "%s: work is NULL", who);
+  if (nbytes < least_bytes(s, nloc) || !fit_map(s, nloc, nbytes, m))
+    return set_error(DP_ERR_SHAPE, "%s: work holds %zu bytes, needs %zu", who, nbytes, work_bytes(s, nloc));
+  if (reinterpret_cast<uintptr_t>(work) % 256) return set_error(DP_ERR_SHAPE, "%s: work is not 256-byte aligned", who);
   return DP_OK;
 }
 
-int check_work(const FitShape &s, int64_t nloc, const void *work, size_t nbytes, const char *who) {
-  const size_t need = work_bytes(s, nloc);
-  if (need > 0 && !work) return set_error(DP_ERR_NULL, "%s: work is NULL", who);
-  if (nbytes < need) return set_error(DP_ERR_SHAPE, "%s: work holds %zu bytes, needs %zu", who, nbytes, need);
-  if (reinterpret_cast<uintptr_t>(work) % 256) return set_error(DP_ERR_SHAPE, "%s: work is not 256-byte aligned", who);
+// One direction over one batch of types: its weights split, then `layers` called for each chunk of row tiles.
+struct Run {
+  const FitShape &s;
+  const WorkMap &m;
+  bool fwd;
+  const double *params;  // the batch's first type's
+  unsigned char *work;
+  cudaStream_t st;
+  const char *who;
+  Tiles G;
+  Layer L[kMaxGemms];
+  int nsm;
+
+  int split_weights(int types) {
+    SplitB B{};
+    B.params = params;
+    B.pstride = s.P;
+    B.count = gemm_count(s);
+    layout(s, fwd, L);
+    for (int q = 0; q < B.count; ++q) {
+      B.K[q] = L[q].K;
+      B.N[q] = L[q].N;
+      B.woff[q] = s.woff[gemm_layer(s, fwd, q)];
+      B.planes[q] = L[q].planes;
+      B.fexp[q] = L[q].fexp;
+      B.group0[q + 1] = B.group0[q] + L[q].Np / 8;
+    }
+    B.bstride = m.bstride;
+    B.transposed = !fwd;
+    B.work = work;
+    B.tanh_table = fwd ? reinterpret_cast<TanhEntry *>(work + m.tanh_table) : nullptr;
+    if (B.count == 0) return DP_OK;
+    split_b_kernel<16><<<dim3((unsigned)(B.group0[B.count] + (fwd ? 1 : 0)), (unsigned)types), 512, 0, st>>>(B);
+    return launch_status(who);
+  }
+
+  // GEMM q over the chunk's row tiles, from A's source to the epilogue's outputs
+  int gemm(int q, const SplitA &src, const Epilogue &E, bool dz = false) {
+    SplitA A = src;
+    A.G = G;
+    A.K = L[q].K;
+    A.Kp = L[q].Kp;
+    A.planes = work + m.aplanes;
+    A.exps = reinterpret_cast<int *>(work + m.aexp);
+    A.pstride = s.P;
+    const unsigned blocks = (unsigned)(G.tiles * (kTM / 8));
+    if (dz)
+      split_a_kernel<4, true><<<blocks, 128, 0, st>>>(A);
+    else
+      split_a_kernel<4, false><<<blocks, 128, 0, st>>>(A);
+    int rc = launch_status(who);
+    if (rc) return rc;
+    Gemm C{};
+    C.G = G;
+    C.E = E;
+    C.E.N = L[q].N;
+    C.E.pstride = s.P;
+    C.E.tanh_table = reinterpret_cast<const TanhEntry *>(work + m.tanh_table);
+    C.nt = L[q].Np / kTNF;
+    C.ka = L[q].Kp / kTK;
+    C.ks = shares_for((int64_t)G.tiles * C.nt, C.ka);
+    C.per = (C.ka + C.ks - 1) / C.ks;
+    C.aplanes = A.planes;
+    C.Eexp = A.exps;
+    C.bplanes = work + L[q].planes;
+    C.Fexp = reinterpret_cast<const int *>(work + L[q].fexp);
+    C.bstride = m.bstride;
+    C.fstride = m.bstride / sizeof(int);
+    C.part = reinterpret_cast<longlong2 *>(work + m.part);
+    const unsigned grid = (unsigned)std::min<int64_t>(nsm, (int64_t)G.tiles * C.nt * C.ks);
+    if (fwd)
+      fit_gemm_kernel<true><<<grid, kThreadsF, kSmemF, st>>>(C);
+    else
+      fit_gemm_kernel<false><<<grid, kThreadsF, kSmemF, st>>>(C);
+    if ((rc = launch_status(who))) return rc;
+    if (C.ks > 1) {
+      const int64_t warps = (int64_t)G.tiles * 4 * ((C.E.N + 3) / 4);
+      const unsigned rb = (unsigned)((warps + 3) / 4);
+      if (fwd)
+        fit_reduce_kernel<true><<<rb, 128, 0, st>>>(C);
+      else
+        fit_reduce_kernel<false><<<rb, 128, 0, st>>>(C);
+      rc = launch_status(who);
+    }
+    return rc;
+  }
+};
+
+// Batches of types and chunks of row tiles; layers(run) runs a chunk, rows(run, row0, n) a batch's rows after.
+template <class Layers, class Rows>
+int over_batches(const FitShape &s, const WorkMap &m, bool fwd, const double *params, unsigned char *work,
+                 cudaStream_t st, const char *who, Layers &&layers, Rows &&rows) {
+  int dev = 0, nsm = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return set_error(DP_ERR_CUDA, "%s: %s", who, cudaGetErrorString(cudaGetLastError()));
+  const int step = std::max(1, m.types);
+  for (int t0 = 0; t0 < s.ntypes; t0 += step) {
+    const int types = std::min(step, s.ntypes - t0);
+    const int64_t r0 = s.start[t0], r1 = s.start[t0 + types];
+    if (r0 == r1) continue;
+    Run R{s, m, fwd, params + (size_t)t0 * s.P, work, st, who, Tiles{}, {}, std::max(1, nsm)};
+    R.G.ntypes = types;
+    for (int t = 0; t < types; ++t) {
+      R.G.start[t] = s.start[t0 + t];
+      R.G.t0[t + 1] = R.G.t0[t] + (int)((s.start[t0 + t + 1] - s.start[t0 + t] + kTM - 1) / kTM);
+    }
+    R.G.start[types] = r1;
+    int rc = R.split_weights(types);
+    const int all = R.G.t0[types];
+    for (int c = 0; c < all && !rc && gemm_count(s) > 0; c += m.tiles) {
+      R.G.tile0 = c;
+      R.G.tiles = std::min(m.tiles, all - c);
+      rc = layers(R);
+    }
+    if (!rc) rc = rows(R, r0, r1 - r0);
+    if (rc) return rc;
+  }
   return DP_OK;
 }
 
@@ -599,69 +664,45 @@ int fwd(const double *params, const int32_t *widths, int nlayer, int ntypes, con
   const int64_t nloc = s.start[ntypes];
   if (nloc == 0) return DP_OK;
   if (!params || !D || !E || (s.H > 0 && !act)) return set_error(DP_ERR_NULL, "%s: NULL array", who);
-  if ((rc = check_work(s, nloc, work, work_nbytes, who)) || (rc = set_smem(who))) return rc;
+  WorkMap m{};
+  if ((rc = check_work(s, nloc, work, work_nbytes, who, &m)) || (rc = set_smem(who))) return rc;
   const cudaStream_t st = (cudaStream_t)stream;
   unsigned char *wk = static_cast<unsigned char *>(work);
-  Layer L[DP_MAX_LAYERS + 1];
-  layout(s, true, L);
-  const WorkMap m = work_map(s, nloc);
   double *V[2] = {reinterpret_cast<double *>(wk + m.buffers), nullptr};
   V[1] = V[0] + (size_t)nloc * s.maxh;
-  for (int t = 0; t < ntypes; ++t) {
-    const int64_t n = s.start[t + 1] - s.start[t];
-    if (n == 0) continue;
-    const double *pt = params + (size_t)t * s.P;
-    for (int q = 0; q < gemm_count(s); ++q)  // this type's weights as digit planes (the previous type's are done with)
-      if ((rc = split_b(pt + s.woff[gemm_layer(s, true, q)], L[q], true, wk, st, who))) return rc;
-    const double *in = D;  // v_{l-1}: D, then the layer outputs with their skips
-    int64_t ldin = s.w[0];
-    for (int l = 1; l < nlayer; ++l) {
-      TcGemm G{};
-      G.r0 = s.start[t];
-      G.n = n;
-      G.K = s.w[l - 1];
-      G.N = s.w[l];
-      G.A = in;
-      G.lda = ldin;
-      G.skip = s.w[l] == s.w[l - 1];
-      G.bias = pt + s.woff[l] + (size_t)G.K * G.N;
-      G.act = act + s.aoff[l];
-      G.ldact = s.H;
-      G.V = V[(l - 1) & 1];
-      G.ldv = s.maxh;
-      if ((rc = gemm<true>(G, L[l - 1], wk, m, st, who))) return rc;
-      in = G.V;
-      ldin = G.ldv;
+  auto layers = [&](Run &R) {
+    for (int q = 0; q < gemm_count(s); ++q) {  // layer l = q + 1; input v_{l-1}: D, then the layers' outputs
+      const int l = q + 1;
+      SplitA A{};
+      A.X = l == 1 ? D : V[l & 1];
+      A.ldx = l == 1 ? s.w[0] : s.maxh;
+      Epilogue P{};
+      P.A = A.X;
+      P.lda = A.ldx;
+      P.bias = R.params + s.woff[l] + (size_t)s.w[l - 1] * s.w[l];
+      if (l < nlayer) {
+        P.skip = s.w[l] == s.w[l - 1];
+        P.act = act + s.aoff[l];
+        P.ldact = s.H;
+        P.V = V[(l - 1) & 1];
+        P.ldv = s.maxh;
+      } else {  // several outputs: E_i = v W_out + b_out
+        P.lin = true;
+        P.V = E;
+        P.ldv = s.nout;
+      }
+      if (int e = R.gemm(q, A, P)) return e;
     }
-    if (s.nout == 1) {  // output layer: E_i = v_{L-1} . wo + bo, a dot product per atom (FP64 pipe)
-      FitGemm<double> O{};
-      O.r0 = s.start[t];
-      O.n = n;
-      O.K = s.w[nlayer - 1];
-      O.N = 1;
-      O.src[0] = in;
-      O.lds[0] = ldin;
-      O.nsrc = 1;
-      O.wo = pt + s.woff[nlayer];
-      fit_out_kernel<double><<<(unsigned)((n + 3) / 4), 128, 0, st>>>(O, O.wo + O.K, E);
-      rc = launch_status(who);
-    } else {  // several outputs: E_i = v_{L-1} W_out + b_out, a GEMM on the tensor cores without tanh
-      TcGemm G{};
-      G.r0 = s.start[t];
-      G.n = n;
-      G.K = s.w[nlayer - 1];
-      G.N = s.nout;
-      G.A = in;
-      G.lda = ldin;
-      G.lin = true;
-      G.bias = pt + s.woff[nlayer] + (size_t)G.K * G.N;
-      G.V = E;
-      G.ldv = s.nout;
-      rc = gemm<true>(G, L[nlayer - 1], wk, m, st, who);
-    }
-    if (rc) return rc;
-  }
-  return DP_OK;
+    return (int)DP_OK;
+  };
+  auto rows = [&](Run &R, int64_t r0, int64_t n) {
+    if (s.nout > 1) return (int)DP_OK;
+    fit_energy_kernel<<<(unsigned)((n + 3) / 4), 128, 0, st>>>(R.G, r0, n, nlayer == 1 ? D : V[nlayer & 1],
+                                                               nlayer == 1 ? s.w[0] : s.maxh, s.w[nlayer - 1],
+                                                               R.params + s.woff[nlayer], s.P, E);
+    return launch_status(who);
+  };
+  return over_batches(s, m, true, params, wk, st, who, layers, rows);
 }
 
 int grad(const double *params, const int32_t *widths, int nlayer, int ntypes, const int64_t *type_start,
@@ -676,75 +717,61 @@ int grad(const double *params, const int32_t *widths, int nlayer, int ntypes, co
   if (nlayer == 1) return set_error(DP_ERR_UNSUPPORTED, "a fitting net without hidden layers has dD = wo");
   if (!params || !dD || (s.H > 0 && !act)) return set_error(DP_ERR_NULL, "%s: NULL array", who);
   if (s.nout > 1 && !g) return set_error(DP_ERR_NULL, "%s: g is NULL for a net of %d outputs", who, s.nout);
-  if ((rc = check_work(s, nloc, work, work_nbytes, who)) || (rc = set_smem(who))) return rc;
+  WorkMap m{};
+  if ((rc = check_work(s, nloc, work, work_nbytes, who, &m)) || (rc = set_smem(who))) return rc;
   const cudaStream_t st = (cudaStream_t)stream;
   unsigned char *wk = static_cast<unsigned char *>(work);
-  Layer L[DP_MAX_LAYERS + 1];
-  layout(s, false, L);
-  const WorkMap m = work_map(s, nloc);
   double *buf = reinterpret_cast<double *>(wk + m.buffers);
   const size_t bs = (size_t)nloc * s.maxh;
   double *Z[2] = {buf, buf + bs}, *Sb[2] = {buf + 2 * bs, buf + 3 * bs};
-  for (int t = 0; t < ntypes; ++t) {
-    const int64_t n = s.start[t + 1] - s.start[t];
-    if (n == 0) continue;
-    const double *pt = params + (size_t)t * s.P;
-    for (int q = 0; q < gemm_count(s); ++q)
-      if ((rc = split_b(pt + s.woff[gemm_layer(s, false, q)], L[q], false, wk, st, who))) return rc;
-    const double *wo = pt + s.woff[nlayer];
+  auto layers = [&](Run &R) {
+    const double *wo = R.params + s.woff[nlayer];
     const double *S = nullptr;  // dE/dv of the layer being walked; NULL: g wo (the last hidden layer)
     const int q0 = s.nout > 1 ? 1 : 0;  // the hidden layers' GEMMs come after g W_out^T
-    if (s.nout > 1) {  // dE/dv_{nlayer-1} = g W_out^T ([n][nout] x [nout][widths[nlayer-1]], tensor cores),
-                       // into Sb[1], which the walk below first writes after its first GEMM has read it
-      TcGemm G{};
-      G.r0 = s.start[t];
-      G.n = n;
-      G.K = s.nout;
-      G.N = s.w[nlayer - 1];
-      G.A = g;
-      G.lda = s.nout;
-      G.out = Sb[1];
-      G.ldo = s.maxh;
-      if ((rc = gemm<false>(G, L[0], wk, m, st, who))) return rc;
+    if (s.nout > 1) {  // dE/dv_{nlayer-1} = g W_out^T into Sb[1], which the walk below first writes after
+                       // its first GEMM has read it
+      SplitA A{};
+      A.X = g;
+      A.ldx = s.nout;
+      Epilogue P{};
+      P.out = Sb[1];
+      P.ldo = s.maxh;
+      if (int e = R.gemm(0, A, P)) return e;
       S = Sb[1];
-    }
-    {  // dz of the last hidden layer
-      const int K = s.w[nlayer - 1];
-      last_dz_kernel<<<(unsigned)std::min<int64_t>(n, 152 * 32), 256, 0, st>>>(s.start[t], n, K, g, wo, S, s.maxh,
-                                                                             act + s.aoff[nlayer - 1], s.H, Z[0],
-                                                                             s.maxh);
-      if ((rc = launch_status(who))) return rc;
     }
     int cur = 0;
     for (int l = nlayer - 1; l >= 1; --l) {
-      TcGemm G{};
-      G.r0 = s.start[t];
-      G.n = n;
-      G.K = s.w[l];
-      G.N = s.w[l - 1];
-      G.A = Z[cur];
-      G.lda = s.maxh;
-      G.skip = s.w[l] == s.w[l - 1];
-      G.S = S;
-      G.ldS = s.maxh;
-      G.g = g;
-      G.wo = wo;
+      SplitA A{};
+      const bool last = l == nlayer - 1;  // its dz is formed as it is split
+      A.X = last ? act + s.aoff[l] : Z[cur];
+      A.ldx = last ? s.H : s.maxh;
+      A.S = last ? S : nullptr;
+      A.ldS = s.maxh;
+      A.g = g;
+      A.wo = wo;
+      Epilogue P{};
+      P.skip = s.w[l] == s.w[l - 1];
+      P.S = S;
+      P.ldS = s.maxh;
+      P.g = g;
+      P.wo = wo;
       if (l > 1) {
-        G.T = act + s.aoff[l - 1];
-        G.ldT = s.H;
-        G.Snext = Sb[cur];
-        G.Z = Z[cur ^ 1];
-        G.ldz = s.maxh;
+        P.T = act + s.aoff[l - 1];
+        P.ldT = s.H;
+        P.Snext = Sb[cur];
+        P.Z = Z[cur ^ 1];
+        P.ldz = s.maxh;
       } else {
-        G.out = dD;
-        G.ldo = s.w[0];
+        P.out = dD;
+        P.ldo = s.w[0];
       }
-      if ((rc = gemm<false>(G, L[q0 + nlayer - 1 - l], wk, m, st, who))) return rc;
-      S = G.Snext;
+      if (int e = R.gemm(q0 + nlayer - 1 - l, A, P, last)) return e;
+      S = P.Snext;
       cur ^= 1;
     }
-  }
-  return DP_OK;
+    return (int)DP_OK;
+  };
+  return over_batches(s, m, false, params, wk, st, who, layers, [](Run &, int64_t, int64_t) { return (int)DP_OK; });
 }
 
 size_t work_bytes_api(const int32_t *widths, int nlayer, int64_t nloc) {
@@ -755,7 +782,7 @@ size_t work_bytes_api(const int32_t *widths, int nlayer, int64_t nloc) {
   if (fit_shape(widths, nlayer, 1, ts, &s, true)) return 0;
   return work_bytes(s, nloc);
 }
-}  // namespace tc
+}  // namespace tf
 
 
 // ------------------------------------------------- backward without allocation
@@ -846,17 +873,17 @@ int dp_fitting_grad_df64(const double *params, const int32_t *widths, int nlayer
 }
 
 size_t dp_fitting_tc_work_bytes(const int32_t *widths, int nlayer, int64_t nloc) {
-  return dpc::tc::work_bytes_api(widths, nlayer, nloc);
+  return dpc::tf::work_bytes_api(widths, nlayer, nloc);
 }
 int dp_fitting_fwd_tc_f64(const double *params, const int32_t *widths, int nlayer, int ntypes,
                           const int64_t *type_start, const double *D, double *E, double *act, void *work,
                           size_t work_bytes, void *stream) {
-  return dpc::tc::fwd(params, widths, nlayer, ntypes, type_start, D, E, act, work, work_bytes, stream);
+  return dpc::tf::fwd(params, widths, nlayer, ntypes, type_start, D, E, act, work, work_bytes, stream);
 }
 int dp_fitting_grad_tc_f64(const double *params, const int32_t *widths, int nlayer, int ntypes,
                            const int64_t *type_start, const double *act, const double *g, double *dD, void *work,
                            size_t work_bytes, void *stream) {
-  return dpc::tc::grad(params, widths, nlayer, ntypes, type_start, act, g, dD, work, work_bytes, stream);
+  return dpc::tf::grad(params, widths, nlayer, ntypes, type_start, act, g, dD, work, work_bytes, stream);
 }
 
 }  // extern "C"

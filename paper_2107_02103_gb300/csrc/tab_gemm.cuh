@@ -170,32 +170,6 @@ __device__ __forceinline__ Walk walk_of(const Params &P) {
   return Walk{(int)blockIdx.x, *P.nunits, (int)gridDim.x};
 }
 
-// A wait on an mbarrier phase, bounded in time (2 s on the global timer), that also gives up once another
-// role has.  The waiting thread is suspended between polls (try_wait's time hint), so that a waiting
-// thread takes no issue slots or shared-memory bandwidth from the copies and the MMAs.
-__device__ __forceinline__ uint64_t global_ns() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-__device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t parity, volatile int *abortf) {
-  const uint64_t t0 = global_ns();
-  for (;;) {
-    uint32_t done;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n selp.u32 %0, 1, 0, p;\n}"
-        : "=r"(done)
-        : "r"(bar), "r"(parity), "r"(20000u)
-        : "memory");
-    if (done) return true;
-    if (*abortf) return false;
-    if (global_ns() - t0 > 2000000000ull) {
-      *abortf = 1;
-      return false;
-    }
-  }
-}
-
 constexpr size_t kBarOff = (size_t)kStages * kStageBytes;  // full[4], empty[4], acc_full, tmem_free
 constexpr size_t kMiscOff = kBarOff + (2 * kStages + 2) * 8;  // tmem address, abort flag
 constexpr size_t kListOff = kMiscOff + 16;                     // producer's slice list
@@ -281,7 +255,7 @@ __global__ void __launch_bounds__(kThreadsP, 1) tgemm_kernel(const Params P) {
       __syncwarp();  // the list is reused by the next unit
     }
   } else if (warp == 1) {
-    // ---- MMA issuer: per slice the 45 digit products as 13 MMAs (see gemm_kernel), per unit a commit
+    // ---- MMA issuer: per slice the 45 digit products as 13 MMAs, per unit a commit
     // on acc_full once they have all completed
     if (lane == 0) {
       int g = 0, li = 0;
@@ -297,6 +271,9 @@ __global__ void __launch_bounds__(kThreadsP, 1) tgemm_kernel(const Params P) {
           const uint64_t a0 = smem_desc(sbase + st * kStageBytes), b0 = smem_desc(sbase + st * kStageBytes + kS * kPlaneA);
 #pragma unroll
           for (int s = 0; s < kS; ++s) {
+            // Digit s of A against B's digits t <= 8 - s: B's planes lie back to back in the stage (48 rows each,
+            // one row stride), so together they are one operand of 48 (9 - s) rows, and with the accumulator
+            // address moved by s diagonals the block of plane t lands on diagonal s + t; N <= 256.
             const uint64_t ad = a0 + (uint64_t)((s * kPlaneA) >> 4);
 #pragma unroll
             for (int t0 = 0; t0 < kS - s; t0 += kMaxPlanesPerMma) {

@@ -25,7 +25,6 @@ namespace dpc {
 namespace {
 namespace tb {
 using namespace tc;
-using tg::wait_or_abort;
 
 constexpr int kSB = Digits7x8::kNS;      // 7 digits of 8 bits
 constexpr int kTNB = 32;                 // columns per unit: 8 atoms x 4 (k)

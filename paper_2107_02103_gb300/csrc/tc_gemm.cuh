@@ -25,43 +25,22 @@ namespace {
 // Every (A_s B_t)_ij is a sum of integer products |A_s B_t| <= 1024; a diagonal
 // d has at most 9 of them, so its fp32 sum on the tensor cores is exact while
 // a block's share of K is at most kMaxShareK = 1792 (9 x 1792 x 1024 < 2^24).
-// The 9 diagonal sums of an output are combined on the FP32 pipe into four
-// floats (the two largest by an exact two-sum, the rest in float-float, whose
-// rounding lies ~2^-60 below the result); the caller's epilogue (Sum3 below)
-// adds the shares' floats into a three-float sum by exact two-sums and
-// converts it to f64 once -- or, in the tabulation's GEMMs, recombines the
-// diagonals exactly as one 128-bit integer and rounds that once (diag_s128,
-// s128_to_f64).  The tabulation's backward, whose K is M1 <= 144, splits into
-// seven 8-bit digits instead (Digits7x8; 28 products, diag7_s128).
-// What rounds is that conversion, the 53-bit truncation of the operands and
-// the dropped terms: |error| <~ K 2^-49 max_k|a_ik| max_k|b_kj|, against
-// K 2^-53 sum_k |a_ik b_kj| for an f64 dot product.  A row or column with an
-// inf or NaN gives NaN outputs.
+// The diagonal sums of an output are recombined exactly as one 128-bit integer
+// and rounded once (diag_s128, s128_to_f64).  What rounds is that conversion,
+// the 53-bit truncation of the operands and the dropped terms: |error| <~
+// K 2^-49 max_k|a_ik| max_k|b_kj|, against K 2^-53 sum_k |a_ik b_kj| for an f64
+// dot product.  A row or column with an inf or NaN gives NaN outputs.
 //
-// gemm_kernel: one CTA of 128 threads per 128 x 48 output tile and share of K,
-// one CTA per SM (its 9 diagonal accumulators take 432 of the SM's 512 TMEM
-// columns).  The digit planes of A (per chunk of rows) and B (per call) are
-// made by split_rows_kernel, once per element, as the shared-memory image of
-// each (tile, 16-deep K slice) block: the tcgen05 K-major layout without
-// swizzle (8-row x 16-byte core matrices).  Lane 0 of warp 0 moves a slice's
-// A and B blocks into one of four stages with two bulk async copies counted in
-// bytes on the stage's "full" mbarrier; lane 0 of warp 1 issues the slice's 45
-// digit products as 13 MMAs (M 128, K 16, fp16 in, fp32 accumulators in TMEM,
-// one 48-column block per diagonal; digit s of A against all of B's digits
-// t <= 8 - s at once, N up to 240) and commits them to the stage's "empty" mbarrier, which
-// the producer waits on before refilling the stage.  A last commit on a
-// barrier used once releases the four warps, which read their TMEM lane
-// quadrant (rows), combine the diagonals and write the share's result as four
-// floats; the caller's epilogue kernel sums the shares in a fixed order,
-// scales by 2^(E+F) and finishes the outputs.  Two optional modes serve sparse
-// operands (the tabulated embedding's interval moments): a per-tile list of the
-// K slices in use (the others are zero and are skipped; the shares then cut the
-// used slices, and a tile whose used slices fit one share can write its f64
-// outputs itself), and per-tile slice flags that skip unwanted output tiles,
-// whose wanted outputs are scattered to per-run slots instead of a dense array.
-// Every wait on an mbarrier is bounded; a wait that gives up makes the tile's
-// outputs NaN (the accumulators are not read) and counts one timeout in
-// g_wait_timeouts, which the host reads through dp_tc_wait_timeouts.
+// Three schemes of digits (Digits below) serve the kernels: nine of 6 bits, the
+// tabulation's forward (tab_gemm.cuh; K up to 1792 a share); eight of 7 bits,
+// the fitting net (fit_gemm.cuh; 36 products, K up to 512 a share); seven of 8
+// bits, the tabulation's backward, whose K is M1 <= 144 (tab_gemm_b8.cuh; 28
+// products).  This file has what they share: the splitting of operands into
+// digit planes (as the shared-memory image of each (tile, 16-deep K slice)
+// block, the tcgen05 K-major layout without swizzle), the recombination, the
+// descriptors and the bounded waits.  A wait on an mbarrier that gives up makes
+// the kernel's outputs NaN and counts one timeout in g_wait_timeouts, which the
+// host reads through dp_tc_wait_timeouts.
 namespace tc {
 constexpr int kS = 9;      // digits per operand element
 constexpr int kBits = 6;   // bits per digit
@@ -72,7 +51,6 @@ constexpr int kPad = kS * kBits - kFrac;  // a digit vector stands for 2^(E + kP
 constexpr int64_t kDigitBias = 32ll * ((1ll << 48) - 1ll) / 63ll;
 constexpr int kTM = 128, kTN = 48, kTK = 16;  // CTA tile; K per stage (one MMA)
 constexpr int kStages = 4;
-constexpr int kThreads = 128;  // one warp per TMEM lane quadrant; lane 0 of warps 0 and 1: producer and MMA issuer
 constexpr int kMaxShareK = 1792;
 constexpr int kNonFinite = 1 << 20;  // exponent of a row or column holding inf or NaN
 constexpr uint32_t kLBO = 128, kSBO = 256;  // core matrices: next along K at +128 B, next 8 rows at +256 B
@@ -80,13 +58,10 @@ constexpr int kPlaneA = kTM * kTK * 2, kPlaneB = kTN * kTK * 2;  // bytes of one
 constexpr int kStageBytes = kS * (kPlaneA + kPlaneB);
 constexpr uint32_t kTmemCols = 512;  // allocation (a power of two); kS * kTN = 432 used
 constexpr int kMaxShareSlices = kMaxShareK / kTK;
-constexpr size_t kSmemTail = (size_t)kStages * kStageBytes + (2 * kStages + 1) * 8 + 16;  // used-slice list
 constexpr int kScatKeys = kTM / 4 + 1, kScatAtoms = kTN / 4;  // scatter: keys (kq >= 4) and atoms of a tile
-constexpr size_t kSmemTotal = kSmemTail + (kMaxShareSlices + 2) * 4 + kScatKeys * kScatAtoms * 4;
 static_assert((size_t)kS * kMaxShareK * 32 * 32 < (1u << 24), "fp32 diagonal sums must stay exact");
 static_assert(kDigitBias < (1ll << 48) && kFrac == 53 && kS == 9, "top digit floor((f + bias) / 2^48) within [-32, 32]");
 static_assert(kMaxShareK % kTK == 0 && kS * kTN <= (int)kTmemCols, "shares and TMEM");
-static_assert(kSmemTotal <= 227 * 1024, "shared memory per block");
 
 __host__ __device__ constexpr int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 
@@ -110,8 +85,10 @@ struct Digits {
   static_assert(kBias < (1ll << (NB * (NS - 1))) && NB * (NS - 1) <= 56 && NB <= 9, "balanced top digit in range");
 };
 using Digits9x6 = Digits<9, 6>;
+using Digits8x7 = Digits<8, 7>;
 using Digits7x8 = Digits<7, 8>;
 static_assert(Digits9x6::kBias == kDigitBias && Digits9x6::kFrac == kFrac && Digits9x6::kPad == kPad, "the 9 x 6 scheme");
+static_assert(Digits8x7::kFrac == 55 && Digits8x7::kPad == 1 && Digits8x7::kBias < (1ll << 49), "the 8 x 7 scheme");
 static_assert(Digits7x8::kFrac == 55 && Digits7x8::kPad == 1 && Digits7x8::kBias < (1ll << 48), "the 7 x 8 scheme");
 
 // x 2^(kFrac - E) truncated toward zero (|x| < 2^E, so |.| < 2^kFrac), plus the scheme's bias (see digit_pairs)
@@ -146,7 +123,7 @@ __device__ __forceinline__ void digit_pairs(int64_t g0, int64_t g1, uint32_t (&h
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 // Rows of a matrix as digit planes, laid out as the shared-memory image of each (tile of RT rows,
-// 16-deep K slice) block that gemm_kernel copies in one piece: block (r / RT, k / 16) holds the kS
+// 16-deep K slice) block that the GEMM kernels copy in one piece: block (r / RT, k / 16) holds the kS
 // planes of those rows and columns, plane s at s RT 32 bytes, and in a plane the tcgen05 K-major
 // core matrices (8 rows x 8 k = 128 bytes; the second 8 k of the slice at +128 B, the next 8 rows
 // at +256 B).  Also the rows' exponents [rows_p].  Element (r, k) of the source is X[r ld_r + k ld_k];
@@ -199,104 +176,6 @@ __global__ void __launch_bounds__(128) split_rows_kernel(const double *__restric
   }
 }
 
-// f 2^e as a double, exactly, by moving fields (f finite; |e| < 900, so a normal result stays normal
-// and a float that is zero stays zero; float subnormals, which the sums do not produce, widen to 0)
-__device__ __forceinline__ double widen_pow2(float f, int e) {
-  const double d = dfl::widen(f);
-  const long long b = __double_as_longlong(d);
-  return (b & 0x7fffffffffffffffll) ? __longlong_as_double(b + ((long long)e << 52)) : d;
-}
-
-// The shares' results of one output summed in a fixed order: each share's four floats are added
-// into a three-float sum by exact two-sums on the FP32 pipe (only the last component rounds, ~2^-72
-// below the sum), which is converted to f64 once and scaled by the row and column powers of two.
-struct Sum3 {
-  float s0 = 0.f, s1 = 0.f, s2 = 0.f;
-  __device__ __forceinline__ void add(float x) {
-    float t = __fadd_rn(s0, x), z = __fsub_rn(t, s0);
-    const float e0 = __fadd_rn(__fsub_rn(s0, __fsub_rn(t, z)), __fsub_rn(x, z));
-    s0 = t;
-    t = __fadd_rn(s1, e0);
-    z = __fsub_rn(t, s1);
-    const float e1 = __fadd_rn(__fsub_rn(s1, __fsub_rn(t, z)), __fsub_rn(e0, z));
-    s1 = t;
-    s2 = __fadd_rn(s2, e1);
-  }
-  __device__ __forceinline__ void add(const float4 q) {
-    add(q.x);
-    add(q.y);
-    add(q.z);
-    add(q.w);
-  }
-  // the sum times 2^(E + F); NaN for a row or column with an inf or NaN, or a NaN share
-  __device__ __forceinline__ double value(int E, int F) const {
-    if (E >= kNonFinite || F >= kNonFinite || s0 != s0) return __longlong_as_double(0x7ff8000000000000ll);
-    const int e = E + F + 2 * kPad;
-    if (e > -900 && e < 900)  // the scaling moves exponent fields only (sums stay normal)
-      return __dadd_rn(__dadd_rn(widen_pow2(s0, e), widen_pow2(s1, e)), widen_pow2(s2, e));
-    return scalbn(__dadd_rn(__dadd_rn(dfl::widen(s0), dfl::widen(s1)), dfl::widen(s2)), e);
-  }
-};
-
-// One hidden-layer GEMM of a chunk of one type's atoms: rows r0 .. r0 + n - 1 of the plain
-// row-major A [*][K] (as digit planes) times B (digit planes), K cut into shares of at most
-// kMaxShareK (grid z); the shares' f64 results go to `part`, and epilogue_kernel sums them and
-// applies the layer's epilogue.
-struct TcGemm {
-  int64_t r0, n;  // output rows r0 .. r0 + n - 1; A's planes hold rows 0 .. n - 1 of this chunk
-  int K, N;
-  const double *A;  // the layer input itself (forward: its skip term)
-  int64_t lda;
-  const unsigned char *aplanes;  // A's blocks [Mp / kTM][Kp / kTK] of kS x kPlaneA bytes
-  const int *Eexp;          // [Mp]
-  int64_t Mp;
-  const unsigned char *planes;   // B's blocks [Np / kTN][Kp / kTK] of kS x kPlaneB bytes
-  const int *Fexp;
-  int Np, Kp;
-  float4 *part;             // [ksplit][Mp][Np]: each share's result (grid z) as four floats, see gemm_kernel
-  int slices_per_split;
-  // sparse operands (NULL for dense ones)
-  const unsigned char *kocc;  // [Np / kTN][Kp / kTK]: nonzero where the B tile has a nonzero entry in the
-                              // slice; share z of a tile then takes its used slices z S .. z S + S - 1
-                              // (S = slices_per_split), and a share past its last used slice writes nothing
-  const unsigned char *sflags;  // [Np / kTN][nsf]: flags of the K slices the atoms of a B tile use; output
-                                // tile (x, y) is wanted when one of slices 8 y .. 8 y + 7 is flagged
-  int nsf;
-  // scatter (with sflags): output (row kq key + q, column 4 a + k), q < 6 <= kq, key < nkeys, a < natoms,
-  // goes to scat[(a cap + slot) 24 + 6 k + q] when atom atom0 + a has type alpha (atype clamped into
-  // [0, ntypes)) and key is keys[(atom0 + a) cap + slot] for a slot < nslots[atom0 + a]; nothing is
-  // written to part
-  float4 *scat;
-  const short *keys;
-  const int *nslots;
-  const int32_t *atype;
-  int64_t natoms, atom0;
-  int nkeys, cap, alpha, ntypes, kq;
-  // direct output (with kocc): a tile whose used slices fit one share writes its outputs as f64,
-  // scaled by 2^(E_row + F_col), to tout[((atom0 + a) 4 + k) ldt + row] for row < ldt and the atoms
-  // a < natoms of type alpha, and nothing to part (the forward tabulation's T)
-  double *tout;
-  int ldt;
-  bool skip;
-  // forward
-  bool lin;  // an output layer of several outputs: V[row][col] = acc + bias, no tanh, act unused
-  const double *bias;
-  double *act;
-  int64_t ldact;
-  double *V;
-  int64_t ldv;
-  // backward
-  const double *S;  // NULL: S(row, col) = g_row wo_col
-  int64_t ldS;
-  const double *g, *wo;
-  const double *T;  // tanh outputs of the layer below (NULL: the last GEMM)
-  int64_t ldT;
-  double *Snext, *Z;
-  int64_t ldz;
-  double *out;
-  int64_t ldo;
-};
-
 // shared-memory descriptor of a K-major operand without swizzle (tcgen05): start address, the byte
 // offsets of the next core matrix along K (leading) and along the rows (stride), version 1
 __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr) {
@@ -323,36 +202,33 @@ int take_wait_timeouts(unsigned int *count) {
   return DP_OK;
 }
 
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-  uint32_t done = 0;
-  for (int it = 0; it < (1 << 24) && !done; ++it)
-    asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-                 : "=r"(done)
-                 : "r"(bar), "r"(parity)
-                 : "memory");
-  return done != 0;
+// A wait on an mbarrier phase, bounded in time (2 s on the global timer), that also gives up once another
+// role has.  The waiting thread is suspended between polls (try_wait's time hint), so that a waiting
+// thread takes no issue slots or shared-memory bandwidth from the copies and the MMAs.
+__device__ __forceinline__ uint64_t global_ns() {
+  uint64_t t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
 }
-
-// sum_d v[d][c] 64^-(d+2) (the diagonal sums of one output, read from TMEM) as four floats on the FP32
-// pipe: diagonals 2 and 3 (d = 0, 1) as an exact two-sum, 4 .. 10 in float-float, smallest first (its
-// rounding lies ~2^-60 below the sum).
-template <int W>
-__device__ __forceinline__ float4 diag_combine_w(const float (&v)[kS][W], int c) {
-  dfl::df64 lo(0.0f);
-#pragma unroll
-  for (int d = kS - 1; d >= 2; --d) {
-    const float x = v[d][c] * __uint_as_float((uint32_t)(127 - kBits * (d + 2)) << 23);  // exact: 64^-(d+2)
-    lo = lo + dfl::df64(x);
+__device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t parity, volatile int *abortf) {
+  const uint64_t t0 = global_ns();
+  for (;;) {
+    uint32_t done;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n selp.u32 %0, 1, 0, p;\n}"
+        : "=r"(done)
+        : "r"(bar), "r"(parity), "r"(20000u)
+        : "memory");
+    if (done) return true;
+    if (*abortf) return false;
+    if (global_ns() - t0 > 2000000000ull) {
+      *abortf = 1;
+      return false;
+    }
   }
-  const float a = v[0][c] * 0x1p-12f, b = v[1][c] * 0x1p-18f;  // exact
-  const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
-  const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-  return make_float4(s, e, lo.hi, lo.lo);
 }
-__device__ __forceinline__ float4 diag_combine(const float (&v)[kS][8], int c) { return diag_combine_w<8>(v, c); }
-__device__ __forceinline__ float4 diag_combine4(const float (&v)[kS][4], int c) { return diag_combine_w<4>(v, c); }
 
-// A float that holds an integer below 2^24 in magnitude (a diagonal sum) as an int: exact.
+// A float that holds an integer of at most 2^24 in magnitude (a diagonal sum) as an int: exact.
 __device__ __forceinline__ int exact_int(float f) { return __float2int_rz(f); }
 
 // The nine diagonal sums of one output (exact integers below 2^24; diagonal d weighs 64^-(d+2)) as one
@@ -364,18 +240,6 @@ __device__ __forceinline__ __int128 diag_int(const float (&v)[kS][W], int c) {
 #pragma unroll
   for (int d = 2; d < kS; ++d) lo += (long long)exact_int(v[d][c]) << (kBits * (kS - 1 - d));
   const long long hi = (long long)exact_int(v[0][c]) * 64 + exact_int(v[1][c]);  // diagonals 2, 3 over 2^42
-  return ((__int128)hi << 42) + lo;
-}
-
-// diag_int for diagonal sums below 2^22 in magnitude: each converts to int by one FP32 add of
-// 1.5 2^23 (the sum's integer lands in the low significand bits exactly) and one integer subtract.
-template <int W>
-__device__ __forceinline__ __int128 diag_int_small(const float (&v)[kS][W], int c) {
-  auto to_int = [](float f) { return __float_as_int(__fadd_rn(f, 12582912.0f)) - 0x4B400000; };
-  long long lo = 0;
-#pragma unroll
-  for (int d = 2; d < kS; ++d) lo += (long long)to_int(v[d][c]) << (kBits * (kS - 1 - d));
-  const long long hi = (long long)to_int(v[0][c]) * 64 + to_int(v[1][c]);
   return ((__int128)hi << 42) + lo;
 }
 
@@ -493,227 +357,6 @@ __device__ __noinline__ double output_value_rare(float v0, float v1, float v2, f
                                                  float v7, float v8, int E, int F) {
   const float v[kS][1] = {{v0}, {v1}, {v2}, {v3}, {v4}, {v5}, {v6}, {v7}, {v8}};
   return output_value(diag_int(v, 0), E, F);
-}
-
-__global__ void __launch_bounds__(kThreads, 1) gemm_kernel(const TcGemm P) {
-  extern __shared__ __align__(1024) unsigned char smem[];
-  uint64_t *full = reinterpret_cast<uint64_t *>(smem + kStages * kStageBytes);  // stage loaded
-  uint64_t *empty = full + kStages;                                               // stage's MMAs done
-  uint64_t *done = empty + kStages;                                               // every MMA done (one use)
-  uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(done + 1);
-  int *flags = reinterpret_cast<int *>(tmem_holder + 1);                          // producer / issuer ok
-  int *slist = reinterpret_cast<int *>(smem + kSmemTail);  // used slices, their count, the tile's total
-  int *stab = slist + kMaxShareSlices + 2;  // scatter: slot of (key, atom) of the tile, or -1; direct: atom wanted
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int64_t m0 = (int64_t)blockIdx.y * kTM;
-  const int n0 = blockIdx.x * kTN;
-  const int nslices = P.Kp / kTK;
-  const int i0 = blockIdx.z * P.slices_per_split;
-  if (P.sflags) {  // an output tile no atom of the B tile uses is skipped (uniform)
-    const unsigned char *f = P.sflags + (size_t)blockIdx.x * P.nsf;
-    const int lo = (int)(m0 / kTK), hi = min(P.nsf, (int)((m0 + kTM) / kTK));
-    bool any = false;
-    for (int x = lo; x < hi; ++x) any |= f[x] != 0;
-    if (!any) return;
-  }
-  if (P.scat) {  // the tile's slots: (key of the tile, atom) -> slot, or -1
-    int *nsa = slist;  // the slot count of each atom of the tile (0: not of type alpha); slist is free here
-    for (int x = tid; x < kScatKeys * kScatAtoms; x += kThreads) stab[x] = -1;
-    if (tid < kScatAtoms) {
-      const int64_t a = (int64_t)(n0 / 4) + tid, i = P.atom0 + a;
-      nsa[tid] = a < P.natoms && (!P.atype || clampi(P.atype[i], 0, P.ntypes - 1) == P.alpha) ? P.nslots[i] : 0;
-    }
-    __syncthreads();
-    const int key0 = (int)(m0 / P.kq);
-    for (int al = warp; al < kScatAtoms; al += kThreads / 32) {  // a warp per atom, its lanes over the slots
-      const short *keys = P.keys + (P.atom0 + n0 / 4 + al) * P.cap;
-      for (int slot = lane; slot < nsa[al]; slot += 32) {
-        const int key = keys[slot];
-        if (key >= key0 && key < key0 + kScatKeys) stab[(key - key0) * kScatAtoms + al] = slot;
-      }
-    }
-  }
-  if (P.tout)
-    for (int x = tid; x < kScatAtoms; x += kThreads) {
-      const int64_t a = (int64_t)(n0 / 4) + x;
-      stab[x] = a < P.natoms && (!P.atype || clampi(P.atype[P.atom0 + a], 0, P.ntypes - 1) == P.alpha);
-    }
-  int nsl = min(nslices - i0, P.slices_per_split);  // dense: > 0, no empty share
-  if (P.kocc) {
-    // this share's used slices, in order, by a ballot over the tile's flags
-    if (warp == 0) {
-      const unsigned char *occ = P.kocc + (size_t)blockIdx.x * nslices;
-      const int last = i0 + P.slices_per_split;
-      int rank = 0;
-      for (int b = 0; b < nslices && (rank < last || P.tout); b += 32) {  // uniform; direct output counts all
-        const int i = b + lane;
-        const bool used = i < nslices && occ[i] != 0;
-        const unsigned m = __ballot_sync(0xffffffffu, used);
-        const int r = rank + __popc(m & ((1u << lane) - 1u));
-        if (used && r >= i0 && r < last) slist[r - i0] = i;
-        rank += __popc(m);
-      }
-      if (lane == 0) {
-        slist[kMaxShareSlices] = min(max(rank - i0, 0), P.slices_per_split);
-        slist[kMaxShareSlices + 1] = rank;
-      }
-    }
-    __syncthreads();
-    nsl = slist[kMaxShareSlices];
-    if (nsl == 0) return;  // uniform: no slice left for this share
-  }
-  const bool direct = P.tout && P.kocc && slist[kMaxShareSlices + 1] <= P.slices_per_split;
-
-  if (tid == 0) {
-    for (int s = 0; s < kStages; ++s) {
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(full + s)));
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(empty + s)));
-    }
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(done)));
-    asm volatile("fence.mbarrier_init.release.cluster;");
-  }
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_holder)),
-                 "r"(kTmemCols));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;");
-  const uint32_t tmem = *tmem_holder;
-  const uint32_t sbase = smem_u32(smem);
-  bool ok = true;
-
-  if (warp == 0 && lane == 0) {
-    // producer: each slice's A and B blocks, one bulk copy each, counted in bytes on the stage's
-    // "full" barrier; a stage is reused once the MMAs that read it have completed ("empty")
-    for (int j = 0; j < nsl && ok; ++j) {
-      const int sl = P.kocc ? slist[j] : i0 + j;
-      const unsigned char *asrc = P.aplanes + ((size_t)blockIdx.y * nslices + sl) * (kS * kPlaneA);
-      const unsigned char *bsrc = P.planes + ((size_t)blockIdx.x * nslices + sl) * (kS * kPlaneB);
-      const int st = j % kStages;
-      if (j >= kStages) ok = mbar_wait(smem_u32(empty + st), (uint32_t)((j / kStages - 1) & 1));
-      if (!ok) break;
-      const uint32_t bar = smem_u32(full + st), dst = sbase + st * kStageBytes;
-      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"((uint32_t)kStageBytes)
-                   : "memory");
-      asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-                   "l"(asrc), "r"((uint32_t)(kS * kPlaneA)), "r"(bar)
-                   : "memory");
-      asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                       dst + kS * kPlaneA),
-                   "l"(bsrc), "r"((uint32_t)(kS * kPlaneB)), "r"(bar)
-                   : "memory");
-    }
-  } else if (warp == 1 && lane == 0) {
-    // MMA issuer: the 45 digit products of each slice once it has landed, then a commit that frees the stage
-    for (int i = 0; i < nsl && ok; ++i) {
-      const int st = i % kStages;
-      ok = mbar_wait(smem_u32(full + st), (uint32_t)((i / kStages) & 1));
-      if (!ok) break;
-      asm volatile("tcgen05.fence::after_thread_sync;");
-      const uint64_t a0 = smem_desc(sbase + st * kStageBytes), b0 = smem_desc(sbase + st * kStageBytes + kS * kPlaneA);
-      // Digit s of A against digits t = 0 .. kS-1-s of B in one MMA: B's planes lie back to back in
-      // the stage (48 rows each, one row stride), so together they are one operand of 48 (kS - s)
-      // rows, and with the accumulator address moved by s diagonals the block of plane t lands on
-      // diagonal s + t.  N is at most 256, so up to 5 planes (240 columns) per MMA: 13 MMAs per
-      // slice instead of 45, each reading its A tile once for up to 240 columns.
-#pragma unroll
-      for (int s = 0; s < kS; ++s) {
-        const uint64_t ad = a0 + (uint64_t)((s * kPlaneA) >> 4);  // start-address field, in 16-byte units
-#pragma unroll
-        for (int t0 = 0; t0 < kS - s; t0 += kMaxPlanesPerMma) {
-          const int np = min(kMaxPlanesPerMma, kS - s - t0);
-          const uint64_t bd = b0 + (uint64_t)((t0 * kPlaneB) >> 4);
-          const uint32_t idesc = kIdescNoN | ((uint32_t)((np * kTN) >> 3) << 17);
-          const uint32_t acc = (i > 0 || s > 0) ? 1u : 0u;  // digit 1 of A writes every diagonal first
-          asm volatile(
-              "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-              " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem + (uint32_t)((s + t0) * kTN)),
-              "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
-        }
-      }
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-          smem_u32(empty + st)));
-    }
-    // one more commit, on a barrier used once: it completes when every MMA issued above has (also
-    // after a wait that gave up, so that nobody waits on it in vain)
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(done)));
-  }
-  if (lane == 0 && warp < 2) flags[warp] = ok;
-  __syncwarp();
-  // The other warps wait here rather than on a stage barrier: a parity wait can only tell apart the
-  // current phase and the one before, and they would start it phases ahead of the MMAs.
-  __syncthreads();
-  ok = flags[0] && flags[1];
-  ok = mbar_wait(smem_u32(done), 0) && ok;
-  ok = __syncthreads_and(ok) != 0;  // one answer for the CTA: its accumulators are read only if every wait ended
-  if (!ok && tid == 0) atomicAdd(&g_wait_timeouts, 1u);
-  asm volatile("tcgen05.fence::after_thread_sync;");
-
-  // combine the diagonals of row 32 (warp % 4) + lane (the warp's TMEM lane quadrant), the warp's
-  // third of the columns, 8 at a time
-  const int rl = 32 * (warp & 3) + lane;
-  float4 *outp = P.scat ? nullptr : P.part + ((size_t)blockIdx.z * P.Mp + m0 + rl) * P.Np + n0;
-  const int key = P.scat ? (int)((m0 + rl) / P.kq) : 0, q = P.scat ? (int)(m0 + rl - (int64_t)key * P.kq) : 0;
-  const int key_l = P.scat ? key - (int)(m0 / P.kq) : 0;  // this thread's row's key, in the tile
-  const bool row_wanted = P.scat && q < 6 && key < P.nkeys;
-  const int Erow = direct && m0 + rl < P.ldt ? P.Eexp[m0 + rl] : 0;
-  const uint32_t trow = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
-  constexpr int kColsPerWarp = kTN / (kThreads / 128);
-  static_assert(kColsPerWarp % 8 == 0, "column share");
-#pragma unroll 1
-  for (int c0 = (warp >> 2) * kColsPerWarp; c0 < (warp >> 2) * kColsPerWarp + kColsPerWarp; c0 += 8) {
-    float v[kS][8];
-    if (ok) {  // uniform over the CTA
-#pragma unroll
-      for (int d = 0; d < kS; ++d)
-        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                     : "=f"(v[d][0]), "=f"(v[d][1]), "=f"(v[d][2]), "=f"(v[d][3]), "=f"(v[d][4]), "=f"(v[d][5]),
-                       "=f"(v[d][6]), "=f"(v[d][7])
-                     : "r"(trow + (uint32_t)(d * kTN + c0)));
-      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-    } else {
-#pragma unroll
-      for (int d = 0; d < kS; ++d)
-#pragma unroll
-        for (int c = 0; c < 8; ++c) v[d][c] = 0.0f;
-    }
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      // The scaling by 2^(E+F+2 kPad), and all f64 arithmetic, is left to the epilogue (or, for a direct
-      // output, to the two f64 adds below).
-      const float4 val = ok ? diag_combine(v, c) : make_float4(__int_as_float(0x7fc00000), 0.f, 0.f, 0.f);
-      if (direct) {
-        if (m0 + rl < P.ldt && stab[(c0 + c) >> 2]) {
-          Sum3 acc;
-          acc.add(val);
-          const int64_t a = (int64_t)(n0 >> 2) + ((c0 + c) >> 2);
-          P.tout[((P.atom0 + a) * 4 + ((c0 + c) & 3)) * P.ldt + m0 + rl] = acc.value(Erow, P.Fexp[n0 + c0 + c]);
-        }
-      } else if (outp) {
-        outp[c0 + c] = val;
-      } else if (row_wanted) {
-        const int al = (c0 + c) >> 2, k = (c0 + c) & 3;  // the tile's atom, its column k
-        const int slot = stab[key_l * kScatAtoms + al];
-        if (slot >= 0) P.scat[((size_t)((n0 >> 2) + al) * P.cap + slot) * 24 + 6 * k + q] = val;
-      }
-    }
-  }
-
-  asm volatile("tcgen05.fence::before_thread_sync;");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;");
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols));
-}
-
-int set_smem(const char *who) {
-  static std::atomic<bool> done{false};
-  if (done.load(std::memory_order_acquire)) return DP_OK;
-  const cudaError_t e = cudaFuncSetAttribute(gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemTotal);
-  if (e != cudaSuccess) return set_error(DP_ERR_CUDA, "%s: %s", who, cudaGetErrorString(e));
-  done.store(true, std::memory_order_release);
-  return DP_OK;
 }
 
 // split_rows_kernel with the row exponents found in the same kernel: one warp per group of 8 rows and
