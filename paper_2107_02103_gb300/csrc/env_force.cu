@@ -72,8 +72,8 @@ __global__ void __launch_bounds__(kEnvWarps * 32) env_mat_kernel(const EnvParams
                    dy = from_io<real>(P.coord[3 * (int64_t)j + 1] - yi),
                    dz = from_io<real>(P.coord[3 * (int64_t)j + 2] - zi);
         const real r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-        const real r = sqrt(r2);
-        const real inv_r = recip(r);
+        real r, inv_r;
+        radius(r2, r, inv_r);
         real sv, dsv;
         weight(P, r, inv_r, sv, dsv);
         const real a = sv * inv_r * P.inv_std_all;
@@ -121,8 +121,8 @@ __global__ void __launch_bounds__(kEnvWarps * 32) force_virial_kernel(const EnvP
       const real d[3] = {from_io<real>(P.coord[3 * (int64_t)j] - xi), from_io<real>(P.coord[3 * (int64_t)j + 1] - yi),
                          from_io<real>(P.coord[3 * (int64_t)j + 2] - zi)};
       const real r2 = fma(d[0], d[0], fma(d[1], d[1], d[2] * d[2]));
-      const real r = sqrt(r2);
-      const real inv_r = recip(r);
+      real r, inv_r;
+      radius(r2, r, inv_r);
       real sv, dsv;
       weight(P, r, inv_r, sv, dsv);
       const Vec4<real> gR = ld4r<real>(P.dRt + row * 4);

@@ -280,12 +280,13 @@ struct EnvRow {
   const int32_t *nlist;  // [nloc][nnei]: the neighbour's index into coord, or -1 (each segment's first)
   double rcs, rc, inv_width, mean, inv_std, inv_std_all;
   int kind;
+  bool unit;  // mean 0, std 1, std_all 1: the normalisation's operations change no bit and are left out
 };
 
 // Row (i, j) as dp_env_mat forms it, by the same operations: d = x_j - x_i, r, 1/r, s(r) and ds/dr, the
 // table input and R~[0] sh = (s - mean)/std, and R~[1 .. 3] = s d / (r std_all).
 struct EnvVals {
-  double d[3], inv_r, sv, dsv, r4[4];
+  double d[3], inv_r, sv, dsv, a, r4[4];  // a = s / r
 };
 __device__ __forceinline__ EnvVals env_vals(const EnvRow &E, int64_t i, int j) {
   EnvVals v;
@@ -294,11 +295,12 @@ __device__ __forceinline__ EnvVals env_vals(const EnvRow &E, int64_t i, int j) {
   v.d[1] = E.coord[3 * (int64_t)j + 1] - yi;
   v.d[2] = E.coord[3 * (int64_t)j + 2] - zi;
   const double r2 = fma(v.d[0], v.d[0], fma(v.d[1], v.d[1], v.d[2] * v.d[2]));
-  const double r = sqrt(r2);
-  v.inv_r = recip(r);
+  double r;
+  radius(r2, r, v.inv_r);
   weight(E, r, v.inv_r, v.sv, v.dsv);
-  const double a = v.sv * v.inv_r * E.inv_std_all;
-  v.r4[0] = (v.sv - E.mean) * E.inv_std;
+  v.a = v.sv * v.inv_r;
+  const double a = E.unit ? v.a : v.a * E.inv_std_all;
+  v.r4[0] = E.unit ? v.sv : (v.sv - E.mean) * E.inv_std;
   v.r4[1] = a * v.d[0];
   v.r4[2] = a * v.d[1];
   v.r4[3] = a * v.d[2];
@@ -1009,7 +1011,7 @@ __global__ void __launch_bounds__(32 * kRowsWarps, 7) rows_kernel(const RowsPara
 // rows_kernel does, and from them, in registers, the row's force contribution g = dE/d(x_j - x_i) by
 // dp_force_virial's arithmetic: F_i += g, F_j -= g (atomics), virial -= d (x) g; s, R~, ds and dR~ never
 // reach memory.  The per-atom sums are reduced over the warp and added once.
-__global__ void __launch_bounds__(32 * kRowsWarps) rows_force_kernel(const RowsParams P) {
+__global__ void __launch_bounds__(32 * kRowsWarps, 4) rows_force_kernel(const RowsParams P) {
   __shared__ int nvbw[kRowsWarps][DP_MAX_TYPES];
   extern __shared__ __align__(16) short smapw[];  // [kRowsWarps][map_stride(nkeys)]
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1029,9 +1031,9 @@ __global__ void __launch_bounds__(32 * kRowsWarps) rows_force_kernel(const RowsP
   const int2 *kexp = P.kexp + (size_t)(P.atype ? clampi(__ldg(P.atype + i), 0, P.ntypes - 1) : 0) * P.nkeys;
   bool plain;
   const int4 ge = atom_exps(P, a, plain);
-  double f[3] = {0.0, 0.0, 0.0}, w[9];
+  double sum[16];  // the force on atom i, the virial (nine), padding
 #pragma unroll
-  for (int x = 0; x < 9; ++x) w[x] = 0.0;
+  for (int x = 0; x < 16; ++x) sum[x] = 0.0;
   for (int v = lane; v < nv; v += 32) {
     int b;
     const int row = valid_row(v, nvb, P.sel, P.ntypes, b);
@@ -1043,47 +1045,47 @@ __global__ void __launch_bounds__(32 * kRowsWarps) rows_force_kernel(const RowsP
     const int key = b * P.g.nint + l;
     const fx::Fix *slot = dWa + (size_t)smap[key] * 24;
     const RowPoly R = row_poly(__ldg(kexp + key), plain, t, l < P.g.n0 ? P.e0 : P.e1);
-    double d4[4], ds = 0.0;
+    // dE/ds = sum_k R~[k] P_k', R~[1 .. 3] = ce d
+    double d4[4], dp[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      double dp;
-      row_component(R, slot, k, k == 0 ? ge.x : k == 1 ? ge.y : k == 2 ? ge.z : ge.w, d4[k], dp);
-      ds = fma(ev.r4[k], dp, ds);
-    }
+    for (int k = 0; k < 4; ++k)
+      row_component(R, slot, k, k == 0 ? ge.x : k == 1 ? ge.y : k == 2 ? ge.z : ge.w, d4[k], dp[k]);
+    double ce = ev.a;
+    if (!P.env.unit) ce *= P.env.inv_std_all;  // uniform
+    double ds = fma(dp[1], ev.d[0], fma(dp[2], ev.d[1], dp[3] * ev.d[2]));
+    ds = fma(ce, ds, ev.r4[0] * dp[0]);
     ds = clamped ? 0.0 : ds;
     // as dp_force_virial: the s column feeds both the table input and R~[0]
     const double g0 = ds + d4[0];
     const double p = fma(d4[1], ev.d[0], fma(d4[2], ev.d[1], d4[3] * ev.d[2]));
-    const double cd = fma(g0 * ev.dsv, ev.inv_r * P.env.inv_std,
-                          (ev.dsv - ev.sv * ev.inv_r) * ev.inv_r * ev.inv_r * p * P.env.inv_std_all);
-    const double ce = ev.sv * ev.inv_r * P.env.inv_std_all;
+    double hs = g0 * ev.dsv, hp = (ev.dsv - ev.a) * ev.inv_r;
+    if (!P.env.unit) hs *= P.env.inv_std, hp *= P.env.inv_std_all;
+    const double cd = fma(hp, p, hs) * ev.inv_r;
     const double g[3] = {fma(cd, ev.d[0], ce * d4[1]), fma(cd, ev.d[1], ce * d4[2]), fma(cd, ev.d[2], ce * d4[3])};
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      f[c] += g[c];
+      sum[c] += g[c];
       atomicAdd(P.F + 3 * (int64_t)j + c, -g[c]);
     }
 #pragma unroll
     for (int x = 0; x < 3; ++x)
 #pragma unroll
-      for (int y = 0; y < 3; ++y) w[3 * x + y] = fma(-ev.d[x], g[y], w[3 * x + y]);
+      for (int y = 0; y < 3; ++y) sum[3 + 3 * x + y] = fma(-ev.d[x], g[y], sum[3 + 3 * x + y]);
   }
+  // the twelve sums over the warp, halving the values a lane holds at each step (16 adds; 60 summed apart):
+  // lane 16 a + 8 b + 4 c + 2 d holds value 8 a + 4 b + 2 c + d
 #pragma unroll
-  for (int c = 0; c < 3; ++c)
+  for (int h = 8; h >= 1; h >>= 1) {
+    const bool up = lane & (2 * h);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) f[c] += __shfl_xor_sync(0xffffffffu, f[c], o);
-#pragma unroll
-  for (int x = 0; x < 9; ++x)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) w[x] += __shfl_xor_sync(0xffffffffu, w[x], o);
-  if (lane < 3) atomicAdd(P.F + 3 * i + lane, lane == 0 ? f[0] : lane == 1 ? f[1] : f[2]);
-  if (lane < 9) {
-    double vv = w[0];
-#pragma unroll
-    for (int x = 1; x < 9; ++x)
-      if (lane == x) vv = w[x];
-    atomicAdd(P.virial + lane, vv);
+    for (int x = 0; x < h; ++x) {
+      const double send = up ? sum[x] : sum[x + h], keep = up ? sum[x + h] : sum[x];
+      sum[x] = keep + __shfl_xor_sync(0xffffffffu, send, 2 * h);
+    }
   }
+  sum[0] += __shfl_xor_sync(0xffffffffu, sum[0], 1);
+  const int at = lane >> 1;
+  if ((lane & 1) == 0 && at < 12) atomicAdd(at < 3 ? P.F + 3 * i + at : P.virial + at - 3, sum[0]);
 }
 
 int check_work(const Layout &L, const void *work, size_t nbytes, const char *who) {
@@ -1534,6 +1536,7 @@ EnvRow env_row(const dp_env_info *e, const double *coord, const int32_t *nlist) 
   E.inv_std = 1.0 / e->std;
   E.inv_std_all = 1.0 / e->std_all;
   E.kind = e->kind;
+  E.unit = e->mean == 0.0 && e->std == 1.0 && e->std_all == 1.0;
   return E;
 }
 

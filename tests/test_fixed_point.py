@@ -110,3 +110,52 @@ def test_bounds_hold():
         assert sum(q * a[q] for q in range(1, 6)) < Fr(2) ** slope
         assert a[0] <= Fr(2) ** (value - 1) and slope < value
         assert math.log2(float(sum(q * a[q] for q in range(1, 6)))) > slope - 2
+
+
+def _constants():
+    """The switch's coefficient tables, from the source."""
+    import os
+    import re
+    src = open(os.path.join(os.path.dirname(__file__), "..", "paper_2107_02103_gb300", "csrc", "env_row.cuh")).read()
+    return [[int(x) for x in re.search(rf"{n}\[12\] = {{(.*?)}}", src, re.S).group(1).split(",")] for n in ("kSin", "kCos")]
+
+
+@pytest.mark.parametrize("kind", [0, 1])
+def test_switch(kind):
+    """The weighting function and its derivative in fixed point against 60-digit arithmetic over u in [0, 1]: within
+    2^-55 and 2^-53 (eleven Horner steps each off by at most two units of 2^-60, over 4; their last powers' sum)."""
+    from decimal import Decimal as Dc, getcontext
+    getcontext().prec = 60
+    pi = Dc("3.14159265358979323846264338327950288419716939937510582097494459")
+
+    def series(x, first):  # sin (first = 1) or cos (first = 0) of x
+        term = x if first else Dc(1)
+        total, n = term, first
+        while abs(term) > Dc(10) ** -50:
+            term *= -x * x / ((n + 1) * (n + 2))
+            total += term
+            n += 2
+        return total
+
+    ksin, kcos = _constants()
+    rng = np.random.default_rng(2)
+    for uf in [0.0, 2.0 ** -60, 1e-9, 0.5, 1 - 2.0 ** -53, 1.0, *rng.random(200)]:
+        u = int(Fr(uf) * 2**60)
+        U = Dc(u) / Dc(2) ** 60
+        if kind == 1:
+            u2 = mul(u, u, L)
+            u3 = mul(u2, u, L)
+            q8 = (2 * u - (u >> 3)) - (u2 - (u2 >> 2)) - (5 << 58)
+            w, dw = (1 << 60) + 8 * mul(u3, q8, L), -(15 * mul(u2 - u, u2 - u, L) >> 1)
+            ew, ed = U**3 * (-6 * U * U + 15 * U - 10) + 1, -30 * U * U * (U - 1) ** 2
+        else:
+            x = u - (1 << 59)
+            z = mul(x, x, L)
+            p, q = ksin[11], kcos[11]
+            for k in range(10, -1, -1):
+                p, q = ksin[k] + mul(p, z, L), kcos[k] + mul(q, z, L)
+                assert max(abs(p), abs(q)) < 1 << 61
+            w, dw = (1 << 59) - 2 * mul(p, x, L), -q
+            ew, ed = series(pi * U, 0) / 2 + Dc("0.5"), -(pi / 2) * series(pi * U, 1)
+        assert abs(w) < 1 << 62 and abs(Dc(w) / Dc(2) ** 60 - ew) < Dc(2) ** -55
+        assert abs(Dc(dw) / Dc(2) ** 58 - ed) < Dc(2) ** -53
