@@ -1,6 +1,8 @@
 // Persistent exact-f64 GEMM for the tensor-core tabulation's backward where the channels fit one
 // share of the 7 x 8-bit digit scheme (M1 <= 144): dW = dT C'^T over the used 128-row output tiles of
 // every 8-atom tile, each output scattered to its atom's run slot (the rows kernel reads it there).
+// One launch takes the units of every centre type: the list of (8-atom tile, 128-row tile, type) is
+// built on the device, and a launch per type would leave its last wave of 152 CTAs part empty each time.
 //
 // Against the forward's kernel (tab_gemm.cuh) two things change.  The operands are split into seven
 // 8-bit balanced digits (Digits7x8: 28 digit products per output instead of 45, seven MMAs per 16-deep
@@ -10,12 +12,16 @@
 // the tensor core waiting for every epilogue.  Roles: warp 0 moves each slice's A and B blocks into a
 // ring of five stages (bulk copies counted on the stage's "full" barrier), lane 0 of warp 1 issues the
 // MMAs into accumulator buffer (unit & 1) once the epilogue has released it ("tmem_free") and commits
-// "acc_full" for that buffer, warp 10 builds each unit's slot table (the run slot of every (interval,
-// atom) of the unit, from the atoms' slot keys) and column exponents into table buffer (unit & 1)
-// ahead of the epilogue ("tbl_full", released by "tbl_empty"), and eight epilogue warps (two per TMEM
-// lane quadrant, 16 columns each) finish the outputs.  (Measured: with the epilogue warps building the
-// tables themselves, the tensor core waited for the epilogue about 40 % of the time.)  Every wait is bounded; a wait that gives up stops the CTA's copies and MMAs,
-// the rows kernel's results are then NaN (bad) and one timeout is counted (dp_tc_wait_timeouts).
+// "acc_full" for that buffer, eight epilogue warps (two per TMEM lane quadrant, 16 columns each) finish
+// the outputs, and warps 10 and 11 each build every second unit's slot table (the run slot of every
+// (interval, atom) of the unit, from the atoms' slot keys) and column exponents into their table buffer
+// ahead of the epilogue ("tbl_full", released by "tbl_empty").  A table is a chain of dependent loads
+// (unit, atom types, slot counts, keys), longer than a unit's MMAs: with one table warp the kernel took
+// 300 us on the 16,384-atom H2O step and 47 us on the 4,096-atom Cu step, with two 234 and 44; four and
+// six give no more (239 and 45), and with the tables left out it is 218 and 37.  Copies, MMAs and the
+// epilogue's arithmetic are each hidden (leaving one out gains 1 to 10 %).  Every wait is bounded; a wait
+// that gives up stops the CTA's copies and MMAs, the rows kernel's results are then NaN (bad) and one
+// timeout is counted (dp_tc_wait_timeouts).
 #pragma once
 
 #include "tab_gemm.cuh"
@@ -35,7 +41,8 @@ constexpr int kPlaneBB = kTNB * kTK * 2; // of a 32-row B block: 1 KB
 constexpr int kStageBytesB = kSB * (kPlaneAB + kPlaneBB);
 constexpr int kMaxKB = 144;              // K (channels, padded to 16) of one exact share
 constexpr int kEpiWarpsB = 8;
-constexpr int kThreadsB = 32 * (3 + kEpiWarpsB);  // producer, MMA issuer, epilogue, table warp
+constexpr int kTableWarps = 2;           // and table buffers: unit li is warp li % kTableWarps's
+constexpr int kThreadsB = 32 * (2 + kEpiWarpsB + kTableWarps);  // producer, MMA issuer, epilogue, table warps
 constexpr int kTableWarp = 2 + kEpiWarpsB;
 constexpr int kEpiColsB = kTNB / 2;      // columns per epilogue warp
 constexpr uint32_t kBufColsB = 256;      // TMEM columns per accumulator buffer (7 x 32 used)
@@ -45,14 +52,15 @@ static_assert(kSB * kTNB <= (int)kBufColsB && 2 * kBufColsB <= kTmemCols, "two a
 static_assert(kStageBytesB % 1024 == 0, "stages stay 1024-byte aligned");
 
 struct Params {
-  const unsigned char *aplanes;  // A = C'_alpha: blocks [Mp / 128][ka] of kSB x kPlaneAB bytes
-  const int *Eexp;               // [Mp] row exponents
+  const unsigned char *aplanes;  // A = C'_t of type t at t astride: blocks [Mp / 128][ka] of kSB x kPlaneAB bytes
+  size_t astride;
+  const int *Eexp;               // [ntypes][Mp] row exponents
   int ka;                        // K slices: the channels padded to 16, / 16 (<= 9)
   const unsigned char *bplanes;  // B = dT^T of the chunk: blocks [ntiles][ka] of kSB x kPlaneBB bytes
   const int *Fexp;               // [32 ntiles] column exponents
   int64_t Mp;
   fx::Fix *scat;      // [natoms][cap][24]: the wanted outputs, per run slot, as fixed points (tg::key_exps)
-  const int2 *kexp;   // [nkeys] of the launch's centre type
+  const int2 *kexp;   // [ntypes][nkeys]
   const int *gexp;    // [32 ntiles]
   int n0, nint, e0, e1;  // fine intervals, intervals; binary places of u in the two segments
   int *bad;              // set when a CTA gave up a wait: the rows kernel's results are then NaN
@@ -61,19 +69,32 @@ struct Params {
   int cap, nkeys, kq;
   const int32_t *atype;
   int64_t natoms, atom0;
-  int alpha, ntypes;
-  const int *units;   // the launch's units (tile | mt << 16), in any order
+  int ntypes;
+  const int *units;   // the launch's units, every centre type's, in any order (unit_code)
   const int *nunits;  // their count (device)
 };
 
-__host__ __device__ constexpr int unit_code(int tile, int mt) { return tile | (mt << 16); }
+// A unit packed into an int: tile (< 2^16), 128-row tile of A (< 2^8), centre type.
+__host__ __device__ constexpr int unit_code(int tile, int mt, int type) { return tile | mt << 16 | type << 24; }
+struct Unit {
+  int tile, mt, type;
+};
+__device__ __forceinline__ Unit unit_of(int c) { return Unit{c & 0xffff, (c >> 16) & 0xff, c >> 24}; }
+
+// (T 2^32 + A) / 2^sh as the rows kernel's limbs, |.| < 2^61: each part rounded (halves up), which is exact
+// for T up to sh = 32.
+__device__ __forceinline__ fx::Fix fix_of(long long T, long long A, int sh) {
+  const int a = clampi(sh, 1, 62), r = clampi(sh - 32, 0, 62), l = clampi(32 - sh, 0, 31);
+  const long long hi = sh <= 32 ? T << l : (T + (1ll << max(r - 1, 0))) >> r;
+  return fx::limbs<tg::kGradLimb>(hi + ((A + (1ll << (a - 1))) >> a));
+}
 
 // full[5], empty[5], acc_full[2], tmem_free[2], tbl_full[2], tbl_empty[2]
 constexpr size_t kBarOffB = (size_t)kStagesB * kStageBytesB;
-constexpr size_t kMiscOffB = kBarOffB + (2 * kStagesB + 8) * 8;   // tmem address, abort flag
-constexpr size_t kStabOffB = kMiscOffB + 16;                      // two tables: slots, exponents; flags
+constexpr size_t kMiscOffB = kBarOffB + (2 * kStagesB + 4 + 2 * kTableWarps) * 8;  // tmem address, abort flag
+constexpr size_t kStabOffB = kMiscOffB + 16;                      // the tables: slots, exponents; flags
 constexpr int kTableInts = kScatKeysB * kAtomsB + kTNB;          // one table buffer
-constexpr size_t kSmemB = kStabOffB + (2 * kTableInts + 4) * 4;
+constexpr size_t kSmemB = kStabOffB + (kTableWarps * kTableInts + 4) * 4;
 static_assert(kSmemB <= 227 * 1024, "shared memory per block");
 
 __global__ void __launch_bounds__(kThreadsB, 1) bgemm_kernel(const Params P) {
@@ -83,12 +104,12 @@ __global__ void __launch_bounds__(kThreadsB, 1) bgemm_kernel(const Params P) {
   uint64_t *acc_full = empty + kStagesB;
   uint64_t *tmem_free = acc_full + 2;
   uint64_t *tbl_full = tmem_free + 2;
-  uint64_t *tbl_empty = tbl_full + 2;
+  uint64_t *tbl_empty = tbl_full + kTableWarps;
   uint32_t *tmem_holder = reinterpret_cast<uint32_t *>(smem + kMiscOffB);
   volatile int *abortf = reinterpret_cast<volatile int *>(smem + kMiscOffB + 4);
   // table buffer b: (key of the unit, atom) -> slot or -1, then G - F of the unit's 32 columns
   int *tables = reinterpret_cast<int *>(smem + kStabOffB);
-  int *uflag = tables + 2 * kTableInts;  // [0]: the unit's accumulators and table are ready
+  int *uflag = tables + kTableWarps * kTableInts;  // [0]: the unit's accumulators and table are ready
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int nunits = *P.nunits;
 
@@ -100,6 +121,8 @@ __global__ void __launch_bounds__(kThreadsB, 1) bgemm_kernel(const Params P) {
     for (int b = 0; b < 2; ++b) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(acc_full + b)));
       asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(tmem_free + b)), "r"(kEpiWarpsB));
+    }
+    for (int b = 0; b < kTableWarps; ++b) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(tbl_full + b)));
       asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(tbl_empty + b)), "r"(kEpiWarpsB));
     }
@@ -123,13 +146,13 @@ __global__ void __launch_bounds__(kThreadsB, 1) bgemm_kernel(const Params P) {
       int g = 0;  // slices loaded so far by this CTA
       bool ok = true;
       for (int u = blockIdx.x; u < nunits && ok; u += gridDim.x) {
-        const int c = P.units[u], tile = c & 0xffff, mt = c >> 16;
+        const Unit U = unit_of(P.units[u]);
         for (int j = 0; j < P.ka; ++j, ++g) {
           const int st = g % kStagesB;
           if (g >= kStagesB && !(ok = wait_or_abort(smem_u32(empty + st), (uint32_t)((g / kStagesB - 1) & 1), abortf)))
             break;
-          const unsigned char *asrc = P.aplanes + ((size_t)mt * P.ka + j) * (kSB * kPlaneAB);
-          const unsigned char *bsrc = P.bplanes + ((size_t)tile * P.ka + j) * (kSB * kPlaneBB);
+          const unsigned char *asrc = P.aplanes + U.type * P.astride + ((size_t)U.mt * P.ka + j) * (kSB * kPlaneAB);
+          const unsigned char *bsrc = P.bplanes + ((size_t)U.tile * P.ka + j) * (kSB * kPlaneBB);
           const uint32_t bar = smem_u32(full + st), dst = sbase + st * kStageBytesB;
           asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"((uint32_t)kStageBytesB)
                        : "memory");
@@ -182,15 +205,17 @@ __global__ void __launch_bounds__(kThreadsB, 1) bgemm_kernel(const Params P) {
       }
     }
     __syncwarp();
-  } else if (warp == kTableWarp) {
-    // ---- table warp: each unit's slot table and column exponents into table buffer (unit & 1)
-    int li = 0;
-    for (int u = blockIdx.x; u < nunits; u += gridDim.x) {
-      const int c = P.units[u], tile = c & 0xffff, mt = c >> 16;
-      const int b = li & 1;
-      if (li >= 2) {
+  } else if (warp >= kTableWarp) {
+    // ---- table warps: each unit's slot table and column exponents, ahead of the epilogue.  Unit li of the
+    // CTA's walk is warp li % kTableWarps's, in that table buffer.
+    const int b = warp - kTableWarp;
+    int nb = 0;  // tables built in this buffer
+    for (int u = blockIdx.x + b * gridDim.x; u < nunits; u += kTableWarps * gridDim.x) {
+      const Unit U = unit_of(P.units[u]);
+      const int tile = U.tile, mt = U.mt;
+      if (nb >= 1) {
         int wv = 1;
-        if (lane == 0) wv = wait_or_abort(smem_u32(tbl_empty + b), (uint32_t)(((li >> 1) - 1) & 1), abortf);
+        if (lane == 0) wv = wait_or_abort(smem_u32(tbl_empty + b), (uint32_t)((nb - 1) & 1), abortf);
         if (!__shfl_sync(0xffffffffu, wv, 0)) break;
       }
       int *stab = tables + b * kTableInts, *fexp_s = stab + kScatKeysB * kAtomsB;
@@ -203,7 +228,7 @@ __global__ void __launch_bounds__(kThreadsB, 1) bgemm_kernel(const Params P) {
       int nsl = 0;
       if (lane < kAtomsB) {
         const int64_t a = a_first + lane, i = P.atom0 + a;
-        nsl = a < P.natoms && (!P.atype || clampi(P.atype[i], 0, P.ntypes - 1) == P.alpha) ? P.nslots[i] : 0;
+        nsl = a < P.natoms && (!P.atype || clampi(P.atype[i], 0, P.ntypes - 1) == U.type) ? P.nslots[i] : 0;
       }
       int nmax = nsl;
 #pragma unroll
@@ -222,7 +247,7 @@ __global__ void __launch_bounds__(kThreadsB, 1) bgemm_kernel(const Params P) {
       }
       __syncwarp();
       if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(tbl_full + b)) : "memory");
-      ++li;
+      ++nb;
     }
   } else {
     // ---- epilogue: warps 2 .. 9, TMEM lane quadrant warp % 4, columns 16 ((warp - 2) / 4) .. + 15
@@ -231,25 +256,27 @@ __global__ void __launch_bounds__(kThreadsB, 1) bgemm_kernel(const Params P) {
     const int rl = 32 * q + lane;
     int li = 0;
     for (int u = blockIdx.x; u < nunits; u += gridDim.x) {
-      const int c = P.units[u], tile = c & 0xffff, mt = c >> 16;
+      const Unit U = unit_of(P.units[u]);
+      const int tile = U.tile, mt = U.mt;
       const int b = li & 1;
       const int64_t m0 = (int64_t)mt * kTM;
       const int64_t a_first = (int64_t)tile * kAtomsB;  // the unit's first atom in the chunk
-      const int *stab = tables + b * kTableInts, *fexp_s = stab + kScatKeysB * kAtomsB;
+      const int tw = li % kTableWarps;
+      const int *stab = tables + tw * kTableInts, *fexp_s = stab + kScatKeysB * kAtomsB;
       const int key0 = (int)(m0 / P.kq);
       if (et == 0)
-        uflag[0] = !*abortf && wait_or_abort(smem_u32(tbl_full + b), (uint32_t)((li >> 1) & 1), abortf) &&
+        uflag[0] = !*abortf && wait_or_abort(smem_u32(tbl_full + tw), (uint32_t)((li / kTableWarps) & 1), abortf) &&
                    wait_or_abort(smem_u32(acc_full + b), (uint32_t)((li >> 1) & 1), abortf);
       asm volatile("bar.sync 1, %0;" ::"r"(32 * kEpiWarpsB));  // the table is built and the MMAs done
       const bool ok = uflag[0] != 0;
       asm volatile("tcgen05.fence::after_thread_sync;");
-      const int Erow = m0 + rl < P.Mp ? P.Eexp[m0 + rl] : 0;
+      const int Erow = m0 + rl < P.Mp ? P.Eexp[U.type * P.Mp + m0 + rl] : 0;
       const int key = (int)((m0 + rl) / P.kq), qq = (int)(m0 + rl - (int64_t)key * P.kq);
       const int key_l = key - key0;
       const bool row_wanted = qq < 6 && key < P.nkeys;
       const uint32_t trow = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)b * kBufColsB;
       // the row's part of the shift from the exact integer's units to the fixed point's
-      const int2 ke = row_wanted ? P.kexp[key] : make_int2(0, 0);
+      const int2 ke = row_wanted ? P.kexp[(int64_t)U.type * P.nkeys + key] : make_int2(0, 0);
       const int qe = qq * (key % P.nint < P.n0 ? P.e0 : P.e1);  // d_q = dW[k][q] 2^-qe
       const int shr = (qq ? ke.y : ke.x) - tg::kGradPlaces - (Erow - qe + kOutExp7x8);
       // the warp's 16 columns, four (one atom) at a time: each output's seven diagonals recombined
@@ -278,10 +305,9 @@ __global__ void __launch_bounds__(kThreadsB, 1) bgemm_kernel(const Params P) {
         fx::Fix val[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-          long long hi;
-          unsigned long long lo;
-          diag7_s128(v, k, hi, lo);
-          val[k] = tg::grad_fix(hi, lo, qq, clampi(shr + fexp_s[c_lo + c0 + k], 0, 126));
+          long long T, A;  // the exact integer is T 2^32 + A
+          diag7_parts(v, k, T, A);
+          val[k] = fix_of(T, A, shr + fexp_s[c_lo + c0 + k]);
         }
         if (at >= 0)
 #pragma unroll
@@ -291,7 +317,7 @@ __global__ void __launch_bounds__(kThreadsB, 1) bgemm_kernel(const Params P) {
       __syncwarp();
       if (lane == 0) {
         asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(tmem_free + b)) : "memory");
-        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(tbl_empty + b)) : "memory");
+        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(tbl_empty + tw)) : "memory");
       }
       ++li;
     }

@@ -167,7 +167,7 @@ PlanLayout plan_layout(const Shape &s) {
   L.afwd = take(off, nt * kS * (size_t)s.Mpf * s.Kp * 2);
   L.efwd = take(off, nt * s.Mpf * sizeof(int));
   L.abwd = take(off, nt * (s.b8 ? tb::kSB : kS) * (size_t)s.Mpb * s.Kpm * 2);
-  L.ebwd = take(off, nt * s.Mpb * sizeof(int));
+  L.ebwd = take(off, nt * s.Mpb * sizeof(int) + 256);  // (longer than a plan whose backward held c_q: those are refused)
   L.total = off;
   return L;
 }
@@ -200,7 +200,8 @@ Layout make_layout(const Shape &s) {
 // C'[alpha][6 key + q][m] = c_q Delta_l^q / N_c (key = beta nint + l; rows past the keys: 0).
 // The interval's block of the table is pair-planar [3][M1][2] holding (a, b, c, d, e, f), the
 // coefficients of t^5 .. t^0.
-// kU: the coefficients of u^q, c_q Delta^q (the forward's); else of t^q, c_q (the backward's)
+// kU: the coefficients of u^q, c_q Delta^q (the forward's); else of the derivative, q c_q, and the constant c_0
+// (the backward's)
 __global__ void __launch_bounds__(256) coef_kernel(const double *__restrict__ table, TableGeom g, int ntypes, int M1,
                                                    int Kp, double scale, bool kU, double *__restrict__ Cp) {
   const int64_t total = (int64_t)ntypes * Kp * M1;
@@ -219,7 +220,7 @@ __global__ void __launch_bounds__(256) coef_kernel(const double *__restrict__ ta
       double p = 1.0;
       if (kU)
         for (int e = 0; e < q; ++e) p *= delta;
-      v = c * p * scale;
+      v = kU ? c * p * scale : (q > 1 ? q * c : c) * scale;
     }
     Cp[x] = v;
   }
@@ -739,8 +740,8 @@ __global__ void __launch_bounds__(128) bwd_units_kernel(const unsigned char *__r
 }
 
 // The 7 x 8-bit backward GEMM's units: the (8-atom tile, 128-row output tile) pairs that hold the slot
-// of some atom of the tile of type t, from the atoms' slot keys (a key's rows are 6 key .. 6 key + 5),
-// per centre type; one block per (type, tile), a warp per atom, the row tiles marked in a shared-memory
+// of some atom of the tile of type t, from the atoms' slot keys (a key's rows are 6 key .. 6 key + 5), of every
+// centre type in one list; one block per (type, tile), a warp per atom, the row tiles marked in a shared-memory
 // bit set.
 constexpr int kMaxRowTiles = 256;
 static_assert((int64_t)kMaxKeys * kQ <= (int64_t)kMaxRowTiles * kTM, "row tiles of the backward A fit the bit set");
@@ -748,7 +749,7 @@ __global__ void __launch_bounds__(32 * tb::kAtomsB) bwd_units8_kernel(const shor
                                                                     const int *__restrict__ nslots,
                                                                     const int32_t *__restrict__ atype, int ntypes,
                                                                     int cap, int64_t atom0, int64_t natoms,
-                                                                    int64_t ntiles8, int64_t maxunits8,
+                                                                    int64_t ntiles8,
                                                                     int *__restrict__ units, int *__restrict__ nunits,
                                                                     const GradExps X) {
   fill_key_exps(X, ntypes);
@@ -779,10 +780,9 @@ __global__ void __launch_bounds__(32 * tb::kAtomsB) bwd_units8_kernel(const shor
   }
   const int total = __shfl_sync(0xffffffffu, before, 31);
   int base = 0;
-  if (lane == 0 && total) base = atomicAdd(nunits + t, total);
+  if (lane == 0 && total) base = atomicAdd(nunits, total);
   base = __shfl_sync(0xffffffffu, base, 0) + before - cnt;
-  for (unsigned m = word; m; m &= m - 1u)
-    units[(size_t)t * maxunits8 + base++] = tb::unit_code((int)tile, 32 * lane + __ffs((int)m) - 1);
+  for (unsigned m = word; m; m &= m - 1u) units[base++] = tb::unit_code((int)tile, 32 * lane + __ffs((int)m) - 1, t);
 }
 
 // The forward's finish, one block per atom of the chunk: T of an atom whose item (its centre type, its
@@ -1421,41 +1421,39 @@ int grad(const dp_tc_plan *plan, const dp_table_info *info, const double *s, con
         return set_error(DP_ERR_CUDA, "%s: cudaMemsetAsync: %s", who, cudaGetErrorString(cudaGetLastError()));
       const int64_t ntiles8 = (n + tb::kAtomsB - 1) / tb::kAtomsB, nlist = (int64_t)ntypes * ntiles8;
       bwd_units8_kernel<<<(unsigned)nlist, 32 * tb::kAtomsB, 0, st>>>(
-          R.keys, R.nslots, atype, ntypes, S.cap, c0, n, ntiles8, S.maxunits8, reinterpret_cast<int *>(wk + L.units),
+          R.keys, R.nslots, atype, ntypes, S.cap, c0, n, ntiles8, reinterpret_cast<int *>(wk + L.units),
           reinterpret_cast<int *>(wk + L.nunits), X);
       if ((rc = launch_status(who))) return rc;
       prof_mark("tc_units", st);
-      for (int t = 0; t < ntypes; ++t) {
-        tb::Params G{};
-        G.aplanes = pk + PL.abwd + (size_t)t * tb::kSB * S.Mpb * S.Kpm * 2;
-        G.Eexp = reinterpret_cast<const int *>(pk + PL.ebwd) + (size_t)t * S.Mpb;
-        G.ka = S.Kpm / kTK;
-        G.bplanes = wk + L.bplanes;
-        G.Fexp = R.fexp;
-        G.Mp = S.Mpb;
-        G.scat = dW;
-        G.kexp = X.kexp + (size_t)t * S.nkeys;
-        G.gexp = X.gexp;
-        G.n0 = g.n0;
-        G.nint = g.nint;
-        G.e0 = X.e0;
-        G.e1 = X.e1;
-        G.bad = reinterpret_cast<int *>(wk + L.nunits) + kBadFlag;
-        G.keys = R.keys;
-        G.nslots = R.nslots;
-        G.cap = S.cap;
-        G.nkeys = S.nkeys;
-        G.kq = kQ;
-        G.atype = atype;
-        G.natoms = n;
-        G.atom0 = c0;
-        G.alpha = t;
-        G.ntypes = ntypes;
-        G.units = reinterpret_cast<const int *>(wk + L.units) + (size_t)t * S.maxunits8;
-        G.nunits = reinterpret_cast<const int *>(wk + L.nunits) + t;
-        if ((rc = tb::launch(G, st, who))) return rc;
-        prof_mark("tc_gemm_grad", st);
-      }
+      tb::Params G{};
+      G.aplanes = pk + PL.abwd;
+      G.astride = (size_t)tb::kSB * S.Mpb * S.Kpm * 2;
+      G.Eexp = X.Eexp;
+      G.ka = S.Kpm / kTK;
+      G.bplanes = wk + L.bplanes;
+      G.Fexp = R.fexp;
+      G.Mp = S.Mpb;
+      G.scat = dW;
+      G.kexp = X.kexp;
+      G.gexp = X.gexp;
+      G.n0 = g.n0;
+      G.nint = g.nint;
+      G.e0 = X.e0;
+      G.e1 = X.e1;
+      G.bad = reinterpret_cast<int *>(wk + L.nunits) + kBadFlag;
+      G.keys = R.keys;
+      G.nslots = R.nslots;
+      G.cap = S.cap;
+      G.nkeys = S.nkeys;
+      G.kq = kQ;
+      G.atype = atype;
+      G.natoms = n;
+      G.atom0 = c0;
+      G.ntypes = ntypes;
+      G.units = reinterpret_cast<const int *>(wk + L.units);
+      G.nunits = reinterpret_cast<const int *>(wk + L.nunits);
+      if ((rc = tb::launch(G, st, who))) return rc;
+      prof_mark("tc_gemm_grad", st);
     } else {
       // B = dT^T: the columns 4 a + k are the rows of this chunk's dT
       if ((rc = split_rows(dT + c0 * kCols * M1, M1, 1, kCols * n, M1, Np, S.Kpm, kTN, wk + L.bplanes, wk + L.fexp, st,

@@ -339,16 +339,14 @@ __device__ __forceinline__ double diag_to_f64(const float (&v)[kS][W], int c, in
 // The 7 x 8-bit scheme (Digits7x8): seven diagonal sums, diagonal d weighing 256^-(d+2), as one exact
 // integer S = sum_d v[d][c] 2^(8 (6 - d)), |S| < 2^72.01; an output is S 2^(E + F + kOutExp7x8).
 constexpr int kOutExp7x8 = 2 * Digits7x8::kPad - 2 * 8 - 8 * 6;
+// Its parts, S = T 2^32 + A, |T| < 2^40.01, |A| < 2^48.01.
 template <int W>
-__device__ __forceinline__ void diag7_s128(const float (&v)[7][W], int c, long long &hi, unsigned long long &lo) {
+__device__ __forceinline__ void diag7_parts(const float (&v)[7][W], int c, long long &T, long long &A) {
   int x[7];
 #pragma unroll
   for (int d = 0; d < 7; ++d) x[d] = exact_int(v[d][c]);
-  const long long T = (long long)x[0] * 65536 + (long long)x[1] * 256 + x[2];  // |T| < 2^40.01
-  const long long A = (long long)x[3] * 16777216 + (long long)x[4] * 65536 + (long long)x[5] * 256 + x[6];  // < 2^48.01
-  const unsigned long long tl = (unsigned long long)T << 32;
-  lo = tl + (unsigned long long)A;
-  hi = (T >> 32) + (A >> 63) + (lo < tl ? 1 : 0);
+  T = (long long)x[0] * 65536 + (long long)x[1] * 256 + x[2];
+  A = (long long)x[3] * 16777216 + (long long)x[4] * 65536 + (long long)x[5] * 256 + x[6];
 }
 
 // The rare case of diag_to_f64 (a result outside the normal range), out of line so that the epilogue
