@@ -32,11 +32,10 @@ using namespace tc;
 // ---- the backward's results as fixed points, for the rows kernel's integer arithmetic
 // dW[k][q] of (atom, interval) is exact in the GEMM's epilogue (a 128-bit integer).  The rows kernel takes
 // the constant d_0 = dW[k][0] and the derivative's coefficients D_q = q dW[k][q] 2^(-e q) (u = t 2^e, the
-// derivative sum_q D_q u^(q-1) by u), rounded to units of 2^(X + G - 61); the factor q is in the plan's
-// coefficients.  G bounds the atom's column, sum_m |dT_km| < 2^G; X comes from the table's rows of the interval
-// (exponents E_q, max_m |q c_q| < 2^E_q), apart for the constant and the rest so that neither loses places to
-// the other:
-//   q >= 1: 2^slope > sum_q 2^(E_q - e q), which bounds the derivative and its terms' sum;
+// derivative sum_q D_q u^(q-1) by u), rounded to units of 2^(X + G - 61).  G bounds the atom's column,
+// sum_m |dT_km| < 2^G; X comes from the table's rows of the interval (exponents E_q, max_m |c_q| < 2^E_q),
+// apart for the constant and the rest so that neither loses places to the other:
+//   q >= 1: 2^slope > sum_q q 2^(E_q - e q), which bounds the derivative and its terms' sum;
 //   q = 0:  value = max(E_0, slope) + 1, which bounds the polynomial and all its parts.
 // (With one exponent for all six the derivative would lose seven places at Delta = 0.01.)
 constexpr int kGradPlaces = 61;
@@ -53,15 +52,18 @@ __device__ __forceinline__ int2 key_exps(const int *__restrict__ E6, int e) {  /
       top = max(top, E[q] - e * q);
     }
   }
-  unsigned sum = 0;  // above sum_q 2^(E_q - e q - top + 20), below 2^23
+  unsigned sum = 0;  // above sum_q q 2^(E_q - e q - top + 20), below 2^24
 #pragma unroll
-  for (int q = 1; q < 6; ++q) sum += ((1u << 20) >> min(top - (E[q] - e * q), 31)) + 1u;
+  for (int q = 1; q < 6; ++q) sum += (((unsigned)q << 20) >> min(top - (E[q] - e * q), 31)) + 1u;
   const int slope = nf1 ? kNonFinite : top - 20 + 32 - __clz((int)sum);
   return make_int2(nf1 || E[0] >= kNonFinite ? kNonFinite : max(E[0], slope) + 1, slope);
 }
 
-// The 128-bit integer (hi, lo), |.| < 2^78, over 2^sh to the nearest integer (halves up).
-__device__ __forceinline__ fx::Fix grad_fix(long long hi, unsigned long long lo, int sh) {
+// The 128-bit integer (hi, lo) times max(q, 1), |.| < 2^80, over 2^sh to the nearest integer (halves up).
+__device__ __forceinline__ fx::Fix grad_fix(long long hi, unsigned long long lo, int q, int sh) {
+  const unsigned f = (unsigned)max(q, 1);
+  hi = hi * (long long)f + (long long)__umul64hi(lo, (unsigned long long)f);
+  lo *= f;
   const int a = min(sh, 63), b = min(max(sh - 64, 0), 62);
   const unsigned long long low = (lo >> a) | ((unsigned long long)hi << 1 << (63 - a));
   const unsigned long long half = sh > 0 ? (lo >> max(a - 1, 0)) & 1ull : 0ull;
@@ -475,7 +477,7 @@ __global__ void __launch_bounds__(kThreadsP, 1) tgemm_kernel(const Params P) {
               diag_s128(v, k, hi, lo);  // |.| < 2^74, in units three places above the finest asked for
               const int c = c_lo + c0 + k;
               const int sh = (qq ? ke.y : ke.x) + P.gexp[n0 + c] - kGradPlaces - (Erow - qe + fexp_s[c] + kOutExp) + 3;
-              P.scat[at + k * ldk] = grad_fix(hi << 3 | (long long)(lo >> 61), lo << 3, clampi(sh, 0, 126));
+              P.scat[at + k * ldk] = grad_fix(hi << 3 | (long long)(lo >> 61), lo << 3, qq, clampi(sh, 0, 126));
             }
           continue;
         }

@@ -81,9 +81,11 @@ struct Unit {
 };
 __device__ __forceinline__ Unit unit_of(int c) { return Unit{c & 0xffff, (c >> 16) & 0xff, c >> 24}; }
 
-// (T 2^32 + A) / 2^sh as the rows kernel's limbs, |.| < 2^61: each part rounded (halves up), which is exact
-// for T up to sh = 32.
-__device__ __forceinline__ fx::Fix fix_of(long long T, long long A, int sh) {
+// f (T 2^32 + A) / 2^sh as the rows kernel's limbs, |.| < 2^61 (f < 6; f |T| < 2^43, f |A| < 2^51): each part
+// rounded (halves up), which is exact for T up to sh = 32.
+__device__ __forceinline__ fx::Fix fix_of(long long T, long long A, int f, int sh) {
+  T *= f;
+  A *= f;
   const int a = clampi(sh, 1, 62), r = clampi(sh - 32, 0, 62), l = clampi(32 - sh, 0, 31);
   const long long hi = sh <= 32 ? T << l : (T + (1ll << max(r - 1, 0))) >> r;
   return fx::limbs<tg::kGradLimb>(hi + ((A + (1ll << (a - 1))) >> a));
@@ -307,7 +309,7 @@ __global__ void __launch_bounds__(kThreadsB, 1) bgemm_kernel(const Params P) {
         for (int k = 0; k < 4; ++k) {
           long long T, A;  // the exact integer is T 2^32 + A
           diag7_parts(v, k, T, A);
-          val[k] = fix_of(T, A, shr + fexp_s[c_lo + c0 + k]);
+          val[k] = fix_of(T, A, max(qq, 1), shr + fexp_s[c_lo + c0 + k]);
         }
         if (at >= 0)
 #pragma unroll

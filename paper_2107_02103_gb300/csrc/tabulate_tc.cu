@@ -167,7 +167,7 @@ PlanLayout plan_layout(const Shape &s) {
   L.afwd = take(off, nt * kS * (size_t)s.Mpf * s.Kp * 2);
   L.efwd = take(off, nt * s.Mpf * sizeof(int));
   L.abwd = take(off, nt * (s.b8 ? tb::kSB : kS) * (size_t)s.Mpb * s.Kpm * 2);
-  L.ebwd = take(off, nt * s.Mpb * sizeof(int) + 256);  // (longer than a plan whose backward held c_q: those are refused)
+  L.ebwd = take(off, nt * s.Mpb * sizeof(int));
   L.total = off;
   return L;
 }
@@ -200,8 +200,7 @@ Layout make_layout(const Shape &s) {
 // C'[alpha][6 key + q][m] = c_q Delta_l^q / N_c (key = beta nint + l; rows past the keys: 0).
 // The interval's block of the table is pair-planar [3][M1][2] holding (a, b, c, d, e, f), the
 // coefficients of t^5 .. t^0.
-// kU: the coefficients of u^q, c_q Delta^q (the forward's); else of the derivative, q c_q, and the constant c_0
-// (the backward's)
+// kU: the coefficients of u^q, c_q Delta^q (the forward's); else of t^q, c_q (the backward's)
 __global__ void __launch_bounds__(256) coef_kernel(const double *__restrict__ table, TableGeom g, int ntypes, int M1,
                                                    int Kp, double scale, bool kU, double *__restrict__ Cp) {
   const int64_t total = (int64_t)ntypes * Kp * M1;
@@ -220,7 +219,7 @@ __global__ void __launch_bounds__(256) coef_kernel(const double *__restrict__ ta
       double p = 1.0;
       if (kU)
         for (int e = 0; e < q; ++e) p *= delta;
-      v = kU ? c * p * scale : (q > 1 ? q * c : c) * scale;
+      v = c * p * scale;
     }
     Cp[x] = v;
   }
