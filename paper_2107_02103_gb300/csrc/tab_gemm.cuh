@@ -9,8 +9,8 @@
 // over the grid.  The TMEM accumulators (nine diagonals x 48 columns), the mbarriers and the stage ring
 // are set up once per CTA, and the roles run ahead of each other: warp 0 moves each slice's A block
 // (and in the backward its B block) into a ring of four stages (bulk copies counted on the stage's
-// "full" barrier); in the forward a split warp per stage writes the B block from the moments, as digit
-// planes, and arrives on the same barrier; lane 0 of warp 1 issues the slice's 13 MMAs and frees the
+// "full" barrier); in the forward two split warps per stage write the B block from the moments, as digit
+// planes, and arrive on the same barrier; lane 0 of warp 1 issues the slice's 13 MMAs and frees the
 // stage ("empty") when they complete; eight epilogue warps (two per TMEM lane quadrant, 24 columns
 // each) read the unit's accumulators once its last MMA has completed ("acc_full"), recombine each
 // output's diagonals exactly as an integer and round it once to f64 (diag_to_f64) -- or, for a piece
@@ -73,7 +73,8 @@ __device__ __forceinline__ fx::Fix grad_fix(long long hi, unsigned long long lo,
 
 constexpr int kEpiWarps = 8;    // two per TMEM lane quadrant
 constexpr long long kPartNaN = 1ll << 62;  // high word of a piece's output whose accumulators were not read
-constexpr int kSplitWarps = 4;  // forward: the B digit planes of each slice, made in shared memory
+constexpr int kSplitPerStage = 2;  // forward: the warps that make a slice's B digit planes in shared memory
+constexpr int kSplitWarps = kStages * kSplitPerStage;
 constexpr int kThreadsP = 32 * (2 + kEpiWarps + kSplitWarps);  // producer, MMA issuer, epilogue, split warps
 constexpr int kEpiCols = kTN / 2;              // columns per epilogue warp
 constexpr int kMaxUnitSlices = kMaxShareSlices;
@@ -200,7 +201,7 @@ __global__ void __launch_bounds__(kThreadsP, 1) tgemm_kernel(const Params P) {
   constexpr bool fused = kFwd;  // B made in shared memory by the split warps
   if (tid == 0) {
     for (int s = 0; s < kStages; ++s) {
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(full + s)), "r"(fused ? 2 : 1));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(full + s)), "r"(fused ? 1 + kSplitPerStage : 1));
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(empty + s)));
     }
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(acc_full)));
@@ -300,31 +301,34 @@ __global__ void __launch_bounds__(kThreadsP, 1) tgemm_kernel(const Params P) {
   } else if (warp >= 2 + kEpiWarps) {
     // ---- split warps (forward): each slice's B block -- B[6 key + q][4 a + k] = W_a[k][(key, q)], the
     // moments of the atom's run slot of that interval -- as balanced digit planes in the stage, in the
-    // tcgen05 K-major core-matrix layout.  Warp w owns stage w (the slices g with g % 4 == w), so four
-    // slices are made at once.  Lane (k = lane / 8, kp = lane % 8) makes the K entries 2 kp, 2 kp + 1 of
-    // column 4 i + k for the tile's atoms i = 0 .. 11 (one key per lane and slice, 6 being even): the
-    // column exponents and the unit's slice list are read once per unit, the run slots of the warp's
+    // tcgen05 K-major core-matrix layout.  Warps w and w + 4 own stage w (the slices g with g % 4 == w), half of
+    // the tile's atoms each, so four slices are made at once.  Lane (k = lane / 8, kp = lane % 8) makes the K
+    // entries 2 kp, 2 kp + 1 of column 4 i + k for the warp's six atoms i (one key per lane and slice, 6 being
+    // even): the column exponents and the unit's slice list are read once per unit, the run slots of the warp's
     // next slice are loaded while this slice's moments are, and the stage is waited for only before
     // the stores; then a fence makes the writes visible to the tensor core and the warp arrives on the
     // stage's "full" barrier.  (Measured: with a global load chain per slice the tensor core waited
-    // ~0.6 us per slice for its B block.)
-    static_assert(kSplitWarps == kStages, "a split warp per stage");
+    // ~0.6 us per slice for its B block.)  Why two warps a stage: the conversions were the longest part of the
+    // kernel (left out, 30 % less time; the MMAs 23 %, the epilogue 20 %, the copies nothing), and one warp a
+    // stage has nothing to issue while it waits.  The kernel on 4,096 Cu atoms and on 12,288 of water, us: one
+    // warp 92 and 330, two 66 and 239, three 69 and 247, four 71 and 257.
     if (fused) {
-      const int w = warp - (2 + kEpiWarps);
-      constexpr int kPairs = kTileAtomsP;  // per lane and slice: one pair of K entries per atom
-      static_assert(kTN * kTK / 2 == 32 * kPairs, "a pair per lane and atom");
+      const int w = (warp - (2 + kEpiWarps)) % kStages;
+      constexpr int kPairs = kTileAtomsP / kSplitPerStage;  // per lane and slice: one pair of K entries per atom
+      const int i0 = (warp - (2 + kEpiWarps)) / kStages * kPairs;  // the warp's first atom of the tile
+      static_assert(kTN * kTK / 2 == 32 * kPairs * kSplitPerStage, "a pair per lane and atom");
       const int k = lane >> 3, kp = lane & 7;
       int g0 = 0;  // slices of this CTA before the unit
       for (int u = wk.begin; u < wk.end; u += wk.step) {
         if (__shfl_sync(0xffffffffu, (int)*abortf, 0)) break;  // uniform over the warp
         const Unit U = unit_of<kFwd>(P, u);
-        const int64_t a_base = (int64_t)U.tile * kTileAtomsP;
+        const int64_t a_base = (int64_t)U.tile * kTileAtomsP + i0;
         const short *ulist = P.slist + ((size_t)U.alpha * P.ntiles + U.tile) * P.ka + U.s0;
         int E[kPairs];
         bool av[kPairs];
 #pragma unroll
         for (int i = 0; i < kPairs; ++i) {
-          E[i] = P.Fexp[U.tile * kTN + 4 * i + k];
+          E[i] = P.Fexp[U.tile * kTN + 4 * (i0 + i) + k];
           av[i] = a_base + i < P.natoms;
         }
 
@@ -365,7 +369,7 @@ __global__ void __launch_bounds__(kThreadsP, 1) tgemm_kernel(const Params P) {
           unsigned char *bstage = smem + w * kStageBytes + kS * kPlaneA;
 #pragma unroll
           for (int i = 0; i < kPairs; ++i) {
-            const int r = 4 * i + k;
+            const int r = 4 * (i0 + i) + k;
             uint32_t h[kS];
             digit_pairs(biased_fixed(xv[i].x, E[i]), biased_fixed(xv[i].y, E[i]), h);
             unsigned char *dst = bstage + (r >> 3) * kSBO + (r & 7) * 16 + (kp >> 2) * kLBO + (kp & 3) * 4;

@@ -17,7 +17,7 @@
 // (interval, atom) of the unit, from the atoms' slot keys) and column exponents into their table buffer
 // ahead of the epilogue ("tbl_full", released by "tbl_empty").  A table is a chain of dependent loads
 // (unit, atom types, slot counts, keys), longer than a unit's MMAs: with one table warp the kernel took
-// 300 us on the 16,384-atom H2O step and 47 us on the 4,096-atom Cu step, with two 234 and 44; four and
+// 300 us on the 12,288-atom water step and 47 us on the 4,096-atom Cu step, with two 234 and 44; four and
 // six give no more (239 and 45), and with the tables left out it is 218 and 37.  Copies, MMAs and the
 // epilogue's arithmetic are each hidden (leaving one out gains 1 to 10 %).  Every wait is bounded; a wait
 // that gives up stops the CTA's copies and MMAs, the rows kernel's results are then NaN (bad) and one
