@@ -431,7 +431,11 @@ int dp_descriptor_contract_grad_f32(const float *T, const float *dD, int64_t nlo
  * float's exponent range: magnitudes below ~1e-38 (relative parts below
  * ~1e-38 / 2^-24) flush towards zero, above ~3e38 overflow.
  *
- * dp_descriptor_contract_grad_df64 also stages dD_i: it needs
+ * The descriptor calls take no table, only f64 arrays: dp_descriptor_contract_df64
+ * gives dp_descriptor_contract_f64's results, and so does
+ * dp_descriptor_contract_grad_df64 up to M1 = 1024 while
+ * 8 M1 + M1 (M2 + 1) + 4 M2 ceil(M1 / 16) <= 7168 (their fixed-point kernels are
+ * the faster ones); wider, the latter runs in df64 arithmetic and needs
  * M1 (9 + M2) <= 7264 (DP_ERR_UNSUPPORTED beyond).
  *
  * The table is built for this arithmetic: [npair][nint][3][M1][4] float,

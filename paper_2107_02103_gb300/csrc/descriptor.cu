@@ -1,11 +1,12 @@
 // Descriptor (Sec. II): S_i = T_i^T is M1 x 4, S_i^< its first M2 rows, and
 // D_i = S_i (S_i^<)^T is M1 x M2:  D[i][m][n] = sum_k T[i][k][m] T[i][k][n].
 //
-// One warp per atom.  T_i (4 x M1) is staged in shared memory; the M1 x M2
-// output tile is contiguous, so lane l computes elements l, l + 32, ... of it
-// in storage order: every FP64 instruction has 32 busy lanes (M1*M2 is a
-// multiple of 32 for the paper's shapes) and every store is coalesced.
-// Both kernels also run in df64 arithmetic on double arrays (io_t).
+// On f64 arrays (the f64 and the df64 calls) a block per atom, in fixed point on the integer pipes
+// (desc_fixed.cuh).  In f32 one warp per atom: T_i (4 x M1) is staged in shared memory; the M1 x M2 output tile is
+// contiguous, so lane l computes elements l, l + 32, ... of it in storage order, every lane busy (M1*M2 is a
+// multiple of 32 for the paper's shapes) and every store coalesced.
+// The warp-per-atom backward takes f32 and, in f64 or df64 arithmetic (io_t), the shapes too wide for the
+// fixed-point one's shared memory.
 #include <type_traits>
 
 #include "desc_fixed.cuh"
@@ -292,9 +293,10 @@ int descriptor_grad(const io_t<real> *T, const io_t<real> *dD, int64_t nloc, int
   if (!T || !dD || !dT) return set_error(DP_ERR_NULL, "T, dD or dT is NULL");
   const int64_t blocks = (nloc + kDescWarps - 1) / kDescWarps;
   if (blocks > 2147483647LL) return set_error(DP_ERR_SHAPE, "nloc too large");
-  if constexpr (std::is_same<real, double>::value) {
-    // in fixed point wherever the staged dD_i leaves at least four blocks to an SM; the kernel below, which
-    // does not stage it, for wider ones
+  if constexpr (std::is_same<io_t<real>, double>::value) {
+    // in fixed point wherever the staged dD_i leaves at least four blocks to an SM; the kernel below for wider
+    // ones.  Also for the df64 call, whose arrays are f64 (12,288 atoms x 100 x 16: 0.279 ms in df64 arithmetic,
+    // 0.151 here; D 0.077 and 0.058)
     const size_t need = desc_grad_f64_entries(M1, M2) * sizeof(double);
     if (need <= 56 * 1024 && nloc <= 2147483647LL && M1 <= 1024) {
       if (need > 48 * 1024) {
@@ -360,7 +362,7 @@ int dp_descriptor_contract_f32(const float *T, int64_t nloc, int M1, int M2, flo
 }
 
 int dp_descriptor_contract_df64(const double *T, int64_t nloc, int M1, int M2, double *D, void *stream) {
-  return dpc::descriptor<dpc::df64>(T, nloc, M1, M2, D, stream);
+  return dpc::descriptor<double>(T, nloc, M1, M2, D, stream);
 }
 
 int dp_descriptor_contract_grad_df64(const double *T, const double *dD, int64_t nloc, int M1, int M2, double *dT,

@@ -72,3 +72,19 @@ def test_nonfinite_stays_in_its_elements(M1, M2):
         assert np.array_equal(D[i], clean[0][i]) and np.array_equal(dT[i], clean[1][i])
     m = np.isfinite(rT[3])
     assert np.abs(dT[3] - rT[3])[m].max() <= (M1 + M2) * 2.0 ** -53 * np.abs(dD[3]).max() * np.abs(T[3]).max()
+
+
+@pytest.mark.parametrize("M1,M2", [(1, 1), (17, 17), (100, 16), (140, 32), (200, 30)])
+def test_df64_calls_give_the_f64_results(M1, M2):
+    """The df64 calls' arrays are f64; they run the same kernels wherever those take the shape,
+    and refuse what they refused (a backward with M1 (9 + M2) > 7264)."""
+    rng = np.random.default_rng(M1)
+    T = torch.from_numpy(rng.normal(size=(7, 4, M1))).cuda()
+    dD = torch.from_numpy(rng.normal(size=(7, M1, M2))).cuda()
+    d = lib()
+    assert torch.equal(d.dp_descriptor_contract_df64(T, M2), d.dp_descriptor_contract(T, M2))
+    if M1 * (9 + M2) > 7264:
+        with pytest.raises(d.DPError):
+            d.dp_descriptor_contract_grad_df64(T, dD)
+    else:
+        assert torch.equal(d.dp_descriptor_contract_grad_df64(T, dD), d.dp_descriptor_contract_grad(T, dD))
