@@ -65,10 +65,11 @@ def footprint(w, esize: int, hbm_bytes: float = 280e9) -> dict:
             "atoms_per_280GB": int(hbm_bytes // ours), "atoms_per_280GB_uncompressed": int(hbm_bytes // (ours + net))}
 
 
-# f64 fitting GEMMs on the tensor cores: every operand element is split into 9 digits and the 45 digit
-# products with s + t <= 10 run as fp16 MMAs, so a GEMM of 2 n K N FP64 flop issues 45 times as many
-# fp16 MMA flop; their roofline is the dense 16-bit tensor rate (fp16 and bf16 run at the same rate).
-TC_DIGIT_PRODUCTS = 45  # fp16 digit products per FP64-equivalent FMA: nine 6-bit digits (s + t <= 10)
+# f64 GEMMs on the tensor cores: every operand element is split into digits and the digit products run as fp16
+# MMAs, so a GEMM of 2 n K N FP64 flop issues that many times as many fp16 MMA flop; their roofline is the
+# dense 16-bit tensor rate (fp16 and bf16 run at the same rate).
+TC_DIGIT_PRODUCTS = 45  # per FP64-equivalent FMA of the tabulation's GEMMs: nine 6-bit digits (s + t <= 10)
+FITTING_DIGIT_PRODUCTS = 36  # of the fitting net's: eight 7-bit digits (s + t <= 9)
 
 
 def tc_products(kernel: str, M1: int) -> int:
@@ -153,7 +154,8 @@ def interval_runs(w, info, n0: int, n1: int):
     return np.diff(np.concatenate([starts, [k.size]]))
 
 
-# --algo tc: algorithmic FMAs of its kernels, per valid row (FP64 pipe) or per run x M1 (the
+# --algo tc: algorithmic FMAs of its kernels, per valid row (f64 sums, which the kernels take in fixed point on
+# the integer pipes, so their share of the FP64 peak can pass 1) or per run x M1 (the
 # per-interval contraction on the tensor cores, each FMA as 45 fp16 digit products):
 #   tc_runs_moments  W[k][q] += R~_k u^q                 24 per row
 #   tc_rows          dE/dR~ and dE/ds by Horner in u     40 per row (20 + 16 + 4)
@@ -194,7 +196,8 @@ def moment_fmas(runs, M1: int) -> dict:
 # `ncu --set full` capture of its current version (the commit the capture was taken at beside each);
 # absent means no capture of the current kernel exists and `traffic` is reported as null.
 PROFILED_DRAM_BYTES = {("cu85", "f64", "grad", "moments"): 83838464 + 32080640,   # commit 7987c32
-                       ("cu85", "f64", "tc_rows", "tc"): 104717312 + 32222720}    # commit a508952
+                       ("cu85", "f64", "tc_rows", "tc"): 106909440 + 37977088,    # commit e2ecb8c
+                       ("cu85", "f64", "tc_runs_moments", "tc"): 70285312 + 12362496}
 
 
 def peak_tflops(dtype: str, mhz: float = SM_MAX_MHZ, nsm: int = NSM) -> float:
@@ -233,9 +236,10 @@ def step_bytes(w, esize: int) -> dict:
 
 
 def tc_step_bound(w, nruns: float, nsm: int, ms_step: float) -> dict:
-    """The roofline of the step the tensor-core path runs: the slowest of its FP64-pipe work (the per-row
-    moments, 24 FMA, and derivatives, 40 FMA, per valid row, and the descriptor's 4 M1 M2 per atom) at the
-    FP64 peak, its digit-product MMAs (24 M1 FMA per run and direction, 45 fp16 products each forward and
+    """The roofline of the step the tensor-core path runs: the slowest of its f64 work outside the GEMMs (the
+    per-row moments, 24 FMA, and derivatives, 40 FMA, per valid row, and the descriptor's 4 M1 M2 per atom)
+    counted as FMAs at the FP64 peak (the kernels take these sums in fixed point on the integer pipes, faster
+    than that peak), its digit-product MMAs (24 M1 FMA per run and direction, 45 fp16 products each forward and
     28 backward) at the measured dense 16-bit tensor peak, and its algorithmic bytes at the measured HBM
     bandwidth."""
     rows = float(w.evals) / w.M1
@@ -250,7 +254,7 @@ def tc_step_bound(w, nruns: float, nsm: int, ms_step: float) -> dict:
     return {"t_roof_ms": round(t[bound], 4), "bound": bound, "fp64_ms": round(t["fp64"], 4),
             "tensor_ms": round(t["tensor"], 4), "hbm_ms": round(t["hbm"], 4), "ms_per_step": round(ms_step, 4),
             "frac": round(t[bound] / ms_step, 4),
-            "basis": (f"fwd + descriptor + grad as the tc path computes them: FP64 {fp64_fma:.4g} FMA "
+            "basis": (f"fwd + descriptor + grad as the tc path computes them: {fp64_fma:.4g} f64 FMA "
                       f"({peak_basis('f64', nsm)}); tensor {tensor_flop:.4g} flop ({tbasis}); "
                       f"{sum(step_bytes(w, 8).values()):.4g} B ({hbasis})")}
 
@@ -777,7 +781,7 @@ def report(args, w, world, step_ms, k_ms, total_s, evals_all, e2e, clk, t_wall, 
         if k in nbytes:
             e["gbs"] = round(nbytes[k] / (mean[k] * 1e-3) / 1e9, 1)
         if tc and k in ("fitting_fwd", "fitting_grad"):  # FP64-equivalent above; the MMAs it takes here
-            e["tensor_tflops"] = round(TC_DIGIT_PRODUCTS * flops[k] / (mean[k] * 1e-3) / 1e12, 2)
+            e["tensor_tflops"] = round(FITTING_DIGIT_PRODUCTS * flops[k] / (mean[k] * 1e-3) / 1e12, 2)
             e["tensor_frac"] = round(e["tensor_tflops"] / tpk, 4)
         kernels[k] = e
     dom = max((k for k in mean if k in flops), key=mean.get)  # the roofline covers the FMA-counted kernels
@@ -792,7 +796,7 @@ def report(args, w, world, step_ms, k_ms, total_s, evals_all, e2e, clk, t_wall, 
     if tc and dom.startswith("fitting"):
         roofline.update({"bound": "tensor", "achieved": kernels[dom]["tensor_tflops"], "peak": round(tpk, 1),
                          "frac": kernels[dom]["tensor_frac"], "traffic": None,
-                         "peak_basis": f"{tbasis}; achieved counts all {TC_DIGIT_PRODUCTS} fp16 digit products"})
+                         "peak_basis": f"{tbasis}; achieved counts all {FITTING_DIGIT_PRODUCTS} fp16 digit products"})
     if tc_ms:  # the tensor-core tabulation: its own kernels, timed by the events its calls record
         step_mean = sum(step_ms) / len(step_ms)
         tmean = {k: sum(v) / len(v) for k, v in tc_ms.items()}
@@ -841,10 +845,10 @@ def report(args, w, world, step_ms, k_ms, total_s, evals_all, e2e, clk, t_wall, 
                                  "min(18 M1 L, 24 M1 + 40 L) grad" if args.algo in ("moments", "tc")
                                  else "per row: 9 M1 fwd, 18 M1 grad"),
                    **({"tc": ("per-interval contraction on the tensor cores (f64 by exact 9-digit splitting, "
-                              "fp16 MMAs); per-row work on the FP64 pipe: moments 24 FMA, derivatives 40 FMA "
-                              "per valid row")} if args.algo == "tc" else {}),
+                              "fp16 MMAs); per-row sums in fixed point on the integer pipes: moments 24 FMA, "
+                              "derivatives 40 FMA per valid row, counted against the FP64 peak")} if args.algo == "tc" else {}),
                    "l2": "flushed between steps (256 MiB write)",
-                   **({"fitting_gemm": ("tensor cores (tcgen05): f64 by exact 9-digit splitting, fp16 MMAs"
+                   **({"fitting_gemm": ("tensor cores (tcgen05): f64 by exact 8-digit splitting, fp16 MMAs"
                                         if tc else "FP64 pipe")} if getattr(args, "fitting", False) else {}),
                    "evals_per_step_per_gpu": w.evals, "atoms_per_step_per_gpu": w.nloc, "fill": round(w.fill, 4),
                    "device_sms": nsm,
