@@ -37,11 +37,11 @@
 //             uncut item writes its atoms' T, a piece its exact 128-bit partial sums),
 //             fwd_finish_kernel (T of the cut items, and D_i = T_i^T T_i[:, :M2] when asked for);
 //   backward: runs_kernel<false> (slot keys, slice flags; skipped when the forward's are reused),
-//             the split of dT (B), the GEMM units, and per centre type the GEMM (A = C'_alpha: K x
-//             channels, B = dT^T) scattering each used (atom, interval) block to its run slot --
-//             bgemm_kernel (tab_gemm_b8.cuh: 8-atom tiles, seven 8-bit digits) when M1 rounds up to
-//             at most 144, else tgemm_kernel<false> (12-atom tiles, nine 6-bit digits) -- and
-//             rows_kernel (dE/ds, dE/dR~).
+//             the split of dT (B), the GEMM units, and the GEMM (A = C'_alpha: K x channels, B =
+//             dT^T) scattering each used (atom, interval) block, as fixed points, to its run slot --
+//             bgemm_kernel (tab_gemm_b8.cuh: every centre type in one launch, 8-atom tiles, seven 8-bit
+//             digits) when M1 rounds up to at most 144, else tgemm_kernel<false> per centre type (12-atom
+//             tiles, nine 6-bit digits) -- and rows_kernel (dE/ds, dE/dR~).
 // The environment-fused calls (dp_tabulate_fusion_env_*_tc_f64) form each row from coordinates in
 // runs_kernel<.., true> and add each row's force and virial in rows_force_kernel instead.
 // The slot keys, their counts and the slice flags of every atom stay in the work buffer after
@@ -634,14 +634,20 @@ __device__ long long block_scan_1024(long long v, long long *red, long long *tot
 // costs its slice count plus kEpiCost; CTA b takes the cost range [b R, (b + 1) R) of the items' running
 // sum, R = ceil(total / ncta), so that every CTA gets the same work.  An item is cut where a CTA's range
 // begins and every 112 slices (the exactness bound of a share); the pieces of a cut item write their
-// partial results to consecutive part slots, which fwd_finish_kernel sums.  One block of 1024 threads,
-// each over a run of consecutive items.
+// partial results to consecutive part slots, which fwd_finish_kernel sums.  R is at least kMinRange: on a few
+// atoms, ranges of a slice or two took longer to sum than they saved in the GEMM.  One block of 1024 threads,
+// each over a run of consecutive items; costs in 32 bits, a 64-bit division a piece having set its time.
+// Measured, 64 atoms with 32 channels (schedule + GEMM + finish, us): 64 bits and no least range 38, 32 bits and
+// none 33, least range 3: 30, 6: 29, 12: 31; 192 atoms of water 44 without, 42 with 6; above 1,000 atoms no
+// difference but the schedule's own 6.6 -> 6.0.
+constexpr int kMinRange = kEpiCost;
+static_assert((int64_t)DP_MAX_TYPES * (kChunkAtoms / kTileAtoms) * ((DP_MAX_M1 + kTM - 1) / kTM) *
+                      ((kMaxKeys * kQ + kTK - 1) / kTK + kEpiCost) < (1ll << 30), "a schedule's costs fit 32 bits");
 __global__ void __launch_bounds__(1024) fwd_schedule_kernel(const int *__restrict__ scount, int64_t nitems,
                                                             int64_t ntiles, int nmt, int ncta, int4 *__restrict__ pieces,
                                                             int *__restrict__ pcta, int *__restrict__ cta_start,
                                                             int *__restrict__ npieces, int *__restrict__ pfirst) {
   __shared__ long long red[32];
-  __shared__ long long s_R;
   const int64_t per = (nitems + 1023) / 1024;
   const int64_t i0 = min(nitems, (int64_t)threadIdx.x * per), i1 = min(nitems, i0 + per);
   auto ns_of = [&](int64_t it) { return scount[it / nmt]; };  // item (t ntiles + tile) nmt + mt
@@ -651,20 +657,19 @@ __global__ void __launch_bounds__(1024) fwd_schedule_kernel(const int *__restric
     c += ns > 0 ? ns + kEpiCost : 0;
   }
   long long total;
-  const long long P0 = block_scan_1024(c, red, &total);
-  if (threadIdx.x == 0) s_R = max(1ll, (total + ncta - 1) / ncta);
-  __syncthreads();
-  const long long R = s_R;
+  const int P0 = (int)block_scan_1024(c, red, &total);
+  const int R = max(kMinRange, ((int)total + ncta - 1) / ncta);
   // the pieces of an item: cut where P + x reaches a multiple of R and where x reaches a multiple of 112
-  auto for_pieces = [&](long long P, int ns, auto &&f) {
+  auto for_pieces = [&](int P, int ns, auto &&f) {
     for (int x = 0; x < ns;) {
-      const long long nr = ((P + x) / R + 1) * R - P;
-      const int e = (int)min((long long)ns, min(nr, (long long)((x / kShareSlices + 1) * kShareSlices)));
-      f(x, e - x, (int)min((P + x) / R, (long long)ncta - 1));
+      const int b = (P + x) / R;
+      const int e = min(ns, min((b + 1) * R - P, (x / kShareSlices + 1) * kShareSlices));
+      f(x, e - x, min(b, ncta - 1));
       x = e;
     }
   };
-  long long np = 0, nslot = 0, P = P0;
+  long long np = 0, nslot = 0;
+  int P = P0;
   for (int64_t it = i0; it < i1; ++it) {
     const int ns = ns_of(it);
     int n = 0;
