@@ -889,7 +889,7 @@ __device__ __noinline__ double odd_double(long long v, int e, bool nan) {
 struct RowPoly {
   fx::Fix u1, u2, u3, u4, w2, w3, w4, w5;  // u^q and u^q / q
   int2 ke;
-  int e, drop;
+  int e, drop, half;
   bool plain, nan;
 };
 __device__ __forceinline__ RowPoly row_poly(const int2 ke, bool plain, double t, int e) {
@@ -902,7 +902,7 @@ __device__ __forceinline__ RowPoly row_poly(const int2 ke, bool plain, double t,
   R.u3 = fx::limbs<L>(fx::mul<L>(R.u2, R.u1));
   const long long s4 = fx::mul<L>(R.u2, R.u2);
   R.u4 = fx::limbs<L>(s4);
-  constexpr Fix third{0x15555555, 0x15555555}, fifth{0x33333333, 0x0ccccccc};  // 2^60 / 3, 2^60 / 5
+  constexpr Fix third{0x15555555, 0x15555555}, fifth{-0x0ccccccd, 0x0ccccccd};  // 2^60 / 3, 2^60 / 5
   R.w2 = fx::limbs<L>(s2 >> 1);
   R.w3 = fx::limbs<L>(fx::mul<L>(R.u3, third));
   R.w4 = fx::limbs<L>(s4 >> 2);
@@ -910,6 +910,7 @@ __device__ __forceinline__ RowPoly row_poly(const int2 ke, bool plain, double t,
   R.ke = ke;
   R.e = e;
   R.drop = ke.x - ke.y;  // the constant's units over the slope's, as a shift: >= 1
+  R.half = R.drop < 32 ? 1 << (R.drop - 1) : 0;  // so that it rounds (beyond, the constant decides alone)
   R.plain = plain && max(abs(ke.x), abs(ke.y)) <= 400 && R.drop < 32;
   R.nan = (__double2hiint(t) & 0x7ff00000) == 0x7ff00000;  // a NaN s
   return R;
@@ -924,6 +925,7 @@ __device__ __forceinline__ void row_component(const RowPoly &R, const fx::Fix *_
   const Fix c0{c01.x, c01.y}, c1{c01.z, c01.w}, c2{c23.x, c23.y}, c3{c23.z, c23.w}, c4{c45.x, c45.y},
       c5{c45.z, c45.w};
   fx::Acc p, q;
+  p.hi = R.half;
   p.mad(c1, R.u1);
   p.mad(c2, R.w2);
   p.mad(c3, R.w3);
