@@ -392,6 +392,8 @@ int dp_tc_wait_timeouts(unsigned int *count);
  * Descriptor (Sec. II): with S_i = T_i^T (M1 x 4) and S_i^< its first M2
  * rows, D_i = S_i (S_i^<)^T, i.e. D[i][m][n] = sum_k T[i][k][m] * T[i][k][n].
  *   T [nloc][4][M1] input,  D [nloc][M1][M2] output.
+ * In f64 every element is within 4 2^-53 sum_k |T[i][k][m] T[i][k][n]|, however
+ * the channels differ in size.
  * Errors: DP_ERR_NULL, DP_ERR_SHAPE (nloc < 0, M1 < 1, M2 < 1, M2 > M1),
  * DP_ERR_UNSUPPORTED (M1 > 4096, or T_i of four atoms not fitting in 227 KB
  * of shared memory: M1 > 1816 in f64, 3632 in f32), DP_ERR_CUDA.  nloc == 0

@@ -1,6 +1,6 @@
 // The descriptor's contractions (Sec. II: D = S (S^<)^T and its backward) in fixed point (fixed.cuh), for
-// f64 arrays: an atom's T, and its dE/dD, as two-limb integers against the atom's largest element, the
-// products on the integer pipes, one conversion per element on the FP64 pipe.  Shared by descriptor.cu and
+// f64 arrays: an atom's T, and its dE/dD, as two-limb integers against powers of two, the products on the
+// integer pipes, one conversion per element on the FP64 pipe.  Shared by descriptor.cu and
 // the tensor-core forward's finish, so that both give D the same bits.
 #pragma once
 
@@ -19,54 +19,79 @@ __device__ __forceinline__ int places_of(int hw, int places, bool &wild) {
   return hw ? places + 1022 - eb : 0;
 }
 
-// The largest high word, sign off, of x[0 .. n) in shared memory: each warp by itself.
-__device__ __forceinline__ int max_hiword(const double *x, int n, int lane) {
-  int m = 0;
-  for (int e = lane; e < n; e += 32) m = max(m, __double2hiint(x[e]) & 0x7fffffff);
-  return __reduce_max_sync(0xffffffffu, m);
-}
-
-// D's products of 59 places each, in limbs of 30 bits: four of them stay below 2^61 (hi) and 2^63 (mid).
-constexpr int kDescPlaces = 59, kDescLimb = 30;
+// A channel of an atom's T as fixed points against the largest of its four elements, in 60 places and limbs of
+// 30 bits (four products: hi below 2^62, mid below 2^63), with their magnitudes as floats in units of 2^30.
+struct alignas(16) Channel {
+  fx::Fix f[4];
+  float a[4];
+  int sh, pad[7];  // 80 bytes: neither the threads' stores nor their loads of a column meet in a bank
+};
+constexpr int kDescPlaces = 60, kDescLimb = 30;
+// The fixed-point sum of an element is off by at most 5.5 units: half a unit from either factor of each term, a
+// quarter from each dropped product of low limbs, half from the rounding.  From this sum of magnitudes on, that is
+// below 3 2^-53 of it, and with the rounding to f64 below the 4 2^-53 of four FP64 operations.
+constexpr float kDescLeast = 0x1.d8p53f;
+// Shared memory of desc_tile: T [4][M1] and the channels.
+__host__ __device__ constexpr size_t desc_tile_bytes(int M1) { return (size_t)M1 * (4 * sizeof(double) + sizeof(Channel)); }
 
 // One atom's D [M1][M2] by the threads of a block, from its T in Ts [4][M1] (written and synchronised), with
-// room for as many fixed points after it.  Consecutive threads take consecutive elements, M2 to a row.
+// room for the channels after it.  Consecutive threads take consecutive elements, M2 to a row.
 // Why fixed point: four FP64 instructions an element, 272 sub-partition clocks of that pipe a warp, bound
-// the kernels; one conversion takes it 64 and the 12 limb products the integer pipes 29.  Measured, the
-// forward's finish: copper (4,096 atoms x 100 x 16) 0.053 -> 0.033 ms, water (12,288) 0.142 -> 0.076 ms.
+// the kernels; one conversion takes it 64 and the 12 limb products the integer pipes 29.
+// Why an exponent a channel: channels differ in size, and D[m][n] is to be as exact against its own terms as
+// an FP64 sum (one exponent an atom lost 2^20 of an element whose channels were 2^-10 of the largest; an exponent
+// a channel and the test below cost D by itself 59.7 -> 65.8 us, 12,288 atoms x 100 x 16).  Where its two channels have their large elements in different k the sum is far below the
+// product of the two exponents; four FP32 multiply-adds tell, and such an element (like those of a channel
+// with an inf or NaN, or out of the exponents' range) is left to the FP64 pipe.
 __device__ __forceinline__ void desc_tile(const double *Ts, int M1, int M2, double *__restrict__ D) {
-  bool wild = false;
-  const int sh = places_of(max_hiword(Ts, 4 * M1, threadIdx.x & 31), kDescPlaces, wild);
+  Channel *C = reinterpret_cast<Channel *>(const_cast<double *>(Ts) + 4 * M1);
+  for (int m = threadIdx.x; m < M1; m += blockDim.x) {
+    double x[4];
+    int hw = 0, any = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      x[k] = Ts[k * M1 + m];
+      hw = max(hw, __double2hiint(x[k]) & 0x7fffffff);
+      any |= (__double2hiint(x[k]) & 0x7fffffff) | __double2loint(x[k]);
+    }
+    const int eb = hw >> 20;
+    const bool fixed = eb >= 650 && eb <= 1022 + kDescPlaces;
+    Channel c;
+    c.sh = fixed ? kDescPlaces + 1022 - eb : 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      c.f[k] = fixed ? fx::limbs<kDescLimb>(fx::from_double(x[k], c.sh)) : fx::Fix{0, 0};
+      // a channel of zeros passes the test with any other but one that is left to the FP64 pipe
+      c.a[k] = fixed ? (float)abs(c.f[k].hi) : (any ? 0.0f : 0x1p30f);
+    }
+    C[m] = c;
+  }
+  __syncthreads();
   // a thread keeps its column n and takes every step-th row (a block's rows lie back to back; M2 above the
   // block: several columns a thread)
   const int cols = min(M2, (int)blockDim.x), step = (int)blockDim.x / cols;
   const int m0 = (int)threadIdx.x / cols, n0 = (int)threadIdx.x - m0 * cols;
-  if (!wild) {  // uniform over the block
-    fx::Fix *Tf = reinterpret_cast<fx::Fix *>(const_cast<double *>(Ts) + 4 * M1);
-    for (int e = threadIdx.x; e < 4 * M1; e += blockDim.x) Tf[e] = fx::limbs<kDescLimb>(fx::from_double(Ts[e], sh));
-    __syncthreads();
-    const int ex = 2 * kDescLimb - 2 * sh;
-    if (m0 < step)
-      for (int n = n0; n < M2; n += cols) {
-        const fx::Fix b0 = Tf[n], b1 = Tf[M1 + n], b2 = Tf[2 * M1 + n], b3 = Tf[3 * M1 + n];
+  if (m0 >= step) return;
+  for (int n = n0; n < M2; n += cols) {
+    const Channel b = C[n];
 #pragma unroll 2
-        for (int m = m0; m < M1; m += step) {
-          fx::Acc p;
-          p.mad(Tf[m], b0);
-          p.mad(Tf[M1 + m], b1);
-          p.mad(Tf[2 * M1 + m], b2);
-          p.mad(Tf[3 * M1 + m], b3);
-          D[m * M2 + n] = fx::to_double(fx::over_unit<kDescLimb>(p), ex);
-        }
+    for (int m = m0; m < M1; m += step) {
+      const Channel &c = C[m];
+      fx::Acc p;
+      float mag = 0.0f;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        p.mad(c.f[k], b.f[k]);
+        mag = fmaf(c.a[k], b.a[k], mag);
       }
-  } else if (m0 < step) {
-    for (int n = n0; n < M2; n += cols)
-      for (int m = m0; m < M1; m += step) {
-        double v = Ts[m] * Ts[n];
+      double v = fx::to_double(fx::over_unit<kDescLimb>(p), 2 * kDescLimb - c.sh - b.sh);
+      if (mag < kDescLeast) {
+        v = Ts[m] * Ts[n];
 #pragma unroll
         for (int k = 1; k < 4; ++k) v = fma(Ts[k * M1 + m], Ts[k * M1 + n], v);
-        D[m * M2 + n] = v;
       }
+      D[m * M2 + n] = v;
+    }
   }
 }
 

@@ -334,7 +334,7 @@ int descriptor(const io_t<real> *T, int64_t nloc, int M1, int M2, io_t<real> *D,
   if (blocks > 2147483647LL) return set_error(DP_ERR_SHAPE, "nloc too large");
   if ((size_t)kDescWarps * 4 * M1 * sizeof(real) > 227 * 1024)
     return set_error(DP_ERR_UNSUPPORTED, "M1 = %d needs too much shared memory", M1);
-  const size_t smem = (size_t)(f64 ? 2 : kDescWarps) * 4 * M1 * sizeof(real);
+  const size_t smem = f64 ? dfx::desc_tile_bytes(M1) : (size_t)kDescWarps * 4 * M1 * sizeof(real);
   const void *kernel = f64 ? (const void *)descriptor_f64_kernel : (const void *)descriptor_kernel<real>;
   if (smem > 48 * 1024) {
     const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

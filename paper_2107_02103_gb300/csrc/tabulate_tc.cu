@@ -802,7 +802,7 @@ __global__ void __launch_bounds__(128) fwd_finish_kernel(const longlong2 *__rest
                                                          int64_t atom0, const int32_t *__restrict__ atype,
                                                          int ntypes, int M1, double *__restrict__ T, int M2,
                                                          double *__restrict__ D) {
-  extern __shared__ double Ts[];  // [4][M1] twice, when D is wanted: T and its fixed points
+  extern __shared__ __align__(16) double Ts[];  // when D is wanted: [4][M1], T, and desc_tile's room after it
   const int64_t a = blockIdx.x;
   const int64_t tile = a / kTileAtoms;
   const int al = (int)(a - tile * kTileAtoms);
@@ -1319,7 +1319,7 @@ int fwd(const dp_tc_plan *plan, const dp_table_info *info, const double *s, cons
     G.ntypes = ntypes;
     if ((rc = tg::launch(G, st, who, ncta))) return rc;
     prof_mark("tc_gemm_fwd", st);
-    fwd_finish_kernel<<<(unsigned)n, 128, D ? (size_t)2 * kCols * M1 * sizeof(double) : 0, st>>>(
+    fwd_finish_kernel<<<(unsigned)n, 128, D ? dfx::desc_tile_bytes(M1) : 0, st>>>(
         part, S.Mpf, G.Eexp, R.fexp, reinterpret_cast<const int *>(wk + L.npieces),
         reinterpret_cast<const int *>(wk + L.pfirst), ntiles, nmt, c0, atype, ntypes, M1, T, M2, D);
     if ((rc = launch_status(who))) return rc;
