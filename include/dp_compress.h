@@ -409,6 +409,10 @@ int dp_descriptor_contract_f32(const float *T, int64_t nloc, int M1, int M2, flo
  *   dT[i][k][m] = sum_{n<M2} dD[i][m][n] T[i][k][n] + [m < M2] sum_{m'} dD[i][m'][m] T[i][k][m']
  *   T [nloc][4][M1], dD [nloc][M1][M2] inputs;  dT [nloc][4][M1] output, fully
  *   overwritten (feed it to dp_tabulate_fusion_grad_*).
+ * In f64, with an atom's |dD[m][n]| <= R_m C_n, C_n the largest of its column and
+ * R_m the largest of its row over C_n, the first sum is within
+ * 2^-53 M2 R_m max_n C_n |T[k][n]| and the second within
+ * 2^-53 M1 C_m max_m' R_m' |T[k][m']|, and each is rounded to f64 every 16 terms.
  * Errors, limits and the nloc == 0 rule as dp_descriptor_contract_*; the
  * backward stages T_i and dT_i (M1 > 908 in f64, 1816 in f32 is
  * DP_ERR_UNSUPPORTED).
@@ -435,7 +439,7 @@ int dp_descriptor_contract_grad_f32(const float *T, const float *dD, int64_t nlo
  *
  * The descriptor calls take no table, only f64 arrays: dp_descriptor_contract_df64
  * gives dp_descriptor_contract_f64's results, and so does
- * dp_descriptor_contract_grad_df64 up to M1 = 1024 while
+ * dp_descriptor_contract_grad_df64 while
  * 8 M1 + M1 (M2 + 1) + 4 M2 ceil(M1 / 16) <= 7168 (their fixed-point kernels are
  * the faster ones); wider, the latter runs in df64 arithmetic and needs
  * M1 (9 + M2) <= 7264 (DP_ERR_UNSUPPORTED beyond).

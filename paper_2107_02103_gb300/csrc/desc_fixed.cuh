@@ -10,15 +10,6 @@ namespace dpc {
 namespace {
 namespace dfx {
 
-// Binary places sh with |x| 2^sh < 2^places over the values whose largest high word (sign off) is hw, and
-// `wild` where the sums are left to the FP64 pipe: an inf or NaN, or values so large or small that results
-// could leave the normal range.  Zeros only: places 0.
-__device__ __forceinline__ int places_of(int hw, int places, bool &wild) {
-  const int eb = hw >> 20;
-  wild |= hw != 0 && (eb < 650 || eb > 1400);
-  return hw ? places + 1022 - eb : 0;
-}
-
 // A channel of an atom's T as fixed points against the largest of its four elements, in 60 places and limbs of
 // 30 bits (four products: hi below 2^62, mid below 2^63), with their magnitudes as floats in units of 2^30.
 struct alignas(16) Channel {
@@ -40,9 +31,10 @@ __host__ __device__ constexpr size_t desc_tile_bytes(int M1) { return (size_t)M1
 // the kernels; one conversion takes it 64 and the 12 limb products the integer pipes 29.
 // Why an exponent a channel: channels differ in size, and D[m][n] is to be as exact against its own terms as
 // an FP64 sum (one exponent an atom lost 2^20 of an element whose channels were 2^-10 of the largest; an exponent
-// a channel and the test below cost D by itself 59.7 -> 65.8 us, 12,288 atoms x 100 x 16).  Where its two channels have their large elements in different k the sum is far below the
-// product of the two exponents; four FP32 multiply-adds tell, and such an element (like those of a channel
-// with an inf or NaN, or out of the exponents' range) is left to the FP64 pipe.
+// a channel and the test below cost D by itself 59.7 -> 65.8 us, 12,288 atoms x 100 x 16).  Where its two channels
+// have their large elements in different k the sum is far below the product of the two exponents; four FP32
+// multiply-adds tell, and such an element (like those of a channel with an inf or NaN, or out of the exponents'
+// range) is left to the FP64 pipe.
 __device__ __forceinline__ void desc_tile(const double *Ts, int M1, int M2, double *__restrict__ D) {
   Channel *C = reinterpret_cast<Channel *>(const_cast<double *>(Ts) + 4 * M1);
   for (int m = threadIdx.x; m < M1; m += blockDim.x) {

@@ -156,78 +156,167 @@ __global__ void __launch_bounds__(kDescWarps * 32)
 }
 
 // The same in f64, a block per atom, in fixed point (fixed.cuh): T_i [4][M1] and dD_i [M1][M2] staged in
-// shared memory as two-limb integers (T against the largest of each k, dD against its own), every sum taken in
-// pieces of 16 terms whose limb products stay exact in 64 bits (57 places, limbs of 28 bits: hi below 2^62),
-// one conversion to f64 per piece.  First the 4 M1 sums over n (M2 terms), then the 4 M2 sums over m' (M1
-// terms), spread over the block by piece and added in their order.  Rows of dD are padded to M2 + 1 entries.
+// shared memory as two-limb integers, every sum taken in pieces of 16 terms whose limb products stay exact in 64
+// bits (57 places, limbs of 28 bits: hi below 2^62), one conversion to f64 per piece.  First the 4 M1 sums over n
+// (M2 terms), then the 4 M2 sums over m' (M1 terms), spread over the block by piece and added in their order.
+// Rows of dD are padded to M2 + 1 entries.
 // Why: 8 M1 M2 FP64 multiply-adds an atom bound the kernel above (79 % of that pipe, copper); as limb
 // products they cost a ninth, and the FP64 pipe converts M1 M2 inputs and a sum per 16 terms.
-// Measured: copper (4,096 x 100 x 16) 0.104 -> 0.058 ms; 1,536 atoms 0.047 -> 0.031 ms.
+// Why the exponents: channels differ in size, so each row and column of dD has its own, 2^(C_n + r_m) above
+// |dD[m][n]|, and what leaves a sum through them goes into its copy of T: T[k][n] 2^C_n against its largest over n
+// for the first sums, T[k][m'] 2^r_m' against its largest over m' for the second.
+// Measured, 4,096 x 100 x 16: FP64 0.104 ms, one exponent for all of dD 0.054, these 0.064; 12,288: the last two
+// 0.152 and 0.181.
 constexpr int kGradPiece = 16, kGradL = 28, kDescGradPlaces = 57;
 constexpr int kDescGradThreads = 128;
 __host__ __device__ constexpr int pieces_of(int n) { return (n + kGradPiece - 1) / kGradPiece; }
-// 8-byte entries of shared memory: T, dD, the first term, the second term's pieces
+// What the choice of kernel goes by: the shared memory, in 8-byte entries, of T, dT, dD and the second sums' pieces.
 __host__ __device__ constexpr size_t desc_grad_f64_entries(int M1, int M2) {
   return (size_t)8 * M1 + (size_t)M1 * (M2 + 1) + (size_t)4 * M2 * pieces_of(M1);
 }
+// What the kernel takes (dT stays in registers; nine blocks an SM, eight with it, for 100 x 16): the two copies of T,
+// dD, the pieces, the exponents of dD's rows and columns.
+__host__ __device__ constexpr size_t desc_grad_f64_bytes(int M1, int M2) {
+  return ((size_t)4 * M1 + (size_t)M1 * (M2 + 1) + (size_t)4 * M2 * (pieces_of(M1) + 1)) * sizeof(double) +
+         (size_t)(M1 + M2) * sizeof(int);
+}
+constexpr int kNoValue = -(1 << 20), kNoKey = -2147483647;  // the exponent of zeros
 __global__ void __launch_bounds__(kDescGradThreads)
     descriptor_grad_f64_kernel(const double *__restrict__ T, const double *__restrict__ dD, int M1, int M2,
                                double *__restrict__ dT) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ int red[5];  // the largest high words: of T's rows, of dD
+  __shared__ int t1[4], t2[4], wild_s;  // exponents of the two copies of T; left to the FP64 pipe
   using fx::Fix;
-  Fix *Tf = reinterpret_cast<Fix *>(smem_raw);              // [4][M1]
-  double *G = reinterpret_cast<double *>(Tf + 4 * M1);       // [4][M1]
-  Fix *Df = reinterpret_cast<Fix *>(G + 4 * M1);             // [M1][M2 + 1]
+  Fix *Tf = reinterpret_cast<Fix *>(smem_raw);               // [4][M1]
+  Fix *Df = Tf + 4 * M1;                                      // [M1][M2 + 1]
   double *H = reinterpret_cast<double *>(Df + M1 * (M2 + 1));  // [pieces][4 M2]
-  const int tid = threadIdx.x, lane = tid & 31;
+  const int np = pieces_of(M1), tid = threadIdx.x, lane = tid & 31;
+  Fix *Tn = reinterpret_cast<Fix *>(H + 4 * M2 * np);  // [4][M2]
+  int *row_e = reinterpret_cast<int *>(Tn + 4 * M2);   // [M1]
+  int *col_e = row_e + M1;                             // [M2]
   const int64_t i = blockIdx.x;
   const double *Ti = T + i * 4 * M1, *Di = dD + i * (int64_t)M1 * M2;
   double *Td = reinterpret_cast<double *>(Tf), *Dd = reinterpret_cast<double *>(Df);
-  if (tid < 5) red[tid] = 0;
+  // exponents are kept as high words, sign off and the mantissa cleared: a field in bits 20 up
+  auto key = [](double x) { return __double2hiint(x) & 0x7fffffff; };
+  auto tiny = [](double x, int h) { return h < (1 << 20) && (h | __double2loint(x)); };  // a subnormal
+  for (int n = tid; n < M2; n += kDescGradThreads) col_e[n] = 0;
+  if (tid < 4) t1[tid] = t2[tid] = kNoValue;
+  if (tid == 4) wild_s = 0;
   __syncthreads();
-  int hd = 0;
+  // a thread's element m, n of every kDescGradThreads, and how it moves on (its column stays where M2 divides the block)
+  const int step_m = kDescGradThreads / M2, step_n = kDescGradThreads - step_m * M2;
+  const int m_first = tid / M2, n_first = tid - m_first * M2;
+  bool wild = false;
   {
-    const int step_m = kDescGradThreads / M2, step_n = kDescGradThreads - step_m * M2;
-    int m = tid / M2, n = tid - m * M2;
+    int m = m_first, n = n_first, c = 0;
 #pragma unroll 4
     for (int e = tid; e < M1 * M2; e += kDescGradThreads) {
       const double x = __ldg(Di + e);
       Dd[m * (M2 + 1) + n] = x;
-      hd = max(hd, __double2hiint(x) & 0x7fffffff);
+      const int h = key(x);
+      wild |= tiny(x, h);
+      c = max(c, h);
       m += step_m;
       n += step_n;
       if (n >= M2) n -= M2, ++m;
     }
+    if (step_n == 0) atomicMax(col_e + n_first, c);
   }
-  hd = __reduce_max_sync(0xffffffffu, hd);
-  if (lane == 0) atomicMax(red + 4, hd);
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    int ht = 0;
-    for (int m = tid; m < M1; m += kDescGradThreads) {
-      const double x = __ldg(Ti + k * M1 + m);
-      Td[k * M1 + m] = x;
-      ht = max(ht, __double2hiint(x) & 0x7fffffff);
+  for (int e = tid; e < 4 * M1; e += kDescGradThreads) Td[e] = __ldg(Ti + e);
+  __syncthreads();
+  if (step_n != 0) {  // uniform
+    const int cols = min(M2, kDescGradThreads), rows = kDescGradThreads / cols, m0 = tid / cols;
+    for (int n = tid - m0 * cols; n < M2 && m0 < rows; n += cols) {
+      int c = 0;
+      for (int m = m0; m < M1; m += rows) c = max(c, key(Dd[m * (M2 + 1) + n]));
+      atomicMax(col_e + n, c);
     }
-    ht = __reduce_max_sync(0xffffffffu, ht);
-    if (lane == 0) atomicMax(red + k, ht);
+    __syncthreads();
+  }
+  // columns: field C_n, kNoValue for zeros.  Rows: the largest of field - C_n
+  for (int m = tid; m < M1; m += kDescGradThreads) {
+    int r = kNoKey;
+#pragma unroll 4
+    for (int n = 0; n < M2; ++n) {
+      const int h = key(Dd[m * (M2 + 1) + n]);
+      r = max(r, h ? h - (col_e[n] & 0x7ff00000) : kNoKey);
+    }
+    row_e[m] = r == kNoKey ? kNoValue : r >> 20;
+    wild |= r != kNoKey && r < -(200 << 20);
   }
   __syncthreads();
-  bool wild = false;
-  const int sd = dfx::places_of(red[4], kDescGradPlaces, wild);
-  int st[4];
+  for (int n = tid; n < M2; n += kDescGradThreads) {
+    const int c = col_e[n] >> 20;
+    wild |= c && (c < 800 || c > 1022 + kDescGradPlaces);
+    col_e[n] = c ? c : kNoValue;
+  }
+  __syncthreads();
 #pragma unroll
-  for (int k = 0; k < 4; ++k) st[k] = dfx::places_of(red[k], kDescGradPlaces, wild);
-  auto places_t = [&](int k) { return k < 2 ? (k ? st[1] : st[0]) : (k == 2 ? st[2] : st[3]); };
-  const int np = pieces_of(M1);
+  for (int k = 0; k < 4; ++k) {
+    int a = kNoValue, b = kNoValue;
+    for (int m = tid; m < M1; m += kDescGradThreads) {
+      const double x = Td[k * M1 + m];
+      const int h = key(x), e = h >> 20;
+      wild |= e > 1500 || tiny(x, h);
+      if (h) {  // (a sum with kNoValue stays far below any other)
+        if (m < M2) a = max(a, e + col_e[m]);
+        b = max(b, e + row_e[m]);
+      }
+    }
+    a = __reduce_max_sync(0xffffffffu, a);
+    b = __reduce_max_sync(0xffffffffu, b);
+    if (lane == 0) atomicMax(t1 + k, a), atomicMax(t2 + k, b);
+  }
+  if (wild) wild_s = 1;
+  __syncthreads();
+  int e1[4], e2[4];  // the copies' exponents; zeros only: so high that all of T falls below the places
+  wild = wild_s != 0;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    e1[k] = t1[k] < -(1 << 14) ? 1 << 14 : t1[k];
+    e2[k] = t2[k] < -(1 << 14) ? 1 << 14 : t2[k];
+    wild |= e1[k] < 1402 || e2[k] < 402;  // results stay normal: exponents sum to 1202 at least
+  }
+  auto pick = [](const int (&e)[4], int k) { return k < 2 ? (k ? e[1] : e[0]) : (k == 2 ? e[2] : e[3]); };
+  double *dTi = dT + i * 4 * M1;
+  auto finish = [&](int k, int m, double v) {  // the first sum and, m < M2, the second's pieces
+    if (m < M2) {
+      double s = H[k * M2 + m];
+      for (int c = 1; c < np; ++c) s += H[c * 4 * M2 + k * M2 + m];
+      v += s;
+    }
+    dTi[k * M1 + m] = v;
+  };
+  constexpr int kTop = kDescGradPlaces + 1022;  // x with field e <= E has |x| 2^(kTop - E) < 2^57
   if (!wild) {  // uniform over the block
-    // (the padding entries hold whatever the memory held and are not read again)
-    for (int e = tid; e < M1 * (M2 + 1); e += kDescGradThreads) Df[e] = fx::limbs<kGradL>(fx::from_double(Dd[e], sd));
+    auto convert = [&](auto same_column) {
+      int m = m_first, n = n_first;
+      const int c = col_e[n];
+#pragma unroll 4
+      for (int e = tid; e < M1 * M2; e += kDescGradThreads) {
+        Fix &d = Df[m * (M2 + 1) + n];
+        // (zeros of a row or column of zeros: any shift up to 899)
+        const int sh = min(kTop - (decltype(same_column)::value ? c : col_e[n]) - row_e[m], 899);
+        d = fx::limbs<kGradL>(fx::from_double(Dd[m * (M2 + 1) + n], sh));
+        m += step_m;
+        if (!decltype(same_column)::value) {
+          n += step_n;
+          if (n >= M2) n -= M2, ++m;
+        }
+      }
+    };
+    if (step_n == 0)
+      convert(std::true_type{});
+    else
+      convert(std::false_type{});
 #pragma unroll
     for (int k = 0; k < 4; ++k)
-      for (int m = tid; m < M1; m += kDescGradThreads)
-        Tf[k * M1 + m] = fx::limbs<kGradL>(fx::from_double(Td[k * M1 + m], st[k]));
+      for (int m = tid; m < M1; m += kDescGradThreads) {
+        const double x = Td[k * M1 + m];
+        if (m < M2) Tn[k * M2 + m] = fx::limbs<kGradL>(fx::from_double_any(x, kTop - e1[k] + col_e[m]));
+        Tf[k * M1 + m] = fx::limbs<kGradL>(fx::from_double_any(x, kTop - e2[k] + row_e[m]));
+      }
     __syncthreads();
     // sum over cnt <= 16 terms of a (stride sa) times b (consecutive), over 2^(2 L)
     auto piece = [&](const Fix *a, int sa, const Fix *b, int cnt) {
@@ -240,25 +329,21 @@ __global__ void __launch_bounds__(kDescGradThreads)
       }
       return fx::over_unit<kGradL>(p);
     };
-    for (int p = tid; p < 4 * M1; p += kDescGradThreads) {  // pairs 4 m + k
-      const int m = p >> 2, k = p & 3, ex = 2 * kGradL - sd - places_t(k);
-      double v = 0.0;
-      for (int n = 0; n < M2; n += kGradPiece)
-        v += fx::to_double(piece(Df + m * (M2 + 1) + n, 1, Tf + k * M1 + n, min(kGradPiece, M2 - n)), ex);
-      G[k * M1 + m] = v;
-    }
+    constexpr int kEx = 2 * kGradL - 2 * kTop;
     for (int p = tid; p < 4 * M2 * np; p += kDescGradThreads) {  // (piece, k, m), m fastest
       const int c = p / (4 * M2), r = p - c * 4 * M2, k = r / M2, m = r - k * M2, m0 = c * kGradPiece;
       H[p] = fx::to_double(piece(Df + m0 * (M2 + 1) + m, M2 + 1, Tf + k * M1 + m0, min(kGradPiece, M1 - m0)),
-                           2 * kGradL - sd - places_t(k));
+                           kEx + col_e[m] + pick(e2, k));
+    }
+    __syncthreads();
+    for (int p = tid; p < 4 * M1; p += kDescGradThreads) {  // pairs 4 m + k
+      const int m = p >> 2, k = p & 3, ex = kEx + row_e[m] + pick(e1, k);
+      double v = 0.0;
+      for (int n = 0; n < M2; n += kGradPiece)
+        v += fx::to_double(piece(Df + m * (M2 + 1) + n, 1, Tn + k * M2 + n, min(kGradPiece, M2 - n)), ex);
+      finish(k, m, v);
     }
   } else {
-    for (int p = tid; p < 4 * M1; p += kDescGradThreads) {
-      const int m = p >> 2, k = p & 3;
-      double v = 0.0;
-      for (int n = 0; n < M2; ++n) v = fma(Dd[m * (M2 + 1) + n], Td[k * M1 + n], v);
-      G[k * M1 + m] = v;
-    }
     for (int p = tid; p < 4 * M2 * np; p += kDescGradThreads) {
       const int c = p / (4 * M2), r = p - c * 4 * M2, k = r / M2, m = r - k * M2;
       double v = 0.0;
@@ -266,18 +351,13 @@ __global__ void __launch_bounds__(kDescGradThreads)
         v = fma(Dd[mp * (M2 + 1) + m], Td[k * M1 + mp], v);
       H[p] = v;
     }
-  }
-  __syncthreads();
-  double *dTi = dT + i * 4 * M1;
-  for (int e = tid; e < 4 * M1; e += kDescGradThreads) {
-    const int k = e / M1, m = e - k * M1;
-    double v = G[e];
-    if (m < M2) {
-      double s = H[k * M2 + m];
-      for (int c = 1; c < np; ++c) s += H[c * 4 * M2 + k * M2 + m];
-      v += s;
+    __syncthreads();
+    for (int p = tid; p < 4 * M1; p += kDescGradThreads) {
+      const int m = p >> 2, k = p & 3;
+      double v = 0.0;
+      for (int n = 0; n < M2; ++n) v = fma(Dd[m * (M2 + 1) + n], Td[k * M1 + n], v);
+      finish(k, m, v);
     }
-    dTi[e] = v;
   }
 }
 
@@ -296,9 +376,9 @@ int descriptor_grad(const io_t<real> *T, const io_t<real> *dD, int64_t nloc, int
   if constexpr (std::is_same<io_t<real>, double>::value) {
     // in fixed point wherever the staged dD_i leaves at least four blocks to an SM; the kernel below for wider
     // ones.  Also for the df64 call, whose arrays are f64 (12,288 atoms x 100 x 16: 0.279 ms in df64 arithmetic,
-    // 0.151 here; D 0.077 and 0.058)
-    const size_t need = desc_grad_f64_entries(M1, M2) * sizeof(double);
-    if (need <= 56 * 1024 && nloc <= 2147483647LL && M1 <= 1024) {
+    // 0.181 here; D 0.077 and 0.066)
+    const size_t need = desc_grad_f64_bytes(M1, M2);
+    if (desc_grad_f64_entries(M1, M2) * sizeof(double) <= 56 * 1024 && nloc <= 2147483647LL) {
       if (need > 48 * 1024) {
         const cudaError_t e = cudaFuncSetAttribute(descriptor_grad_f64_kernel,
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);

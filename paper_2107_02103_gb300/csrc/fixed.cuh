@@ -75,6 +75,12 @@ __device__ __forceinline__ long long from_double(double x, int sh) {
   return __double2ll_rn(__hiloint2double(__double2hiint(x) + (sh << 20), __double2loint(x)));
 }
 
+// The same for any shift, where |x 2^sh| < 2^62: zero from where the exponent would fall below the normal range.
+__device__ __forceinline__ long long from_double_any(double x, int sh) {
+  const int e = ((__double2hiint(x) >> 20) & 0x7ff) + sh;
+  return e > 0 ? from_double(x, sh) : 0ll;
+}
+
 // v 2^e rounded to the nearest double, for e and |v| that keep it normal (|e| <= kSafeExp): one conversion
 // on the FP64 pipe.  (By 32-bit integer operations it takes the integer pipes 28 clocks; measured slower in
 // every kernel here, whose FP64 pipe is idle more than a third of the time.)
