@@ -68,14 +68,15 @@ __device__ __forceinline__ long long mul(const Fix a, const Fix b) {
   return over_unit<L>(p);
 }
 
-// x 2^sh to the nearest integer, |x 2^sh| < 2^62: the exponent moved by an integer add, one conversion on
-// the FP64 pipe (64 sub-partition clocks that the integer pipes do not wait for; by integer shifts it takes
-// them 41, measured).  sh < 900, so that a zero or subnormal x still gives zero.
+// x 2^sh to the nearest integer, |x 2^sh| < 2^62 and 0 <= sh < 900, so that a zero or subnormal x still gives
+// zero: the exponent moved by an integer add, one conversion on the FP64 pipe (64 sub-partition clocks that the
+// integer pipes do not wait for; by integer shifts it takes them 41, measured).  A negative shift would carry a
+// zero's exponent field into its sign.
 __device__ __forceinline__ long long from_double(double x, int sh) {
   return __double2ll_rn(__hiloint2double(__double2hiint(x) + (sh << 20), __double2loint(x)));
 }
 
-// The same for any shift, where |x 2^sh| < 2^62: zero from where the exponent would fall below the normal range.
+// The same for any shift: zero where the exponent would fall below the normal range.
 __device__ __forceinline__ long long from_double_any(double x, int sh) {
   const int e = ((__double2hiint(x) >> 20) & 0x7ff) + sh;
   return e > 0 ? from_double(x, sh) : 0ll;

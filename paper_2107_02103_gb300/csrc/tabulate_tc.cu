@@ -507,7 +507,8 @@ __global__ void __launch_bounds__(32 * kRunsWarps, 7) runs_kernel(const RunsPara
       if (!wild) {
         Fix *fr = reinterpret_cast<Fix *>(&st.r[0][lane]), *ft = reinterpret_cast<Fix *>(&st.tp[0][lane]);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) fr[33 * k] = fx::limbs<L>(fx::from_double(r[k], sh[k]));
+        for (int k = 0; k < 4; ++k)  // (the shift is uniform, and negative from 2^57 up)
+          fr[33 * k] = fx::limbs<L>(sh[k] < 0 ? fx::from_double_any(r[k], sh[k]) : fx::from_double(r[k], sh[k]));
         const Fix u1 = fx::limbs<L>(fx::from_double(u, 2 * L)), u2 = fx::limbs<L>(fx::mul<L>(u1, u1)),
                   u3 = fx::limbs<L>(fx::mul<L>(u2, u1));
         ft[33 * 0] = Fix{0, 1 << L};
@@ -896,7 +897,7 @@ __device__ __forceinline__ RowPoly row_poly(const int2 ke, bool plain, double t,
   constexpr int L = tg::kGradLimb;
   using fx::Fix;
   RowPoly R;
-  R.u1 = fx::limbs<L>(fx::from_double(t, 2 * L + e));
+  R.u1 = fx::limbs<L>(fx::from_double_any(t, 2 * L + e));  // (any step of the table)
   const long long s2 = fx::mul<L>(R.u1, R.u1);
   R.u2 = fx::limbs<L>(s2);
   R.u3 = fx::limbs<L>(fx::mul<L>(R.u2, R.u1));
