@@ -1464,7 +1464,7 @@ int grad(const dp_tc_plan *plan, const dp_table_info *info, const double *s, con
     } else {
       // B = dT^T: the columns 4 a + k are the rows of this chunk's dT
       if ((rc = split_rows(dT + c0 * kCols * M1, M1, 1, kCols * n, M1, Np, S.Kpm, kTN, wk + L.bplanes, wk + L.fexp, st,
-                           who)))
+                           who, kZerosGrad)))
         return rc;
       prof_mark("tc_split_dT", st);
       if (cudaMemsetAsync(wk + L.nunits, 0, (kBadFlag + 1) * sizeof(int), st) != cudaSuccess)

@@ -66,6 +66,7 @@ static_assert(kMaxShareK % kTK == 0 && kS * kTN <= (int)kTmemCols, "shares and T
 __host__ __device__ constexpr int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
 
 __device__ __forceinline__ int exp_bits(double x) { return (int)(((uint64_t)__double_as_longlong(x) >> 52) & 0x7ff); }
+__device__ __forceinline__ bool nonzero(double x) { return ((uint64_t)__double_as_longlong(x) << 1) != 0; }
 // E with max |x| < 2^E from the largest biased exponent (normal x: |x| < 2^(eb - 1022))
 __device__ __forceinline__ int exp_of_max(int ebmax) { return ebmax == 0x7ff ? kNonFinite : max(ebmax, 1) - 1022; }
 
@@ -131,8 +132,9 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)_
 // layer input, RT = kTM) and for B (RT = kTN; forward: the columns of W, ld_r = 1, ld_k = N;
 // backward: the rows of W).
 __global__ void __launch_bounds__(128) row_exps_kernel(const double *__restrict__ X, int64_t ld_r, int64_t ld_k,
-                                                       int64_t nrows, int K, int64_t rows_p, int *__restrict__ exps) {
-  // one warp per row: E with max_k |x_rk| < 2^E
+                                                       int64_t nrows, int K, int64_t rows_p, int zeros,
+                                                       int *__restrict__ exps) {
+  // one warp per row: E with max_k |x_rk| < 2^E, `zeros` for a row of zeros
   const int lane = threadIdx.x & 31;
   const int64_t r = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
   if (r >= rows_p) return;  // warp-uniform
@@ -140,7 +142,11 @@ __global__ void __launch_bounds__(128) row_exps_kernel(const double *__restrict_
   if (r < nrows)
     for (int k = lane; k < K; k += 32) eb = max(eb, exp_bits(__ldg(X + r * ld_r + k * ld_k)));
   eb = __reduce_max_sync(0xffffffffu, eb);
-  if (lane == 0) exps[r] = exp_of_max(eb);
+  bool any = eb != 0;  // zeros, or subnormals?
+  if (!any && r < nrows)
+    for (int k = lane; k < K; k += 32) any |= nonzero(__ldg(X + r * ld_r + k * ld_k));
+  any = __any_sync(0xffffffffu, any);
+  if (lane == 0) exps[r] = any ? exp_of_max(eb) : zeros;
 }
 
 constexpr int kSplitK = 64;  // K per warp of split_rows_kernel
@@ -361,7 +367,10 @@ __device__ __noinline__ double output_value_rare(float v0, float v1, float v2, f
 // all of K (lane = (row ri8 = lane / 4, pair of k kp = lane % 4)), a first pass over the rows for their
 // largest exponents (reduced over the row's four lanes), a second for the digits.  For short rows
 // (the tabulation's dT^T, K = M1 <= 256), where a launch per pass costs more than the passes.  Also G with
-// sum_k |x_rk| < 2^G per row, G >= E (gexps; kNonFinite for a row with an inf or NaN).
+// sum_k |x_rk| < 2^G per row, G >= E (gexps; kNonFinite for a row with an inf or NaN).  A row of zeros (a plane of
+// atoms, a masked gradient) gets the exponent of ordinary data: as the least one it sent every row of the atom out of
+// the rows kernel's fast conversion (3,000 atoms of water, one component zero: the backward 131 us, 147 so).
+constexpr int kZerosGrad = 0;  // the exponent of a column of zeros of dT^T
 template <class D>
 __global__ void __launch_bounds__(128) split_rows_1k_kernel(const double *__restrict__ X, int64_t ld_r, int64_t ld_k,
                                                             int64_t nrows, int K, int64_t rows_p, int Kp, int RT,
@@ -378,7 +387,12 @@ __global__ void __launch_bounds__(128) split_rows_1k_kernel(const double *__rest
   for (int k0 = 0; k0 < Kp; k0 += 8) eb = max(eb, max(exp_bits(x(k0 + 2 * kp)), exp_bits(x(k0 + 2 * kp + 1))));
   eb = max(eb, __shfl_xor_sync(0xffffffffu, eb, 1));
   eb = max(eb, __shfl_xor_sync(0xffffffffu, eb, 2));
-  const int E = exp_of_max(eb);
+  bool any = eb != 0;
+  if (__any_sync(0xffffffffu, !any)) {  // zeros, or subnormals?
+    for (int k0 = 0; k0 < Kp; k0 += 8) any |= nonzero(x(k0 + 2 * kp)) || nonzero(x(k0 + 2 * kp + 1));
+    any = (__ballot_sync(0xffffffffu, any) >> (lane & ~3) & 0xfu) != 0;
+  }
+  const int E = any ? exp_of_max(eb) : kZerosGrad;
   // the row's sum of magnitudes in units of 2^(E - 20), each rounded up: below 2^28 + 2^8
   unsigned mag = 0;
   for (int k0 = 0; k0 < Kp; k0 += 8)
@@ -414,10 +428,12 @@ int split_rows_1k(const double *X, int64_t ld_r, int64_t ld_k, int64_t nrows, in
   return launch_status(who);
 }
 
+// zeros: the exponent of a row of zeros.  The plan's say that a coefficient is nowhere large (key_exps).
+constexpr int kZerosPlan = -1021;
 template <class D = Digits9x6>
 int split_rows(const double *X, int64_t ld_r, int64_t ld_k, int64_t nrows, int K, int64_t rows_p, int Kp, int RT,
-               unsigned char *planes, unsigned char *exps, cudaStream_t st, const char *who) {
-  row_exps_kernel<<<(unsigned)((rows_p + 3) / 4), 128, 0, st>>>(X, ld_r, ld_k, nrows, K, rows_p,
+               unsigned char *planes, unsigned char *exps, cudaStream_t st, const char *who, int zeros = kZerosPlan) {
+  row_exps_kernel<<<(unsigned)((rows_p + 3) / 4), 128, 0, st>>>(X, ld_r, ld_k, nrows, K, rows_p, zeros,
                                                                  reinterpret_cast<int *>(exps));
   int rc = launch_status(who);
   if (rc) return rc;
