@@ -57,8 +57,10 @@ __device__ __forceinline__ void radius(real r2, real &r, real &inv_r) {
   inv_r = recip(r);
 }
 // In f64: from the float 1/sqrt (its argument's and result's fields moved by integer operations) by one step of
-// third order, y (1 + e/2 + 3 e^2/8) with e = 1 - r2 y^2 below 2^-20: six FP64 instructions where the square
-// root and the division took about twenty.  Both within 1.5 units of the last place.
+// third order, y (1 + e/2 + 3 e^2/8) with e = 1 - r2 y^2 below 2^-20, and r = r2 y with its own residual taken off
+// (r2 - r^2) y / 2: eight FP64 instructions where the square root and the division took about twenty.  1/r within a
+// unit of the last place, r rounded as by sqrt but for near ties; without the residual r was off by up to 1.6 units,
+// which in the switch's tail made ds/dr 1.5 times less exact.
 __device__ __forceinline__ void radius(double r2, double &r, double &inv_r) {
   const unsigned hi = (unsigned)__double2hiint(r2), lo = (unsigned)__double2loint(r2);
   if (hi - 0x39b00000u >= 0x0c800000u) {  // outside [2^-100, 2^100), negative, NaN
@@ -71,6 +73,7 @@ __device__ __forceinline__ void radius(double r2, double &r, double &inv_r) {
   const double e = fma(-(r2 * y0), y0, 1.0);
   inv_r = fma(y0, fma(0.375, e, 0.5) * e, y0);
   r = r2 * inv_r;
+  r = fma(fma(-r, r, r2), __hiloint2double(__double2hiint(inv_r) - (1 << 20), __double2loint(inv_r)), r);
 }
 
 // weight() in f64: the switch and its derivative are polynomials of u in fixed point (fixed.cuh; units of
