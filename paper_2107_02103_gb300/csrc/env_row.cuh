@@ -129,7 +129,8 @@ __device__ __forceinline__ void weight(const EP &P, double r, double inv_r, doub
     dsv = -inv_r * inv_r;
   } else if (rb < __double_as_longlong(P.rc)) {
     const SwitchFixed S = switch_fixed(P.kind, fx::from_double((r - P.rcs) * P.inv_width, 60));
-    sv = fx::to_double(S.w, -60) * inv_r;
+    // (rounded by itself: no kernel may fuse it into what it does next, or their rows would not be the same bits)
+    sv = __dmul_rn(fx::to_double(S.w, -60), inv_r);
     dsv = fma(fx::to_double(S.dw, -58), P.inv_width, -sv) * inv_r;
   } else {
     sv = 0.0;

@@ -300,7 +300,7 @@ __device__ __forceinline__ EnvVals env_vals(const EnvRow &E, int64_t i, int j) {
   weight(E, r, v.inv_r, v.sv, v.dsv);
   v.a = v.sv * v.inv_r;
   const double a = E.unit ? v.a : v.a * E.inv_std_all;
-  v.r4[0] = E.unit ? v.sv : (v.sv - E.mean) * E.inv_std;
+  v.r4[0] = E.unit ? v.sv : __dmul_rn(v.sv - E.mean, E.inv_std);  // (the offset s - x_l is formed from it)
   v.r4[1] = a * v.d[0];
   v.r4[2] = a * v.d[1];
   v.r4[3] = a * v.d[2];
