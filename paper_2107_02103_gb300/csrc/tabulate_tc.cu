@@ -893,7 +893,8 @@ struct RowPoly {
   int e, drop, half;
   bool plain, nan;
 };
-__device__ __forceinline__ RowPoly row_poly(const int2 ke, bool plain, double t, int e) {
+// nan: the row's interval has no slot.
+__device__ __forceinline__ RowPoly row_poly(const int2 ke, bool plain, double t, int e, bool nan) {
   constexpr int L = tg::kGradLimb;
   using fx::Fix;
   RowPoly R;
@@ -913,7 +914,7 @@ __device__ __forceinline__ RowPoly row_poly(const int2 ke, bool plain, double t,
   R.drop = ke.x - ke.y;  // the constant's units over the slope's, as a shift: >= 1
   R.half = R.drop < 32 ? 1 << (R.drop - 1) : 0;  // so that it rounds (beyond, the constant decides alone)
   R.plain = plain && max(abs(ke.x), abs(ke.y)) <= 400 && R.drop < 32;
-  R.nan = (__double2hiint(t) & 0x7ff00000) == 0x7ff00000;  // a NaN s
+  R.nan = nan || (__double2hiint(t) & 0x7ff00000) == 0x7ff00000;  // (a NaN s)
   return R;
 }
 // P_k and P_k' of component k, whose column's exponent is g.
@@ -986,8 +987,9 @@ __global__ void __launch_bounds__(32 * kRowsWarps, 7) rows_kernel(const RowsPara
     bool clamped;
     const int l = locate_fast(P.g, P.gf, P.nodes, sv, t, clamped);
     const int key = b * P.g.nint + l;
-    const fx::Fix *slot = dWa + (size_t)smap[key] * 24;
-    const RowPoly R = row_poly(__ldg(kexp + key), plain, t, l < P.g.n0 ? P.e0 : P.e1);
+    const int at = smap[key];  // -1: runs reused from a call on other rows
+    const fx::Fix *slot = dWa + max(at, 0) * 24;
+    const RowPoly R = row_poly(__ldg(kexp + key), plain, t, l < P.g.n0 ? P.e0 : P.e1, at < 0);
     const double2 *rr = reinterpret_cast<const double2 *>(Rrow + (size_t)row * 4);
     double2 *dr = reinterpret_cast<double2 *>(drow + (size_t)row * 4);
     double ds = 0.0;
@@ -1050,8 +1052,9 @@ __global__ void __launch_bounds__(32 * kRowsWarps, 4) rows_force_kernel(const Ro
     bool clamped;
     const int l = locate_fast(P.g, P.gf, P.nodes, ev.r4[0], t, clamped);
     const int key = b * P.g.nint + l;
-    const fx::Fix *slot = dWa + (size_t)smap[key] * 24;
-    const RowPoly R = row_poly(__ldg(kexp + key), plain, t, l < P.g.n0 ? P.e0 : P.e1);
+    const int at = smap[key];  // -1: runs reused from a call on other rows
+    const fx::Fix *slot = dWa + max(at, 0) * 24;
+    const RowPoly R = row_poly(__ldg(kexp + key), plain, t, l < P.g.n0 ? P.e0 : P.e1, at < 0);
     // dE/ds = sum_k R~[k] P_k', R~[1 .. 3] = ce d
     double d4[4], dp[4];
 #pragma unroll
