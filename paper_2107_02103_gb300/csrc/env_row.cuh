@@ -122,8 +122,11 @@ __device__ __forceinline__ SwitchFixed switch_fixed(int kind, long long u) {
 }
 template <typename EP>
 __device__ __forceinline__ void weight(const EP &P, double r, double inv_r, double &sv, double &dsv) {
-  // r >= 0, compared as integers: a NaN's bits, its sign off, lie above every radius
-  const long long rb = __double_as_longlong(r) & 0x7fffffffffffffffll;
+  // r >= 0, compared as integers: a NaN's bits, its sign off, lie above every radius.  (The bits through PTX: of a
+  // square root the compiler takes the sign to be off already, which is not so for a NaN.)
+  long long rb;
+  asm("mov.b64 %0, %1;" : "=l"(rb) : "d"(r));
+  rb &= 0x7fffffffffffffffll;
   if (rb < __double_as_longlong(P.rcs)) {
     sv = inv_r;
     dsv = -inv_r * inv_r;
