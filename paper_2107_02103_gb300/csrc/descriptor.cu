@@ -7,6 +7,7 @@
 // multiple of 32 for the paper's shapes) and every store coalesced.
 // The warp-per-atom backward takes f32 and, in f64 or df64 arithmetic (io_t), the shapes too wide for the
 // fixed-point one's shared memory.
+#include <algorithm>
 #include <type_traits>
 
 #include "desc_fixed.cuh"
@@ -361,6 +362,15 @@ __global__ void __launch_bounds__(kDescGradThreads)
   }
 }
 
+// Launches of a block per atom over as many grids as nloc takes: f(first atom, blocks).
+constexpr int64_t kMaxGrid = 2147483647;
+template <class F>
+int in_grids(int64_t nloc, F &&f) {
+  for (int64_t i0 = 0; i0 < nloc; i0 += kMaxGrid)
+    if (int rc = f(i0, (unsigned)std::min<int64_t>(kMaxGrid, nloc - i0))) return rc;
+  return DP_OK;
+}
+
 template <typename real>
 int descriptor_grad(const io_t<real> *T, const io_t<real> *dD, int64_t nloc, int M1, int M2, io_t<real> *dT,
                     void *stream) {
@@ -372,20 +382,23 @@ int descriptor_grad(const io_t<real> *T, const io_t<real> *dD, int64_t nloc, int
   if (nloc == 0) return DP_OK;
   if (!T || !dD || !dT) return set_error(DP_ERR_NULL, "T, dD or dT is NULL");
   const int64_t blocks = (nloc + kDescWarps - 1) / kDescWarps;
-  if (blocks > 2147483647LL) return set_error(DP_ERR_SHAPE, "nloc too large");
+  if (blocks > kMaxGrid) return set_error(DP_ERR_SHAPE, "nloc too large");
   if constexpr (std::is_same<io_t<real>, double>::value) {
     // in fixed point wherever the staged dD_i leaves at least four blocks to an SM; the kernel below for wider
     // ones.  Also for the df64 call, whose arrays are f64 (12,288 atoms x 100 x 16: 0.279 ms in df64 arithmetic,
     // 0.181 here; D 0.077 and 0.066)
     const size_t need = desc_grad_f64_bytes(M1, M2);
-    if (desc_grad_f64_entries(M1, M2) * sizeof(double) <= 56 * 1024 && nloc <= 2147483647LL) {
+    if (desc_grad_f64_entries(M1, M2) * sizeof(double) <= 56 * 1024) {
       if (need > 48 * 1024) {
         const cudaError_t e = cudaFuncSetAttribute(descriptor_grad_f64_kernel,
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
         if (e != cudaSuccess) return set_error(DP_ERR_CUDA, "dp_descriptor_contract_grad: %s", cudaGetErrorString(e));
       }
-      descriptor_grad_f64_kernel<<<(unsigned)nloc, kDescGradThreads, need, (cudaStream_t)stream>>>(T, dD, M1, M2, dT);
-      return launch_status("dp_descriptor_contract_grad");
+      return in_grids(nloc, [&](int64_t i0, unsigned n) {
+        descriptor_grad_f64_kernel<<<n, kDescGradThreads, need, (cudaStream_t)stream>>>(
+            T + i0 * 4 * M1, dD + i0 * M1 * M2, M1, M2, dT + i0 * 4 * M1);
+        return launch_status("dp_descriptor_contract_grad");
+      });
     }
   }
   const size_t smem = (size_t)kDescWarps * desc_grad_smem_per_warp<real>(M1, M2) * sizeof(real);
@@ -409,22 +422,29 @@ int descriptor(const io_t<real> *T, int64_t nloc, int M1, int M2, io_t<real> *D,
   if (M1 > 4096) return set_error(DP_ERR_UNSUPPORTED, "M1 = %d > 4096", M1);
   if (nloc == 0) return DP_OK;
   if (!T || !D) return set_error(DP_ERR_NULL, "T or D is NULL");
-  constexpr bool f64 = std::is_same<real, double>::value;
-  const int64_t blocks = f64 ? nloc : (nloc + kDescWarps - 1) / kDescWarps;
-  if (blocks > 2147483647LL) return set_error(DP_ERR_SHAPE, "nloc too large");
+  const int64_t blocks = (nloc + kDescWarps - 1) / kDescWarps;
+  if (blocks > kMaxGrid) return set_error(DP_ERR_SHAPE, "nloc too large");
   if ((size_t)kDescWarps * 4 * M1 * sizeof(real) > 227 * 1024)
     return set_error(DP_ERR_UNSUPPORTED, "M1 = %d needs too much shared memory", M1);
-  const size_t smem = f64 ? dfx::desc_tile_bytes(M1) : (size_t)kDescWarps * 4 * M1 * sizeof(real);
-  const void *kernel = f64 ? (const void *)descriptor_f64_kernel : (const void *)descriptor_kernel<real>;
-  if (smem > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return set_error(DP_ERR_CUDA, "dp_descriptor_contract: %s", cudaGetErrorString(e));
-  }
-  if constexpr (f64)
-    descriptor_f64_kernel<<<(unsigned)blocks, kDescWarps * 32, smem, (cudaStream_t)stream>>>(T, M1, M2, D);
-  else
+  auto allow = [&](const void *kernel, size_t smem) {
+    const cudaError_t e = smem > 48 * 1024
+                              ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
+                              : cudaSuccess;
+    return e == cudaSuccess ? DP_OK : set_error(DP_ERR_CUDA, "dp_descriptor_contract: %s", cudaGetErrorString(e));
+  };
+  if constexpr (std::is_same<real, double>::value) {
+    const size_t smem = dfx::desc_tile_bytes(M1);
+    if (int rc = allow((const void *)descriptor_f64_kernel, smem)) return rc;
+    return in_grids(nloc, [&](int64_t i0, unsigned n) {
+      descriptor_f64_kernel<<<n, kDescWarps * 32, smem, (cudaStream_t)stream>>>(T + i0 * 4 * M1, M1, M2, D + i0 * M1 * M2);
+      return launch_status("dp_descriptor_contract");
+    });
+  } else {
+    const size_t smem = (size_t)kDescWarps * 4 * M1 * sizeof(real);
+    if (int rc = allow((const void *)descriptor_kernel<real>, smem)) return rc;
     descriptor_kernel<real><<<(unsigned)blocks, kDescWarps * 32, smem, (cudaStream_t)stream>>>(T, nloc, M1, M2, D);
-  return launch_status("dp_descriptor_contract");
+    return launch_status("dp_descriptor_contract");
+  }
 }
 
 }  // namespace
