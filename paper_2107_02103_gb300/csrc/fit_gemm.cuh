@@ -268,10 +268,11 @@ __global__ void __launch_bounds__(kThreadsF, 1) fit_gemm_kernel(const Gemm P) {
   // unit u: column tile u % nt (the CTAs at work together share A tiles), share, row tile
   auto slices_of = [&](int sh) { return min(P.per, P.ka - sh * P.per); };
 
+  int issued = 0;  // thread 0: slices whose copies it started; thread 32: its commits on acc_full
   if (warp == 0) {
     // ---- producer
     if (lane == 0) {
-      int g = 0;
+      int &g = issued;
       bool ok = true;
       for (int u = blockIdx.x; u < nunits && ok; u += gridDim.x) {
         const int n = u % P.nt, r = u / P.nt, sh = r % P.ks, mt = r / P.ks;
@@ -304,7 +305,7 @@ __global__ void __launch_bounds__(kThreadsF, 1) fit_gemm_kernel(const Gemm P) {
     // ---- MMA issuer: digit s of A against B's digits t <= 7 - s, up to four planes an MMA, the
     // accumulator moved by s + t diagonals (see tab_gemm.cuh)
     if (lane == 0) {
-      int g = 0, li = 0;
+      int g = 0, &li = issued;
       bool ok = true;
       for (int u = blockIdx.x; u < nunits && ok; u += gridDim.x, ++li) {
         if (li > 0 && !(ok = wait_or_abort(smem_u32(tmem_free), (uint32_t)((li - 1) & 1), abortf))) break;
@@ -444,6 +445,11 @@ __global__ void __launch_bounds__(kThreadsF, 1) fit_gemm_kernel(const Gemm P) {
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
+  if (*abortf) {  // uniform
+    if (tid == 0) settle_copies(smem_u32(full), kStagesF, issued);
+    if (tid == 32 && issued > 0) settle(smem_u32(acc_full), (uint32_t)((issued - 1) & 1));
+    __syncthreads();
+  }
   if (tid == 0 && *abortf) atomicAdd(&g_wait_timeouts, 1u);
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols));
 }

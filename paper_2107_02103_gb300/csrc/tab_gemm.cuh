@@ -220,9 +220,10 @@ __global__ void __launch_bounds__(kThreadsP, 1) tgemm_kernel(const Params P) {
   const uint32_t tmem = *tmem_holder;
   const uint32_t sbase = smem_u32(smem);
 
+  int issued = 0;  // thread 0: slices whose copies it started; thread 32: its commits on acc_full
   if (warp == 0) {
     // ---- producer: each slice's A and B blocks into the next stage of the ring
-    int g = 0;  // slices loaded so far by this CTA
+    int &g = issued;
     for (int u = wk.begin; u < wk.end; u += wk.step) {
       if (__shfl_sync(0xffffffffu, (int)*abortf, 0)) break;  // uniform over the warp
       const Unit U = unit_of<kFwd>(P, u);
@@ -259,7 +260,7 @@ __global__ void __launch_bounds__(kThreadsP, 1) tgemm_kernel(const Params P) {
     // ---- MMA issuer: per slice the 45 digit products as 13 MMAs, per unit a commit
     // on acc_full once they have all completed
     if (lane == 0) {
-      int g = 0, li = 0;
+      int g = 0, &li = issued;
       bool ok = true;
       for (int u = wk.begin; u < wk.end && ok; u += wk.step) {
         const Unit U = unit_of<kFwd>(P, u);
@@ -513,6 +514,11 @@ __global__ void __launch_bounds__(kThreadsP, 1) tgemm_kernel(const Params P) {
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
+  if (*abortf) {  // uniform
+    if (tid == 0) settle_copies(smem_u32(full), kStages, issued);
+    if (tid == 32 && issued > 0) settle(smem_u32(acc_full), (uint32_t)((issued - 1) & 1));
+    __syncthreads();
+  }
   if (tid == 0 && *abortf) {
     atomicAdd(&g_wait_timeouts, 1u);
     if (!kFwd) *P.bad = 1;

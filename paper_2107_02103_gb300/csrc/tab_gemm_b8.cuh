@@ -142,10 +142,11 @@ __global__ void __launch_bounds__(kThreadsB, 1) bgemm_kernel(const Params P) {
   const uint32_t tmem = *tmem_holder;
   const uint32_t sbase = smem_u32(smem);
 
+  int issued = 0;  // thread 0: slices whose copies it started; thread 32: its commits on acc_full
   if (warp == 0) {
     // ---- producer: each slice's A and B blocks into the next stage of the ring
     if (lane == 0) {
-      int g = 0;  // slices loaded so far by this CTA
+      int &g = issued;
       bool ok = true;
       for (int u = blockIdx.x; u < nunits && ok; u += gridDim.x) {
         const Unit U = unit_of(P.units[u]);
@@ -175,7 +176,7 @@ __global__ void __launch_bounds__(kThreadsB, 1) bgemm_kernel(const Params P) {
     // ---- MMA issuer: per slice the 28 digit products as 7 MMAs into the unit's buffer, per unit a
     // commit on that buffer's acc_full once they have all completed
     if (lane == 0) {
-      int g = 0, li = 0;
+      int g = 0, &li = issued;
       bool ok = true;
       for (int u = blockIdx.x; u < nunits && ok; u += gridDim.x) {
         const int b = li & 1;
@@ -328,6 +329,11 @@ __global__ void __launch_bounds__(kThreadsB, 1) bgemm_kernel(const Params P) {
   asm volatile("tcgen05.fence::before_thread_sync;");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;");
+  if (*abortf) {  // uniform
+    if (tid == 0) settle_copies(smem_u32(full), kStagesB, issued);
+    if (tid == 32 && issued > 0) settle(smem_u32(acc_full + ((issued - 1) & 1)), (uint32_t)(((issued - 1) >> 1) & 1));
+    __syncthreads();
+  }
   if (tid == 0 && *abortf) {
     atomicAdd(&g_wait_timeouts, 1u);
     *P.bad = 1;

@@ -234,6 +234,32 @@ __device__ __forceinline__ bool wait_or_abort(uint32_t bar, uint32_t parity, vol
   }
 }
 
+// What a CTA still has in flight once a wait of it has given up: its copies into the stages that its producer issued
+// last (the `full` barriers' phases) and the MMAs before its last commit.  The CTA waits for them before it gives up its
+// shared memory and TMEM, each in at most kSettlePolls polls of about 20 us (a wait runs out by the clock, so also
+// where the GPU was taken away from the kernel for seconds, and then all of this is still under way).  False if
+// one did not end: a stage whose other arrivals are missing as well.
+constexpr int kSettlePolls = 500;
+__device__ __forceinline__ bool settle(uint32_t bar, uint32_t parity) {
+  for (int i = 0; i < kSettlePolls; ++i) {
+    uint32_t done;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n selp.u32 %0, 1, 0, p;\n}"
+        : "=r"(done)
+        : "r"(bar), "r"(parity), "r"(20000u)
+        : "memory");
+    if (done) return true;
+  }
+  return false;
+}
+// issued: slices whose copies the producer started, over a ring of `stages` (8-byte barriers from `full` on).
+__device__ __forceinline__ bool settle_copies(uint32_t full, int stages, int issued) {
+  bool all = true;
+  for (int g = max(0, issued - stages); g < issued; ++g)
+    all &= settle(full + 8 * (uint32_t)(g % stages), (uint32_t)((g / stages) & 1));
+  return all;
+}
+
 // A float that holds an integer of at most 2^24 in magnitude (a diagonal sum) as an int: exact.
 __device__ __forceinline__ int exact_int(float f) { return __float2int_rz(f); }
 
