@@ -191,9 +191,9 @@ struct Gemm {
   const unsigned char *aplanes;  // [tiles][ka] blocks
   const int *Eexp;               // [128 tiles]
   const unsigned char *bplanes;  // of type t at t bstride: [nt][ka] blocks
-  const int *Fexp;               // of type t at t fstride: [48 nt]
+  const int *Fexp;               // of type t at t fstride: [64 nt]
   size_t bstride, fstride;
-  longlong2 *part;               // ks > 1: [ks][48 nt][128 tiles] exact integers (lo, hi); hi kPartBad: NaN
+  longlong2 *part;               // ks > 1: [ks][64 nt][128 tiles] exact integers (lo, hi); hi kPartBad: NaN
 };
 constexpr long long kPartBad = 1ll << 62;
 

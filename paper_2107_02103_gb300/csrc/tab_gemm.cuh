@@ -129,8 +129,8 @@ struct Params {
   const int *nunits;  // their count (device)
 };
 
-// A unit packed into an int: tile (< 2^16), 128-row tile of A (< 2^8), share (< 2^8).
-__host__ __device__ constexpr int unit_code(int tile, int mt, int z) { return tile | (mt << 16) | (z << 24); }
+// A unit packed into an int: tile (< 2^16), 128-row tile of A (< 2^8).
+__host__ __device__ constexpr int unit_code(int tile, int mt) { return tile | (mt << 16); }
 
 struct Unit {
   int64_t tile;

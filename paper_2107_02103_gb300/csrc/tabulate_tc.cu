@@ -740,7 +740,7 @@ __global__ void __launch_bounds__(128) bwd_units_kernel(const unsigned char *__r
   for (int mt = 0; mt < nmt; ++mt) {
     bool any = false;
     for (int q = mt * kPer; q < min(nsl, mt * kPer + kPer); ++q) any |= f[q] != 0;
-    if (any) units[(size_t)t * maxunits + atomicAdd(nunits + t, 1)] = tg::unit_code((int)tile, mt, 0);
+    if (any) units[(size_t)t * maxunits + atomicAdd(nunits + t, 1)] = tg::unit_code((int)tile, mt);
   }
 }
 
