@@ -22,8 +22,24 @@ constexpr int kDescPlaces = 60, kDescLimb = 30;
 // quarter from each dropped product of low limbs, half from the rounding.  From this sum of magnitudes on, that is
 // below 3 2^-53 of it, and with the rounding to f64 below the 4 2^-53 of four FP64 operations.
 constexpr float kDescLeast = 0x1.d8p53f;
+// Where D in fixed point pays: the channels' preparation (four conversions each, and 80 bytes of shared memory) has to
+// be earned by their M2 elements.  Measured with 20,000 atoms, fixed over FP64 (a warp per atom): 16 x 8 1.01, 32 x 4
+// 1.02, 24 x 6 0.92, 48 x 4 0.93, 100 x 3 1.03, 400 x 4 0.88; and above 512 channels, two or three blocks an SM, 600 x 6
+// 1.09, 600 x 12 0.72, 800 x 12 1.12, 800 x 16 0.97.
+__host__ __device__ constexpr bool desc_fixed_pays(int M1, int M2) {
+  return M2 >= 4 && M1 * M2 >= 144 && (M1 <= 512 || 50 * M2 >= M1);
+}
 // Shared memory of desc_tile: T [4][M1] and the channels.
-__host__ __device__ constexpr size_t desc_tile_bytes(int M1) { return (size_t)M1 * (4 * sizeof(double) + sizeof(Channel)); }
+__host__ __device__ constexpr size_t desc_tile_bytes(int M1, int M2) {
+  return (size_t)M1 * (4 * sizeof(double) + (desc_fixed_pays(M1, M2) ? sizeof(Channel) : 0));
+}
+// The element in FP64, in the order of descriptor_kernel.
+__device__ __forceinline__ double desc_fp64(const double *Ts, int M1, int m, int n) {
+  double v = Ts[m] * Ts[n];
+#pragma unroll
+  for (int k = 1; k < 4; ++k) v = fma(Ts[k * M1 + m], Ts[k * M1 + n], v);
+  return v;
+}
 
 // One atom's D [M1][M2] by the threads of a block, from its T in Ts [4][M1] (written and synchronised), with
 // room for the channels after it.  Consecutive threads take consecutive elements, M2 to a row.
@@ -36,6 +52,17 @@ __host__ __device__ constexpr size_t desc_tile_bytes(int M1) { return (size_t)M1
 // multiply-adds tell, and such an element (like those of a channel with an inf or NaN, or out of the exponents'
 // range) is left to the FP64 pipe.
 __device__ __forceinline__ void desc_tile(const double *Ts, int M1, int M2, double *__restrict__ D) {
+  if (!desc_fixed_pays(M1, M2)) {  // uniform
+    const int total = M1 * M2, dm = (int)blockDim.x / M2, dn = (int)blockDim.x - dm * M2;
+    int m = (int)threadIdx.x / M2, n = (int)threadIdx.x - m * M2;
+#pragma unroll 1
+    for (int e = threadIdx.x; e < total; e += blockDim.x) {
+      D[e] = desc_fp64(Ts, M1, m, n);
+      m += dm, n += dn;
+      if (n >= M2) n -= M2, ++m;
+    }
+    return;
+  }
   Channel *C = reinterpret_cast<Channel *>(const_cast<double *>(Ts) + 4 * M1);
   for (int m = threadIdx.x; m < M1; m += blockDim.x) {
     double x[4];
@@ -77,11 +104,7 @@ __device__ __forceinline__ void desc_tile(const double *Ts, int M1, int M2, doub
         mag = fmaf(c.a[k], b.a[k], mag);
       }
       double v = fx::to_double(fx::over_unit<kDescLimb>(p), 2 * kDescLimb - c.sh - b.sh);
-      if (mag < kDescLeast) {
-        v = Ts[m] * Ts[n];
-#pragma unroll
-        for (int k = 1; k < 4; ++k) v = fma(Ts[k * M1 + m], Ts[k * M1 + n], v);
-      }
+      if (mag < kDescLeast) v = desc_fp64(Ts, M1, m, n);
       D[m * M2 + n] = v;
     }
   }

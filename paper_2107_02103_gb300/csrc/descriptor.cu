@@ -2,11 +2,12 @@
 // D_i = S_i (S_i^<)^T is M1 x M2:  D[i][m][n] = sum_k T[i][k][m] T[i][k][n].
 //
 // On f64 arrays (the f64 and the df64 calls) a block per atom, in fixed point on the integer pipes
-// (desc_fixed.cuh).  In f32 one warp per atom: T_i (4 x M1) is staged in shared memory; the M1 x M2 output tile is
+// (desc_fixed.cuh), where the shape is large enough for that to pay.  In f32, and in f64 below, one warp per atom:
+// T_i (4 x M1) is staged in shared memory; the M1 x M2 output tile is
 // contiguous, so lane l computes elements l, l + 32, ... of it in storage order, every lane busy (M1*M2 is a
 // multiple of 32 for the paper's shapes) and every store coalesced.
-// The warp-per-atom backward takes f32 and, in f64 or df64 arithmetic (io_t), the shapes too wide for the
-// fixed-point one's shared memory.
+// The warp-per-atom backward takes f32, the small f64 shapes and, in f64 or df64 arithmetic (io_t), those too wide for
+// the fixed-point one's shared memory.
 #include <algorithm>
 #include <type_traits>
 
@@ -371,6 +372,26 @@ int in_grids(int64_t nloc, F &&f) {
   return DP_OK;
 }
 
+// Where dT in fixed point pays.  Measured with 20,000 atoms, fixed over FP64 (a warp per atom): 16 x 16 1.25, 24 x 24
+// 0.98, 32 x 12 1.04, 32 x 16 0.90, 48 x 8 1.17, 48 x 12 0.90, 64 x 6 1.02, 64 x 8 0.93, 80 x 3 1.06, 80 x 6 0.94,
+// 100 x 1 0.74; with 1,500 atoms the same or less.
+constexpr bool desc_grad_fixed_pays(int M1, int M2) { return M1 >= 80 || M1 * M2 >= 512; }
+
+template <typename real>
+int descriptor_grad_warps(const io_t<real> *T, const io_t<real> *dD, int64_t nloc, int M1, int M2, io_t<real> *dT,
+                          void *stream) {
+  const size_t smem = (size_t)kDescWarps * desc_grad_smem_per_warp<real>(M1, M2) * sizeof(real);
+  if (smem > 227 * 1024) return set_error(DP_ERR_UNSUPPORTED, "M1 = %d, M2 = %d need too much shared memory", M1, M2);
+  if (smem > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(descriptor_grad_kernel<real>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return set_error(DP_ERR_CUDA, "dp_descriptor_contract_grad: %s", cudaGetErrorString(e));
+  }
+  descriptor_grad_kernel<real><<<(unsigned)((nloc + kDescWarps - 1) / kDescWarps), kDescWarps * 32, smem,
+                                 (cudaStream_t)stream>>>(T, dD, nloc, M1, M2, dT);
+  return launch_status("dp_descriptor_contract_grad");
+}
+
 template <typename real>
 int descriptor_grad(const io_t<real> *T, const io_t<real> *dD, int64_t nloc, int M1, int M2, io_t<real> *dT,
                     void *stream) {
@@ -384,11 +405,12 @@ int descriptor_grad(const io_t<real> *T, const io_t<real> *dD, int64_t nloc, int
   const int64_t blocks = (nloc + kDescWarps - 1) / kDescWarps;
   if (blocks > kMaxGrid) return set_error(DP_ERR_SHAPE, "nloc too large");
   if constexpr (std::is_same<io_t<real>, double>::value) {
-    // in fixed point wherever the staged dD_i leaves at least four blocks to an SM; the kernel below for wider
-    // ones.  Also for the df64 call, whose arrays are f64 (12,288 atoms x 100 x 16: 0.279 ms in df64 arithmetic,
-    // 0.181 here; D 0.077 and 0.066)
+    // in fixed point wherever that pays and the staged dD_i leaves at least four blocks to an SM; the warps in df64
+    // arithmetic only for wider ones, so that the df64 call gives the f64 call's results (12,288 atoms x 100 x 16:
+    // 0.279 ms in df64 arithmetic, 0.181 here; D 0.077 and 0.066)
     const size_t need = desc_grad_f64_bytes(M1, M2);
     if (desc_grad_f64_entries(M1, M2) * sizeof(double) <= 56 * 1024) {
+      if (!desc_grad_fixed_pays(M1, M2)) return descriptor_grad_warps<double>(T, dD, nloc, M1, M2, dT, stream);
       if (need > 48 * 1024) {
         const cudaError_t e = cudaFuncSetAttribute(descriptor_grad_f64_kernel,
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
@@ -401,16 +423,7 @@ int descriptor_grad(const io_t<real> *T, const io_t<real> *dD, int64_t nloc, int
       });
     }
   }
-  const size_t smem = (size_t)kDescWarps * desc_grad_smem_per_warp<real>(M1, M2) * sizeof(real);
-  if (smem > 227 * 1024) return set_error(DP_ERR_UNSUPPORTED, "M1 = %d, M2 = %d need too much shared memory", M1, M2);
-  if (smem > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(descriptor_grad_kernel<real>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return set_error(DP_ERR_CUDA, "dp_descriptor_contract_grad: %s", cudaGetErrorString(e));
-  }
-  descriptor_grad_kernel<real>
-      <<<(unsigned)blocks, kDescWarps * 32, smem, (cudaStream_t)stream>>>(T, dD, nloc, M1, M2, dT);
-  return launch_status("dp_descriptor_contract_grad");
+  return descriptor_grad_warps<real>(T, dD, nloc, M1, M2, dT, stream);
 }
 
 template <typename real>
@@ -432,19 +445,19 @@ int descriptor(const io_t<real> *T, int64_t nloc, int M1, int M2, io_t<real> *D,
                               : cudaSuccess;
     return e == cudaSuccess ? DP_OK : set_error(DP_ERR_CUDA, "dp_descriptor_contract: %s", cudaGetErrorString(e));
   };
-  if constexpr (std::is_same<real, double>::value) {
-    const size_t smem = dfx::desc_tile_bytes(M1);
-    if (int rc = allow((const void *)descriptor_f64_kernel, smem)) return rc;
-    return in_grids(nloc, [&](int64_t i0, unsigned n) {
-      descriptor_f64_kernel<<<n, kDescWarps * 32, smem, (cudaStream_t)stream>>>(T + i0 * 4 * M1, M1, M2, D + i0 * M1 * M2);
-      return launch_status("dp_descriptor_contract");
-    });
-  } else {
-    const size_t smem = (size_t)kDescWarps * 4 * M1 * sizeof(real);
-    if (int rc = allow((const void *)descriptor_kernel<real>, smem)) return rc;
-    descriptor_kernel<real><<<(unsigned)blocks, kDescWarps * 32, smem, (cudaStream_t)stream>>>(T, nloc, M1, M2, D);
-    return launch_status("dp_descriptor_contract");
-  }
+  if constexpr (std::is_same<real, double>::value)
+    if (dfx::desc_fixed_pays(M1, M2)) {
+      const size_t smem = dfx::desc_tile_bytes(M1, M2);
+      if (int rc = allow((const void *)descriptor_f64_kernel, smem)) return rc;
+      return in_grids(nloc, [&](int64_t i0, unsigned n) {
+        descriptor_f64_kernel<<<n, kDescWarps * 32, smem, (cudaStream_t)stream>>>(T + i0 * 4 * M1, M1, M2, D + i0 * M1 * M2);
+        return launch_status("dp_descriptor_contract");
+      });
+    }
+  const size_t smem = (size_t)kDescWarps * 4 * M1 * sizeof(real);
+  if (int rc = allow((const void *)descriptor_kernel<real>, smem)) return rc;
+  descriptor_kernel<real><<<(unsigned)blocks, kDescWarps * 32, smem, (cudaStream_t)stream>>>(T, nloc, M1, M2, D);
+  return launch_status("dp_descriptor_contract");
 }
 
 }  // namespace

@@ -1323,7 +1323,7 @@ int fwd(const dp_tc_plan *plan, const dp_table_info *info, const double *s, cons
     G.ntypes = ntypes;
     if ((rc = tg::launch(G, st, who, ncta))) return rc;
     prof_mark("tc_gemm_fwd", st);
-    fwd_finish_kernel<<<(unsigned)n, 128, D ? dfx::desc_tile_bytes(M1) : 0, st>>>(
+    fwd_finish_kernel<<<(unsigned)n, 128, D ? dfx::desc_tile_bytes(M1, M2) : 0, st>>>(
         part, S.Mpf, G.Eexp, R.fexp, reinterpret_cast<const int *>(wk + L.npieces),
         reinterpret_cast<const int *>(wk + L.pfirst), ntiles, nmt, c0, atype, ntypes, M1, T, M2, D);
     if ((rc = launch_status(who))) return rc;
