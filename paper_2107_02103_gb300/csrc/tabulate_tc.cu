@@ -912,7 +912,7 @@ __device__ __forceinline__ RowPoly row_poly(const int2 ke, bool plain, double t,
   R.ke = ke;
   R.e = e;
   R.drop = ke.x - ke.y;  // the constant's units over the slope's, as a shift: >= 1
-  R.half = R.drop < 32 ? 1 << (R.drop - 1) : 0;  // so that it rounds (beyond, the constant decides alone)
+  R.half = R.drop < 32 ? (int)((1u << R.drop) >> 1) : 0;  // so that it rounds (beyond, the constant decides alone)
   R.plain = plain && max(abs(ke.x), abs(ke.y)) <= 400 && R.drop < 32;
   R.nan = nan || (__double2hiint(t) & 0x7ff00000) == 0x7ff00000;  // (a NaN s)
   return R;
