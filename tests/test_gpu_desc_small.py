@@ -64,16 +64,15 @@ def _us(call):
     return best
 
 
-@pytest.mark.parametrize("M1,M2,limit", [(1, 1, 1.4), (8, 2, 1.4), (16, 4, 1.8)])
-def test_small_shapes_cost_a_warp_an_atom(M1, M2, limit):
-    """20,000 atoms in f64 against the f32 calls, a warp per atom as well: the memory is twice as much, and the few FP64
-    operations more (D 1.0, 1.0 and 1.5 times, dT 1.2, 1.8 and 2.4); a block per atom took 1.6, 1.6 and 2.0 times, and dT 4.1
-    to 4.9."""
+@pytest.mark.parametrize("M1,M2", [(1, 1), (8, 2), (16, 4)])
+def test_small_shapes_cost_a_warp_an_atom(M1, M2):
+    """200,000 atoms in f64 against the f32 calls, a warp per atom as well: twice the memory and a few FP64 operations (D 1.3,
+    1.3 and 1.9 times the f32 calls, dT 1.4, 2.1 and 2.5); a block per atom took 3.1 to 3.2 times, and dT 6.1 to 8.6."""
     dpc = lib()
-    T, dD = torch.randn(20000, 4, M1, device="cuda"), torch.randn(20000, M1, M2, device="cuda")
+    T, dD = torch.randn(200000, 4, M1, device="cuda"), torch.randn(200000, M1, M2, device="cuda")
     T64, dD64 = T.double(), dD.double()
     o = [torch.empty_like(a) for a in (dD, T, dD64, T64)]
     d32, d64 = (_us(lambda a=a, b=b: dpc.dp_descriptor_contract(a, M2, out=b)) for a, b in ((T, o[0]), (T64, o[2])))
     t32, t64 = (_us(lambda a=a, g=g, b=b: dpc.dp_descriptor_contract_grad(a, g, out=b))
                 for a, g, b in ((T, dD, o[1]), (T64, dD64, o[3])))
-    assert d64 <= limit * d32 and t64 <= 3.0 * t32, (d32, d64, t32, t64)
+    assert d64 <= 2.4 * d32 and t64 <= 3.6 * t32, (d32, d64, t32, t64)
