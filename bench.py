@@ -196,8 +196,8 @@ def moment_fmas(runs, M1: int) -> dict:
 # `ncu --set full` capture of its current version (the commit the capture was taken at beside each);
 # absent means no capture of the current kernel exists and `traffic` is reported as null.
 PROFILED_DRAM_BYTES = {("cu85", "f64", "grad", "moments"): 83838464 + 32080640,   # commit 7987c32
-                       ("cu85", "f64", "tc_rows", "tc"): 106909440 + 37977088,    # commit e2ecb8c
-                       ("cu85", "f64", "tc_runs_moments", "tc"): 70285312 + 12362496}
+                       ("cu85", "f64", "tc_rows", "tc"): 106579200 + 36644096,    # commit 0d79dfc
+                       ("cu85", "f64", "tc_runs_moments", "tc"): 70285824 + 12405248}
 
 
 def peak_tflops(dtype: str, mhz: float = SM_MAX_MHZ, nsm: int = NSM) -> float:

@@ -82,9 +82,10 @@ __device__ __forceinline__ void radius(double r2, double &r, double &inv_r) {
 //   kind 0: with x = u - 1/2, z = x^2 <= 1/4, cos(pi u) = -sin(pi x) and sin(pi u) = cos(pi x) by their Taylor
 //           series in z, twelve terms each (the next is below 2^-63), coefficients over 4.
 // Why: a row's environment took 50 (kind 1) to 66 (kind 0) FP64 instructions, 68 clocks of a sub-partition
-// each, and set the time of the kernels that form rows; now it takes 23.  Measured (copper, 4,096 atoms, kind 1):
-// the fused forward's runs kernel 0.196 -> 0.154 ms, the fused rows and forces 0.345 -> 0.305 ms; water (1,536
-// atoms, kind 0) 0.039 -> 0.029 and 0.051 -> 0.036 ms.
+// each, and set the time of the kernels that form rows; now it takes 25.  Measured (copper, 4,096 atoms, kind 1):
+// the fused forward's runs kernel 0.196 -> 0.160 ms, the fused rows and forces 0.345 -> 0.312 ms; water (1,536
+// atoms, kind 0) 0.039 -> 0.030 and 0.051 -> 0.036 ms.  w and w' have absolute errors; near the cut-off, where both
+// are small, s and ds/dr are still more exact than with w from FP64, whose cancellation there is the larger error.
 struct SwitchFixed {
   long long w, dw;  // units of 2^-60 and 2^-58
 };
