@@ -410,9 +410,10 @@ int dp_descriptor_contract_f32(const float *T, int64_t nloc, int M1, int M2, flo
  *   T [nloc][4][M1], dD [nloc][M1][M2] inputs;  dT [nloc][4][M1] output, fully
  *   overwritten (feed it to dp_tabulate_fusion_grad_*).
  * In f64, with an atom's |dD[m][n]| <= R_m C_n, C_n the largest of its column and
- * R_m the largest of its row over C_n, the first sum is within
- * 2^-53 M2 R_m max_n C_n |T[k][n]| and the second within
- * 2^-53 M1 C_m max_m' R_m' |T[k][m']|, and each is rounded to f64 every 16 terms.
+ * R_m the largest of its row over C_n, the terms of the first sum are exact to
+ * 2^-53 R_m max_n C_n |T[k][n]| each, those of the second to
+ * 2^-53 C_m max_m' R_m' |T[k][m']|; the sums are rounded to f64 every 16 terms
+ * (in small shapes, M1 < 80 and M1 M2 < 512, both are plain f64 sums).
  * Errors, limits and the nloc == 0 rule as dp_descriptor_contract_*; the
  * backward stages T_i and dT_i (M1 > 908 in f64, 1816 in f32 is
  * DP_ERR_UNSUPPORTED).

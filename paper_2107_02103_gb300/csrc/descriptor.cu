@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(kDescGradThreads)
   const int64_t i = blockIdx.x;
   const double *Ti = T + i * 4 * M1, *Di = dD + i * (int64_t)M1 * M2;
   double *Td = reinterpret_cast<double *>(Tf), *Dd = reinterpret_cast<double *>(Df);
-  // exponents are kept as high words, sign off and the mantissa cleared: a field in bits 20 up
+  // exponents are compared as high words, sign off: the field in bits 20 up
   auto key = [](double x) { return __double2hiint(x) & 0x7fffffff; };
   auto tiny = [](double x, int h) { return h < (1 << 20) && (h | __double2loint(x)); };  // a subnormal
   for (int n = tid; n < M2; n += kDescGradThreads) col_e[n] = 0;
